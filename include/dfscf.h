@@ -48,7 +48,10 @@ extern "C" {
 #define DF_ERR_NUMERIC 7     /* NaN/Inf detected in an SCF quantity                     */
 
 /* ---- precision modes -------------------------------------------------------------- */
-#define DF_FP64 0            /* every contraction in FP64                               */
+#define DF_FP64 0            /* every contraction to FP64 accuracy or better: the exchange
+                                contractions run on the tensor cores as exact sums of
+                                base-512 digit products in 64-bit integers, rounded to
+                                FP64 once (entry errors below 2^-51 sqrt(K_mm K_nn))     */
 #define DF_MIXED 1           /* K contractions as split-BF16 GEMMs on tcgen05 tensor
                                 cores.  Every operand row (of B_P, of C^T, of X) is held
                                 as NP BF16 planes, NP = the knob "mixed_planes" (3, 4 or
@@ -439,8 +442,8 @@ int df_j_noalloc(const void* B, int nao, int naux, const double* D, double* J, c
  * auxiliary rows per CTA slice of J's second pass), "eig_ctas" (CTAs of the multi-SM
  * eigensolver: 0 automatic, 1 a single CTA) and "mixed_planes" (3..5 BF16 planes per operand of
  * the mixed exchange: 6, 10 or 15 plane products; it also sizes a mixed B).
- * Tile shapes: "fp64_ht_cols" (0 automatic, 16 or 32 occupied columns per FP64 half-transform
- * CTA), "ht_n" (0: the widest tcgen05 half-transform tile that fits; else a cap, a multiple
+ * Tile shapes: "fp64_ht_cols" (0 automatic, 16 or 32 occupied columns per column group of the FP64
+ * half-transform), "ht_n" (0: the widest tcgen05 half-transform tile that fits; else a cap, a multiple
  * of 16), "jpass1_rows" (1, 2, 4 or 8 auxiliary rows per CTA of J's first pass) and
  * "j_fp64_fma" (1: J's passes with FP64 FMAs instead of double-float products).
  * "mixed_incremental" (0 or 1), "soscf" (0 or 1) and "soscf_cg" (1..64) shape the SCF as

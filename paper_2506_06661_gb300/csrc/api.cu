@@ -133,7 +133,7 @@ static Knob g_knobs[] = {
     {"jpass2_rows", 256, 32, 512},   // auxiliary rows per CTA slice of J's second pass
     {"j_fp64_fma", 0, 0, 1},         // J passes: 0 double-float products on FP32 units, 1 FP64 FMAs
     {"jpass1_rows", 1, 1, 8},        // auxiliary rows per CTA of J's first pass (1, 2, 4 or 8)
-    {"fp64_ht_cols", 0, 0, 32},      // FP64 half-transform tile columns: 0 auto, 16 or 32
+    {"fp64_ht_cols", 0, 0, 32},      // columns per group of the FP64 half-transform: 0 auto, 16 or 32
     {"dm0_eig_cut", 12, 1, 16},      // first exchange of a fractional dm0: occupations below 10^-cut dropped
     {"guess_idem_max", 200, 1, 1000},// largest idempotency error of an accepted dm0, in hundredths
     {"ht_n", 0, 0, 256},             // tcgen05 half-transform tile columns: 0 widest that fits, else a cap
@@ -211,7 +211,8 @@ extern "C" int df_bounds_violations(unsigned long long* count, char* where, size
     const char* name;
     dfscf::BoundsReader read;
   };
-  const Unit units[] = {{"dferr.cu", dfscf::bounds_read_dferr},   {"eig.cu", dfscf::bounds_read_eig},
+  const Unit units[] = {{"dferr.cu", dfscf::bounds_read_dferr},   {"digits.cu", dfscf::bounds_read_digits},
+                        {"eig.cu", dfscf::bounds_read_eig},
                         {"integrals.cu", dfscf::bounds_read_integrals}, {"jk.cu", dfscf::bounds_read_jk},
                         {"linalg.cu", dfscf::bounds_read_linalg}, {"lowdin.cu", dfscf::bounds_read_lowdin},
                         {"lrdf.cu", dfscf::bounds_read_lrdf},     {"mlp.cu", dfscf::bounds_read_mlp},

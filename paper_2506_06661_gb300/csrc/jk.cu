@@ -16,10 +16,12 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 #include <mutex>
 #include <unordered_map>
 
 #include "common.cuh"
+#include "digits.cuh"
 #include "kernels.cuh"
 #include "planes.cuh"
 
@@ -340,93 +342,54 @@ __global__ void jreduce_unpack_kernel(const double* __restrict__ Jpart, int nspl
 }
 
 // ---- FP64 K ---------------------------------------------------------------------------
-// X[m][P][i] = sum_n B_P[m][n] C[n][i]; B_P gathered from the packed row.
-// CTA tile 64 (m) x 16 CI (i), 256 lanes with 4 x CI outputs each (CI = 2: 32 columns, for
-// wide occupied spaces; CI = 1: 16 columns, less padding for small ones; knob
-// "fp64_ht_cols").
-template <int CI>
-__global__ void __launch_bounds__(256) k_halftransform_fp64_kernel(const double* __restrict__ B, long ld, int nao,
-                                                                   int naux, const double* __restrict__ C, int nocc,
-                                                                   double* __restrict__ X) {
-  constexpr int TN = 16 * CI;
-  __shared__ double As[16][65];
-  __shared__ double Cs[16][TN + 1];
-  int P = blockIdx.z;
-  int m0 = blockIdx.y * 64, i0 = blockIdx.x * TN;
-  const double* row = B + (size_t)P * ld;
-  int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;  // tx -> i (CI each, stride 16), ty -> m (4 each, stride 16)
-  double acc[4][CI];
-#pragma unroll
-  for (int u = 0; u < 4; ++u)
-#pragma unroll
-    for (int v = 0; v < CI; ++v) acc[u][v] = 0.0;
-  for (int n0 = 0; n0 < nao; n0 += 16) {
-#pragma unroll
-    for (int r = 0; r < 4; ++r) {
-      int idx = threadIdx.x + 256 * r;
-      int mm = idx >> 4, nn = idx & 15;
-      int gm = m0 + mm, gn = n0 + nn;
-      double v = 0.0;
-      if (gm < nao && gn < nao) {
-        int a = max(gm, gn), b = min(gm, gn);
-        v = row[DF_IX((size_t)a * (a + 1) / 2 + b, ld)];
-      }
-      As[nn][mm] = v;
-    }
-#pragma unroll
-    for (int r = 0; r < CI; ++r) {
-      int idx = threadIdx.x + 256 * r;
-      int nn = idx / TN, ii = idx % TN;
-      int gn = n0 + nn, gi = i0 + ii;
-      Cs[nn][ii] = (gn < nao && gi < nocc) ? C[DF_IX((size_t)gn * nocc + gi, (size_t)nao * nocc)] : 0.0;
-    }
-    __syncthreads();
-#pragma unroll
-    for (int k = 0; k < 16; ++k) {
-      double a[4], c[CI];
-#pragma unroll
-      for (int u = 0; u < 4; ++u) a[u] = As[k][ty + 16 * u];
-#pragma unroll
-      for (int v = 0; v < CI; ++v) c[v] = Cs[k][tx + 16 * v];
-#pragma unroll
-      for (int u = 0; u < 4; ++u)
-#pragma unroll
-        for (int v = 0; v < CI; ++v) acc[u][v] = fma(a[u], c[v], acc[u][v]);
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    int gm = m0 + ty + 16 * u;
-    if (gm >= nao) continue;
-#pragma unroll
-    for (int v = 0; v < CI; ++v) {
-      int gi = i0 + tx + 16 * v;
-      if (gi < nocc) X[DF_IX(((size_t)gm * naux + P) * nocc + gi, (size_t)nao * naux * nocc)] = acc[u][v];
-    }
-  }
-}
-
 // K[m][n] = K[n][m] = sum_split Kpart[split][m][n] over the lower triangle m >= n.
-__global__ void ksum_mirror_kernel(const double* __restrict__ Kpart, int nsplit, int nao, double* __restrict__ K) {
+// NaN when a bounded wait of the tensor-core kernels gave up (*err set).
+__global__ void ksum_mirror_kernel(const double* __restrict__ Kpart, int nsplit, int nao, const int* __restrict__ err,
+                                   double* __restrict__ K) {
   long e = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= (long)nao * nao) return;
   int m = (int)(e / nao), n = (int)(e % nao);
   if (n > m) return;
-  double s = 0.0;
-  for (int k = 0; k < nsplit; ++k) s += Kpart[DF_IX((size_t)k * nao * nao + e, (size_t)nsplit * nao * nao)];
+  double s = 0.0, c = 0.0;  // compensated (Knuth's TwoSum): the splits add no rounding of their own
+  for (int k = 0; k < nsplit; ++k) {
+    const double x = Kpart[DF_IX((size_t)k * nao * nao + e, (size_t)nsplit * nao * nao)], t = s + x, b = t - s;
+    c += (s - (t - b)) + (x - b);
+    s = t;
+  }
+  if (isfinite(c)) s += c;
+  if (*err) s = __longlong_as_double(0x7ff8000000000000LL);
   K[(size_t)m * nao + n] = s;
   K[(size_t)n * nao + m] = s;
 }
 
-int ksplit_count(int nao, long kdim) {
-  // enough CTAs for ~4 waves on 152 SMs over the lower-triangle tiles
-  long tiles = (long)((nao + 63) / 64) * ((nao + 63) / 64 + 1) / 2;
-  long want = (4L * 152 * 4 + tiles - 1) / tiles;
-  long maxs = max(1L, kdim / 512);
-  int forced = knob("fp64_syrk_split");
-  if (forced > 0) return (int)max(1L, min((long)forced, max(1L, kdim / 16)));
-  return (int)max(1L, min(want, min(maxs, 64L)));
+// Block sizes of the FP64 exchange.  Each half-transform launch should fill the GPU for a few
+// waves of 128-row tiles (pb), within 512 MB of B digits; each SYRK launch should have a long K
+// (px), within 1 GB of X and its digits.
+static void fp64_k_blocks(int nao, int naux, int nocc, Fp64KWork* w) {
+  const long coltiles = (nocc + 63) / 64;
+  const long rows = 4L * 152 * digits::BM / coltiles;
+  const size_t bytes_b = digits::plane_bytes(nao, nao), bytes_x = (size_t)nao * nocc * (2 * digits::NS + 8);
+  long pb = std::min((rows + nao - 1) / nao, std::max(1L, (long)((512ul << 20) / bytes_b)));
+  pb = std::max(1L, std::min(pb, (long)naux));
+  long px = std::max(pb, (long)((1ul << 30) / bytes_x) / pb * pb);
+  w->pb = (int)pb;
+  w->px = (int)std::min(px, (long)naux);
+  // splits of the SYRK's K range: least waves x (stages + the cost of a tile's start and end)
+  const long width = nao > 32 ? 64 : 32, ntn = (nao + width - 1) / width;
+  long tiles = 0;
+  for (long m = digits::BM; m < nao + digits::BM; m += digits::BM) tiles += std::min((std::min(m, (long)nao) - 1) / width + 1, ntn);
+  const long nst = ((long)w->px * nocc + digits::BK - 1) / digits::BK;
+  long best = LONG_MAX;
+  w->nsplit = 1;
+  for (long n = std::max(1L, (nst + 4095) / 4096); n <= 64 && n <= std::max(1L, nst / 4); ++n) {
+    const long cost = ((tiles * n + 151) / 152) * ((nst + n - 1) / n + 16);
+    if (cost < best) {
+      best = cost;
+      w->nsplit = (int)n;
+    }
+  }
+  const int forced = knob("fp64_syrk_split");
+  if (forced > 0) w->nsplit = (int)std::max((nst + 4095) / 4096, std::min((long)forced, std::max(1L, nst / 2)));
 }
 
 // fp64_k: also carve the FP64 exchange buffers when precision is DF_MIXED (an SCF that
@@ -436,17 +399,21 @@ JKWork jk_work_layout(int nao, int naux, int nocc, int precision, Arena* a, Size
   long ld = B_ld(nao);
   int rows = max(32, min(JP2_MAX_ROWS, knob("jpass2_rows")));
   int nsplit_j = (naux + rows - 1) / rows;
-  int nsplit_k = ksplit_count(nao, (long)naux * max(nocc, 1));
   w.nsplit_j = nsplit_j;
-  w.nsplit_k = nsplit_k;
 #define TAKE(T, ptr, count) \
   if (a) ptr = a->take<T>(count); else z->take<T>(count);
   TAKE(double, w.Dw, ld);
   TAKE(double, w.d, naux);
   TAKE(double, w.Jpart, (size_t)nsplit_j * ld);
   if (precision == DF_FP64 || fp64_k) {
-    TAKE(double, w.X, (size_t)nao * naux * max(nocc, 1));
-    TAKE(double, w.Kpart, (size_t)nsplit_k * nao * nao);
+    const int oc = max(nocc, 1);
+    fp64_k_blocks(nao, naux, oc, &w.fk);
+    TAKE(char, w.fk.Ct, digit_operand_bytes(oc, nao));
+    TAKE(char, w.fk.Bp, digit_operand_bytes((long)w.fk.pb * nao, nao));
+    TAKE(char, w.fk.Xd, digit_operand_bytes(nao, (long)w.fk.px * oc));
+    TAKE(double, w.fk.X, (size_t)nao * w.fk.px * oc);
+    TAKE(double, w.fk.Kpart, (size_t)w.fk.nsplit * nao * nao);
+    TAKE(int, w.fk.err, 1);
   }
   if (precision == DF_MIXED) mixed_k_work_layout(nao, naux, nocc, a, z, &w.mk);
 #undef TAKE
@@ -507,32 +474,33 @@ int build_J(const void* Bbuf, const BLayout& L, int nao, int naux, int precision
   return DF_OK;
 }
 
-int build_K_fp64(const double* B64, long ld, int nao, int naux, const double* C, int nocc, double* K, const JKWork& w,
-                 cudaStream_t s) {
-  {
-    ProfScope ps("k_halftransform_fp64", s);
-    const int forced = knob("fp64_ht_cols");
-    const int cols = forced == 16 || forced == 32 ? forced : (nocc <= 16 ? 16 : 32);
-    if (cols == 16) {
-      dim3 grid((nocc + 15) / 16, (nao + 63) / 64, naux);
-      k_halftransform_fp64_kernel<1><<<grid, 256, 0, s>>>(B64, ld, nao, naux, C, nocc, w.X);
-    } else {
-      dim3 grid((nocc + 31) / 32, (nao + 63) / 64, naux);
-      k_halftransform_fp64_kernel<2><<<grid, 256, 0, s>>>(B64, ld, nao, naux, C, nocc, w.X);
+int build_K_fp64(const double* B64, long ld, int nao, int naux, const double* C, int nocc, double* K,
+                 const Fp64KWork& w, cudaStream_t s) {
+  DF_CUDA(cudaMemsetAsync(w.err, 0, sizeof(int), s));
+  const DigitOperand ct = digit_operand(w.Ct, nocc, nao);
+  DF_TRY(slice_matrix(C, nocc, true, ct, s));
+  for (int x0 = 0; x0 < naux; x0 += w.px) {
+    const int nx = std::min(w.px, naux - x0);
+    const long kdim = (long)nx * nocc;
+    const DigitOperand xd = digit_operand(w.Xd, nao, kdim);
+    DF_CUDA(cudaMemsetAsync(xd.key, 0, sizeof(unsigned) * (size_t)nao, s));
+    {
+      ProfScope ps("k_halftransform_fp64", s);
+      for (int p0 = x0; p0 < x0 + nx; p0 += w.pb) {
+        const int np = std::min(w.pb, x0 + nx - p0);
+        const DigitOperand bp = digit_operand(w.Bp, (long)np * nao, nao);
+        DF_TRY(slice_packed(B64, ld, nao, naux, p0, np, bp, s));
+        DF_TRY(digit_half_transform(bp, ct, B64, ld, nao, naux, p0, C, nocc, w.X, kdim, (long)(p0 - x0) * nocc, xd.key,
+                                    w.err, s));
+      }
     }
-    DF_LAUNCHED("k_halftransform_fp64_kernel");
-  }
-  long kdim = (long)naux * nocc;
-  long kchunk = (kdim + w.nsplit_k - 1) / w.nsplit_k;
-  kchunk = (kchunk + 15) / 16 * 16;
-  int nsplit = (int)((kdim + kchunk - 1) / kchunk);
-  {
     ProfScope ps("k_syrk_fp64", s);
-    DF_TRY(dgemm(false, true, nao, nao, (int)kdim, 1.0, w.X, kdim, 0, w.X, kdim, 0, 0.0, w.Kpart, nao,
-                 (long)nao * nao, nsplit, s, kchunk, 1));
+    DF_TRY(slice_with_keys(w.X, kdim, xd, s));
+    const DigitSource src{w.X, kdim, 1};
+    DF_TRY(digit_gemm(xd, xd, src, src, 1.0, x0 ? 1.0 : 0.0, w.Kpart, nao, (long)nao * nao, w.nsplit, true, w.err, s));
   }
   long nn = (long)nao * nao;
-  ksum_mirror_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(w.Kpart, nsplit, nao, K);
+  ksum_mirror_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(w.Kpart, w.nsplit, nao, w.err, K);
   DF_LAUNCHED("ksum_mirror_kernel");
   return DF_OK;
 }
@@ -549,8 +517,8 @@ int run_jk(const void* B, int nao, int naux, int precision, const double* D, con
   if (J) DF_TRY(build_J(B, L, nao, naux, precision, D, J, w, s));
   if (K) {
     if (precision == DF_FP64) {
-      DF_REQUIRE(w.X && w.Kpart, DF_ERR_ARG, "FP64 exchange requested with a workspace laid out for mixed precision");
-      DF_TRY(build_K_fp64((const double*)((const char*)B + L.off64), L.ld, nao, naux, C, nocc, K, w, s));
+      DF_REQUIRE(w.fk.X && w.fk.Kpart, DF_ERR_ARG, "FP64 exchange requested with a workspace laid out for mixed precision");
+      DF_TRY(build_K_fp64((const double*)((const char*)B + L.off64), L.ld, nao, naux, C, nocc, K, w.fk, s));
     } else {
       DF_REQUIRE(w.mk.Xp[0] && w.mk.Kpart, DF_ERR_ARG, "mixed exchange requested with a workspace laid out for FP64");
       DF_TRY(build_K_mixed(B, L, nao, naux, C, nocc, K, w.mk, s));

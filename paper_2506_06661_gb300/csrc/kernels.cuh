@@ -66,13 +66,24 @@ struct MixedKWork {
   int planes;              // BF16 planes per operand (3, 4, 5: 6, 10, 15 plane products)
 };
 
+// FP64 exchange on digit products (digits.cuh): auxiliary rows go through in blocks of px (X, its
+// digits and one SYRK per block) whose half-transforms run pb rows of B at a time.
+struct Fp64KWork {
+  void* Ct;        // digits of C^T
+  void* Bp;        // digits of pb symmetric B_P
+  void* Xd;        // digits of X [nao][px * nocc]
+  double* X;       // [nao][px * nocc]
+  double* Kpart;   // [nsplit][nao][nao]
+  int* err;        // a bounded wait gave up
+  int pb, px, nsplit;
+};
+
 struct JKWork {
   double* Dw;
   double* d;
   double* Jpart;
-  double* X;
-  double* Kpart;
-  int nsplit_j, nsplit_k;
+  int nsplit_j;
+  Fp64KWork fk;
   MixedKWork mk;
 };
 
@@ -101,6 +112,7 @@ int build_B(const double* ao_xyz, const double* ao_exp, int nao, const double* a
 // Bounds-check records of the translation units with kernels (checking build; all zero
 // otherwise).
 int bounds_read_dferr(BoundsRecord*);
+int bounds_read_digits(BoundsRecord*);
 int bounds_read_eig(BoundsRecord*);
 int bounds_read_integrals(BoundsRecord*);
 int bounds_read_jk(BoundsRecord*);
