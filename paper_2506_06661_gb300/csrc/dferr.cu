@@ -141,6 +141,7 @@ __global__ void identity_kernel(double* __restrict__ A, int n) {
 }
 
 struct FitWork {
+  char* subst;
   double *L, *Linv, *m1, *pair_tab, *T, *C, *dv, *G, *maxdiag, *delta;
   int* status;
 };
@@ -153,6 +154,8 @@ void fit_layout(int nao, int naux, bool jac, Arena* a, Sizer* z, FitWork* w) {
   TAKE(double, w->L, (size_t)naux * naux);
   TAKE(double, w->pair_tab, 5 * (size_t)npair_of(nao));
   TAKE(double, w->T, big);
+  // the Jacobian also substitutes into the naux x naux identity
+  TAKE(char, w->subst, std::max(forward_substitution_bytes(ld, naux), forward_substitution_bytes(naux, naux)));
   TAKE(double, w->maxdiag, 1);
   TAKE(double, w->delta, 1);
   TAKE(int, w->status, 1);
@@ -213,7 +216,7 @@ extern "C" int df_fit_residual(const double* ao_xyz, const double* ao_exp, int n
   const double* py = px + npair;
   const double* pz = py + npair;
   const double* pk = pz + npair;
-  DF_TRY(forward_substitution(w.T, ld, ld, w.L, naux, s));
+  DF_TRY(forward_substitution(w.T, ld, ld, w.L, naux, w.subst, s));
   residual_kernel<<<(unsigned)((npair + 255) / 256), 256, 0, s>>>(pp, pk, npair, w.T, ld, naux, sigma);
   DF_LAUNCHED("residual_kernel");
   delta_kernel<<<1, 1024, 0, s>>>(sigma, nao, w.delta);
@@ -222,7 +225,7 @@ extern "C" int df_fit_residual(const double* ao_xyz, const double* ao_exp, int n
     // C = M^-1 (P|mn) = L^-T L^-1 (P|mn): L^-1 explicitly, then C = (L^-1)^T T
     identity_kernel<<<(unsigned)(((long)naux * naux + 255) / 256), 256, 0, s>>>(w.Linv, naux);
     DF_LAUNCHED("identity_kernel");
-    DF_TRY(forward_substitution(w.Linv, naux, naux, w.L, naux, s));
+    DF_TRY(forward_substitution(w.Linv, naux, naux, w.L, naux, w.subst, s));
     DF_TRY(dgemm(true, false, naux, (int)ld, naux, 1.0, w.Linv, naux, 0, w.T, ld, 0, 0.0, w.C, ld, 0, 1, s, 0, 0));
     dim3 g3((unsigned)((ld + 255) / 256), (unsigned)naux);
     int3c_dexp_kernel<<<g3, 256, 0, s>>>(pp, px, py, pz, pk, npair, ld, aux_xyz, aux_exp, w.dv);

@@ -41,7 +41,7 @@ struct Params {
   double alpha, beta;
   double* C;
   long ldc, sC;
-  int lower;
+  int lower, trans;     // lower tiles only; C stored transposed (C[col ldc + row])
   // half-transform
   int nao, naux, p0;
   double* X;
@@ -299,37 +299,52 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
         m = row - P * p.nao;
       }
       unsigned big = 0;
+      const long rstep = p.trans ? 1 : p.ldc, cstep = p.trans ? p.ldc : 1;
 #pragma unroll
       for (int g = 0; g < 2; ++g) {
         if (g >= p.groups) break;
 #pragma unroll
-        for (int j = 0; j < CW; ++j) {
-          const int col = col0 + g * G + half * CW + j;
-          if (col >= p.N) break;
-          const unsigned kb = p.kb[col];
-          // digit d_a has the weight 2^(E - 8 - 9 a), E = field - 1022; hi counts order 3
-          double v = assemble(hi[g][j], lo[g][j], fa + key_field(kb) - 2044 - 16 - 27);
-          if (bada || key_bad(kb)) {
-            v = 0.0;
-            const long k0 = (long)s0 * BK, k1 = min(p.K, k0 + (long)nst * BK);
-            for (long k = k0; k < k1; ++k) {
-              double x;
-              if (p.mode == HALF_TRANSFORM) {
-                const long a = max((long)m, k), c = min((long)m, k);
-                x = p.A0[(long)(p.p0 + P) * p.sam + a * (a + 1) / 2 + c];
-              } else {
-                x = p.A0[row * p.sam + k * p.sak];
-              }
-              v = fma(x, p.B0[col * p.sbn + k * p.sbk], v);
+        for (int j0 = 0; j0 < CW; j0 += 8) {
+          const int colb = col0 + g * G + half * CW + j0;
+          double old[8];  // what the outputs add to, loaded ahead of the stores
+          double* cb = nullptr;
+          if (p.mode == MATRIX) {
+            cb = p.C + (size_t)blockIdx.y * p.sC +
+                 DF_IX((size_t)row * rstep + (size_t)min(colb, p.N - 1) * cstep, p.trans ? (size_t)p.N * p.ldc : (size_t)p.M * p.ldc);
+            if (p.beta != 0.0) {
+#pragma unroll
+              for (int j = 0; j < 8; ++j) old[j] = colb + j < p.N ? cb[j * cstep] : 0.0;
             }
           }
-          if (p.mode == HALF_TRANSFORM) {
-            p.X[DF_IX((size_t)m * p.ldx + p.xcol0 + (size_t)P * p.N + col, (size_t)p.nao * p.ldx)] = v;
-            big = max(big, high_key(v));
-          } else {
-            double* c = p.C + (size_t)blockIdx.y * p.sC + DF_IX((size_t)row * p.ldc + col, (size_t)p.M * p.ldc);
-            const double w = p.alpha * v;
-            *c = p.beta == 0.0 ? w : fma(p.beta, *c, w);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const int col = colb + j;
+            if (col >= p.N) break;
+            const unsigned kb = p.kb[col];
+            // digit d_a has the weight 2^(E - 8 - 9 a), E = field - 1022; hi counts order 3
+            double v = assemble(hi[g][j0 + j], lo[g][j0 + j], fa + key_field(kb) - 2044 - 16 - 27);
+            if (bada || key_bad(kb)) {
+              v = 0.0;
+              const long k0 = (long)s0 * BK, k1 = min(p.K, k0 + (long)nst * BK);
+              for (long k = k0; k < k1; ++k) {
+                double x;
+                if (p.mode == HALF_TRANSFORM) {
+                  const long a = max((long)m, k), c = min((long)m, k);
+                  x = p.A0[(long)(p.p0 + P) * p.sam + a * (a + 1) / 2 + c];
+                } else {
+                  x = p.A0[row * p.sam + k * p.sak];
+                }
+                v = fma(x, p.B0[col * p.sbn + k * p.sbk], v);
+              }
+            }
+            if (p.mode == HALF_TRANSFORM) {
+              p.X[DF_IX((size_t)m * p.ldx + p.xcol0 + (size_t)P * p.N + col, (size_t)p.nao * p.ldx)] = v;
+              big = max(big, high_key(v));
+            } else {
+              // FP64 instructions only where they are needed: +-1 factors flip a sign or add
+              const double w = p.alpha == 1.0 ? v : (p.alpha == -1.0 ? -v : p.alpha * v);
+              cb[j * cstep] = p.beta == 0.0 ? w : (p.beta == 1.0 ? old[j] + w : fma(p.beta, old[j], w));
+            }
           }
         }
       }
@@ -352,21 +367,6 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
 }
 
 // ---- slicing ---------------------------------------------------------------------------
-// Eight consecutive K elements of a row into its NS planes (16-byte stores).
-__device__ __forceinline__ void store_digits8(const double (&x)[8], int f, __nv_bfloat16* out, size_t plane) {
-  unsigned w[NS][4];
-#pragma unroll
-  for (int u = 0; u < 4; ++u) {
-    int a[NS], b[NS];
-    split_digits(x[2 * u], f, a);
-    split_digits(x[2 * u + 1], f, b);
-#pragma unroll
-    for (int j = 0; j < NS; ++j) w[j][u] = pack_digits(a[j], b[j]);
-  }
-#pragma unroll
-  for (int j = 0; j < NS; ++j) *reinterpret_cast<uint4*>(out + j * plane) = make_uint4(w[j][0], w[j][1], w[j][2], w[j][3]);
-}
-
 __device__ __forceinline__ unsigned cta_max_key(unsigned v, unsigned* sh) {
   for (int o = 16; o; o >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, o));
   if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = v;
@@ -616,7 +616,7 @@ int slice_packed(const double* B, long ldb, int nao, int naux, int p0, int np, c
 }
 
 int digit_gemm(const DigitOperand& A, const DigitOperand& B, DigitSource A0, DigitSource B0, double alpha, double beta,
-               double* C, long ldc, long sC, int splits, bool lower, int* err, cudaStream_t s) {
+               double* C, long ldc, long sC, int splits, int shape, int* err, cudaStream_t s) {
   DF_REQUIRE(A.rows < INT_MAX && B.rows < INT_MAX && A.K == B.K, DF_ERR_ARG, "digit GEMM: bad operand sizes");
   Params p{};
   p.mode = MATRIX;
@@ -629,7 +629,8 @@ int digit_gemm(const DigitOperand& A, const DigitOperand& B, DigitSource A0, Dig
   p.C = C;
   p.ldc = ldc;
   p.sC = sC;
-  p.lower = lower;
+  p.lower = shape == DIGIT_LOWER;
+  p.trans = shape == DIGIT_TRANSPOSED;
   p.A0 = A0.p;
   p.sam = A0.sr;
   p.sak = A0.sk;

@@ -73,6 +73,21 @@ __device__ __forceinline__ unsigned pack_digits(int a, int b) {
   return __byte_perm(__float_as_uint(fa), __float_as_uint(fb), 0x7632);
 }
 
+// Eight consecutive K elements of a row into its NS planes (16-byte stores).
+__device__ __forceinline__ void store_digits8(const double (&x)[8], int f, __nv_bfloat16* out, size_t plane) {
+  unsigned w[NS][4];
+#pragma unroll
+  for (int u = 0; u < 4; ++u) {
+    int a[NS], b[NS];
+    split_digits(x[2 * u], f, a);
+    split_digits(x[2 * u + 1], f, b);
+#pragma unroll
+    for (int j = 0; j < NS; ++j) w[j][u] = pack_digits(a[j], b[j]);
+  }
+#pragma unroll
+  for (int j = 0; j < NS; ++j) *reinterpret_cast<uint4*>(out + j * plane) = make_uint4(w[j][0], w[j][1], w[j][2], w[j][3]);
+}
+
 }  // namespace digits
 
 // Digit planes of a matrix operand [NS][rows][ld] over K, and the row keys.
@@ -93,14 +108,16 @@ int slice_packed(const double* B, long ldb, int nao, int naux, int p0, int np, c
 int slice_with_keys(const double* A, long lda, const DigitOperand& o, cudaStream_t s);
 
 // C[z][m][n] = alpha sum_k a_mk b_nk + beta C[z][m][n], K split in `splits` ranges (slices sC apart);
-// lower: only tiles that reach n <= m.  A0 (a_mk = A0[m sam + k sak]) and B0 are the operands'
+// DIGIT_LOWER: only tiles that reach n <= m; DIGIT_TRANSPOSED: C[n ldc + m], whose lanes store
+// consecutive m.  A0 (a_mk = A0[m sam + k sak]) and B0 are the operands'
 // FP64 originals.  err: device flag raised when a bounded wait gave up (C is then incomplete).
+enum DigitShape { DIGIT_FULL = 0, DIGIT_LOWER = 1, DIGIT_TRANSPOSED = 2 };
 struct DigitSource {
   const double* p;
   long sr, sk;
 };
 int digit_gemm(const DigitOperand& A, const DigitOperand& B, DigitSource A0, DigitSource B0, double alpha, double beta,
-               double* C, long ldc, long sC, int splits, bool lower, int* err, cudaStream_t s);
+               double* C, long ldc, long sC, int splits, int shape, int* err, cudaStream_t s);
 // Half-transform X[m][(P - p0) nocc + i] = sum_n B_P[m][n] C[n][i] (row stride ldx) of the rows
 // of slice_packed, and xkey[m] = max over the row (atomicMax: zero it first).
 int digit_half_transform(const DigitOperand& A, const DigitOperand& Ct, const double* B, long ldb, int nao, int naux,

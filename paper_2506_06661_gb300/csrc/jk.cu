@@ -497,7 +497,8 @@ int build_K_fp64(const double* B64, long ld, int nao, int naux, const double* C,
     ProfScope ps("k_syrk_fp64", s);
     DF_TRY(slice_with_keys(w.X, kdim, xd, s));
     const DigitSource src{w.X, kdim, 1};
-    DF_TRY(digit_gemm(xd, xd, src, src, 1.0, x0 ? 1.0 : 0.0, w.Kpart, nao, (long)nao * nao, w.nsplit, true, w.err, s));
+    DF_TRY(digit_gemm(xd, xd, src, src, 1.0, x0 ? 1.0 : 0.0, w.Kpart, nao, (long)nao * nao, w.nsplit, DIGIT_LOWER, w.err,
+                      s));
   }
   long nn = (long)nao * nao;
   ksum_mirror_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(w.Kpart, w.nsplit, nao, w.err, K);
@@ -528,11 +529,11 @@ int run_jk(const void* B, int nao, int naux, int precision, const double* D, con
 }
 
 int build_B(const double* ao_xyz, const double* ao_exp, int nao, const double* aux_xyz, const double* aux_exp,
-            int naux, const double* Lfac, int precision, void* Bbuf, double* pair_tab, cudaStream_t s) {
+            int naux, const double* Lfac, int precision, void* Bbuf, double* pair_tab, void* subst, cudaStream_t s) {
   BLayout L = B_layout(nao, naux, precision, mixed_planes());
   double* B64 = (double*)((char*)Bbuf + L.off64);
   DF_TRY(launch_int3c(ao_xyz, ao_exp, nao, aux_xyz, aux_exp, naux, B64, L.ld, pair_tab, s));
-  DF_TRY(forward_substitution(B64, L.ld, L.ld, Lfac, naux, s));
+  DF_TRY(forward_substitution(B64, L.ld, L.ld, Lfac, naux, subst, s));
   if (precision == DF_MIXED) {
     DF_REQUIRE(naux <= 65535, DF_ERR_ARG, "naux too large");
     PlaneOut po{};
@@ -558,8 +559,8 @@ extern "C" size_t df_B_bytes(int nao, int naux, int precision) {
 }
 
 extern "C" size_t df_build_B_work_bytes(int nao, int naux) {
-  (void)naux;
-  return nao > 0 ? align_up(sizeof(double) * 5 * (size_t)npair_of(nao), 256) : 0;
+  if (nao <= 0 || naux <= 0) return nao > 0 ? align_up(sizeof(double) * 5 * (size_t)npair_of(nao), 256) : 0;
+  return align_up(sizeof(double) * 5 * (size_t)npair_of(nao), 256) + forward_substitution_bytes(B_ld(nao), naux);
 }
 
 extern "C" int df_build_B(const double* ao_xyz, const double* ao_exp, int nao, const double* aux_xyz,
@@ -574,7 +575,8 @@ extern "C" int df_build_B(const double* ao_xyz, const double* ao_exp, int nao, c
   DF_REQUIRE(work && work_bytes >= df_build_B_work_bytes(nao, naux), DF_ERR_NOMEM,
              "df_build_B: workspace of %zu bytes < %zu", work_bytes, df_build_B_work_bytes(nao, naux));
   DF_REQUIRE(precision == DF_FP64 || naux <= 65535, DF_ERR_ARG, "df_build_B: naux > 65535 in mixed mode");
-  return build_B(ao_xyz, ao_exp, nao, aux_xyz, aux_exp, naux, L, precision, B, (double*)work, s);
+  return build_B(ao_xyz, ao_exp, nao, aux_xyz, aux_exp, naux, L, precision, B, (double*)work,
+                 (char*)work + align_up(sizeof(double) * 5 * (size_t)npair_of(nao), 256), s);
 }
 
 extern "C" int df_B_get_packed(const void* B, int nao, int naux, int P, double* row, cudaStream_t s) {

@@ -25,7 +25,9 @@ int dgemm(bool ta, bool tb, int M, int N, int K, double alpha, const double* A, 
           long ldb, long sB, double beta, double* C, long ldc, long sC, int batch, cudaStream_t s, long kchunk,
           int lower_only);
 int cholesky_inplace(double* A, int n, int* d_status, double* d_maxdiag, double tol, cudaStream_t s);
-int forward_substitution(double* R, long ld, long ncol, const double* L, int naux, cudaStream_t s);
+// work: forward_substitution_bytes(ncol, naux)
+size_t forward_substitution_bytes(long ncol, int naux);
+int forward_substitution(double* R, long ld, long ncol, const double* L, int naux, void* work, cudaStream_t s);
 
 // ---- eigensolver (eig.cu) ------------------------------------------------------------
 size_t eigh_scratch_doubles(int n);
@@ -107,7 +109,7 @@ int build_J(const void* Bbuf, const BLayout& L, int nao, int naux, int precision
 int run_jk(const void* B, int nao, int naux, int precision, const double* D, const double* C, int nocc, double* J,
            double* K, const JKWork& w, cudaStream_t s);
 int build_B(const double* ao_xyz, const double* ao_exp, int nao, const double* aux_xyz, const double* aux_exp,
-            int naux, const double* Lfac, int precision, void* Bbuf, double* pair_tab, cudaStream_t s);
+            int naux, const double* Lfac, int precision, void* Bbuf, double* pair_tab, void* subst, cudaStream_t s);
 
 // Bounds-check records of the translation units with kernels (checking build; all zero
 // otherwise).

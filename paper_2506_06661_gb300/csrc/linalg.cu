@@ -4,7 +4,10 @@
 // whitening (arXiv 2506.06661, Section "Density fitting").  On this GPU FP64 runs at
 // about 1.9 FMA/clk/SM, so these kernels are FP64-ALU bound by design; they only need
 // coalesced loads and enough independent FMAs per thread.
+#include <algorithm>
+
 #include "common.cuh"
+#include "digits.cuh"
 #include "kernels.cuh"
 
 namespace dfscf {
@@ -217,14 +220,20 @@ int cholesky_inplace(double* A, int n, int* d_status, double* d_maxdiag, double 
 }
 
 // ---- forward substitution B = L^-1 R ---------------------------------------------------
-// Rows k0..k0+b of R are solved against the diagonal block of L, one lane per column.
+// Rows k0..k0+NB of R are solved against the diagonal block of L, one lane per column.  FP64-bound
+// (NB (NB - 1) / 2 FMAs per column and block), so divisions are a product with the reciprocal and
+// one correction step.  With `out`, the digits (digits.cuh) of the solved rows, as row c over the
+// NB terms, are written from registers for the update that follows.
 template <int NB>
 __global__ void __launch_bounds__(128) trsm_diag_kernel(double* __restrict__ R, long ld, long ncol,
-                                                        const double* __restrict__ L, int naux, int k0) {
+                                                        const double* __restrict__ L, int naux, int k0,
+                                                        __nv_bfloat16* __restrict__ out, unsigned* __restrict__ key) {
   __shared__ double Lk[NB][NB];
+  __shared__ double rinv[NB];
   for (int e = threadIdx.x; e < NB * NB; e += blockDim.x) {
     int i = e / NB, j = e % NB;
     Lk[i][j] = (j <= i) ? L[(size_t)(k0 + i) * naux + k0 + j] : 0.0;
+    if (i == j) rinv[i] = 1.0 / L[(size_t)(k0 + i) * naux + k0 + i];
   }
   __syncthreads();
   long c = (long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -237,10 +246,28 @@ __global__ void __launch_bounds__(128) trsm_diag_kernel(double* __restrict__ R, 
     double v = x[p];
 #pragma unroll
     for (int q = 0; q < p; ++q) v = fma(-Lk[p][q], x[q], v);
-    x[p] = v / Lk[p][p];
+    const double r = rinv[p], q = v * r;
+    const double q1 = fma(fma(-Lk[p][p], q, v), r, q);
+    x[p] = isfinite(r) && r != 0.0 ? (isfinite(q1) ? q1 : q) : v / Lk[p][p];
   }
+  unsigned t = 0;
 #pragma unroll
-  for (int p = 0; p < NB; ++p) R[(size_t)(k0 + p) * ld + c] = x[p];
+  for (int p = 0; p < NB; ++p) {
+    R[(size_t)(k0 + p) * ld + c] = x[p];
+    t = max(t, digits::high_key(x[p]));
+  }
+  if (out) {
+    key[c] = t;
+    const bool bad = digits::key_bad(t);
+    const int f = digits::key_field(t);
+#pragma unroll
+    for (int p = 0; p < NB; p += 8) {
+      double y[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) y[u] = bad ? 0.0 : x[p + u];
+      digits::store_digits8(y, f, out + (size_t)c * NB + p, (size_t)ncol * NB);
+    }
+  }
 }
 
 __global__ void trsm_diag_generic_kernel(double* __restrict__ R, long ld, long ncol, const double* __restrict__ L,
@@ -254,21 +281,72 @@ __global__ void trsm_diag_generic_kernel(double* __restrict__ R, long ld, long n
   }
 }
 
-int forward_substitution(double* R, long ld, long ncol, const double* L, int naux, cudaStream_t s) {
-  constexpr int NB = 32;
-  for (int k0 = 0; k0 < naux; k0 += NB) {
-    int b = min(NB, naux - k0);
-    unsigned blocks = (unsigned)((ncol + 127) / 128);
-    if (b == NB)
-      trsm_diag_kernel<NB><<<blocks, 128, 0, s>>>(R, ld, ncol, L, naux, k0);
-    else
-      trsm_diag_generic_kernel<<<blocks, 128, 0, s>>>(R, ld, ncol, L, naux, k0, b);
-    DF_LAUNCHED("trsm_diag_kernel");
-    int rest = naux - k0 - b;
+// A wait of the tensor-core updates gave up: no row may pass for a result.
+__global__ void poison_kernel(const int* __restrict__ err, double* __restrict__ R, long n) {
+  if (*err)
+    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
+      R[i] = __longlong_as_double(0x7ff8000000000000LL);
+}
+
+// Two levels of blocks.  A block of 32 rows is solved in FP64 (FP64 work grows with the block);
+// its digits update the rest of the 128 rows around it; the 128 solved rows together update all
+// rows below, so that those are read and written once per 128 rows.  Columns go through in
+// chunks, which bounds the digits of X to 120 MB.
+constexpr int FS_NB = 32, FS_NBO = 128;
+constexpr long FS_COLS = 65536;
+
+size_t forward_substitution_bytes(long ncol, int naux) {
+  if (naux <= FS_NB) return 256;
+  return digit_operand_bytes(std::min(ncol, FS_COLS), FS_NBO) + digit_operand_bytes(naux, FS_NBO) + 256;
+}
+
+int forward_substitution(double* R, long ld, long ncol, const double* L, int naux, void* work, cudaStream_t s) {
+  const long cmax = std::min(ncol, FS_COLS);
+  char* xmem = (char*)work + 256;
+  char* lmem = xmem + digit_operand_bytes(cmax, FS_NBO);
+  int* err = (int*)work;
+  if (naux > FS_NB) DF_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
+  // R[r0.., :] -= L[r0.., k0..k0+b) R[k0..k0+b, :] over nr rows and the columns of chunk c0 (digits
+  // of R's rows k0.. in x)
+  auto update = [&](int r0, int nr, int k0, int b, long c0, const DigitOperand& x, const DigitOperand& l) -> int {
+    return digit_gemm(x, l, DigitSource{R + (size_t)k0 * ld + c0, 1, ld}, DigitSource{L + (size_t)r0 * naux + k0, naux, 1},
+                      -1.0, 1.0, R + (size_t)r0 * ld + c0, ld, 0, 1, DIGIT_TRANSPOSED, err, s);
+  };
+  for (int j0 = 0; j0 < naux; j0 += FS_NBO) {
+    const int nb = std::min(FS_NBO, naux - j0);
+    for (int k0 = j0; k0 < j0 + nb; k0 += FS_NB) {
+      const int b = std::min(FS_NB, j0 + nb - k0);
+      const int rest = j0 + nb - k0 - b;  // rows of this 128-row block still to solve
+      DigitOperand l;
+      if (rest > 0) {
+        l = digit_operand(lmem, rest, b);
+        DF_TRY(slice_matrix(L + (size_t)(k0 + b) * naux + k0, naux, false, l, s));
+      }
+      for (long c0 = 0; c0 < ncol; c0 += FS_COLS) {
+        const long nc = std::min(FS_COLS, ncol - c0);
+        const unsigned blocks = (unsigned)((nc + 127) / 128);
+        const DigitOperand x = digit_operand(xmem, nc, b);
+        if (b == FS_NB)
+          trsm_diag_kernel<FS_NB><<<blocks, 128, 0, s>>>(R + c0, ld, nc, L, naux, k0, rest > 0 ? x.p : nullptr, x.key);
+        else
+          trsm_diag_generic_kernel<<<blocks, 128, 0, s>>>(R + c0, ld, nc, L, naux, k0, b);
+        DF_LAUNCHED("trsm_diag_kernel");
+        if (rest > 0) DF_TRY(update(k0 + b, rest, k0, b, c0, x, l));
+      }
+    }
+    const int r0 = j0 + nb, rest = naux - r0;
     if (rest <= 0) break;
-    // R[k0+b:, :] -= L[k0+b:, k0:k0+b] R[k0:k0+b, :], in column chunks (grid.x limit is ample)
-    DF_TRY(dgemm(false, false, rest, (int)ncol, b, -1.0, L + (size_t)(k0 + b) * naux + k0, naux, 0,
-                 R + (size_t)k0 * ld, ld, 0, 1.0, R + (size_t)(k0 + b) * ld, ld, 0, 1, s, 0, 0));
+    const DigitOperand l = digit_operand(lmem, rest, nb);
+    DF_TRY(slice_matrix(L + (size_t)r0 * naux + j0, naux, false, l, s));
+    for (long c0 = 0; c0 < ncol; c0 += FS_COLS) {
+      const DigitOperand x = digit_operand(xmem, std::min(FS_COLS, ncol - c0), nb);
+      DF_TRY(slice_matrix(R + (size_t)j0 * ld + c0, ld, true, x, s));
+      DF_TRY(update(r0, rest, j0, nb, c0, x, l));
+    }
+  }
+  if (naux > FS_NB) {
+    poison_kernel<<<64, 256, 0, s>>>(err, R, ncol);
+    DF_LAUNCHED("poison_kernel");
   }
   return DF_OK;
 }

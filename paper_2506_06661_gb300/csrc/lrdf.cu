@@ -174,6 +174,7 @@ extern "C" size_t df_lrdf_build_work_bytes(int nao, int naux) {
   z.take<int>(1);
   z.take<double>(1);
   z.take<double>(5 * (size_t)npair_of(nao));
+  z.take<char>(forward_substitution_bytes(B_ld(nao), naux));
   return z.used;
 }
 
@@ -193,6 +194,7 @@ extern "C" int df_lrdf_build(const double* ao_xyz, const double* ao_exp, int nao
   int* status = a.take<int>(1);
   double* maxdiag = a.take<double>(1);
   double* pair_tab = a.take<double>(5 * (size_t)npair_of(nao));
+  void* subst = a.take<char>(forward_substitution_bytes(B_ld(nao), naux));
   DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, L, s, omega));
   DF_TRY(cholesky_inplace(L, naux, status, maxdiag, 1e-14, s));
   int h = -1;
@@ -202,7 +204,7 @@ extern "C" int df_lrdf_build(const double* ao_xyz, const double* ao_exp, int nao
   const long ld = B_ld(nao);
   double* B64 = (double*)B;
   DF_TRY(launch_int3c(ao_xyz, ao_exp, nao, aux_xyz, aux_exp, naux, B64, ld, pair_tab, s, omega));
-  DF_TRY(forward_substitution(B64, ld, ld, L, naux, s));
+  DF_TRY(forward_substitution(B64, ld, ld, L, naux, subst, s));
   return DF_OK;
 }
 

@@ -606,6 +606,7 @@ struct ScfWork {
   double* dav;  // Davidson subspace of the stability analysis: V, H V [kDavidsonMax][nvir * nocc], G, scalars
   char* guess_ws;      // learned-guess prediction (guess_density), 5 basis functions per centre
   size_t guess_bytes;
+  char* subst;    // digits of the whitening
   void* eig_aux;  // p vector and grid barrier of the multi-SM eigensolver
   ScfStatus* st;
   DiisState* diis;
@@ -623,6 +624,7 @@ static void scf_layout(int nao, int naux, int nocc, int precision, Arena* a, Siz
   w->guess_ws = nullptr;
   if (w->guess_bytes) TAKE(char, w->guess_ws, w->guess_bytes);
   TAKE(double, w->pair_tab, 5 * (size_t)npair_of(nao));
+  TAKE(char, w->subst, forward_substitution_bytes(B_ld(nao), naux));
   TAKE(double, w->S, nn);
   TAKE(double, w->h, nn);
   TAKE(double, w->V, nn);
@@ -833,7 +835,7 @@ static int setup_launch(ScfMol& M) {
   DF_TRY(launch_int2c(mol->aux_xyz, mol->aux_exp, naux, W.L, s));
   DF_TRY(cholesky_inplace(W.L, naux, W.chol_status, W.maxdiag, 1e-14, s));
   DF_TRY(build_B(mol->ao_xyz, mol->ao_exp, nao, mol->aux_xyz, mol->aux_exp, naux, W.L, M.opt.precision, W.B,
-                 W.pair_tab, s));
+                 W.pair_tab, W.subst, s));
   DF_CUDA(cudaMemcpyAsync(W.T1, W.S, sizeof(double) * nn, cudaMemcpyDeviceToDevice, s));
   DF_TRY(eig_rows(W.T1, nao, W.eps, W.ZT, W, s));
   DF_CUDA(cudaMemcpyAsync(M.h_eps, W.eps, sizeof(double) * nao, cudaMemcpyDeviceToHost, s));
