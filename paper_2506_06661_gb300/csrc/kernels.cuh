@@ -24,7 +24,9 @@ int launch_enuc(const double* xyz, const double* z, int natm, double* out, cudaS
 int dgemm(bool ta, bool tb, int M, int N, int K, double alpha, const double* A, long lda, long sA, const double* B,
           long ldb, long sB, double beta, double* C, long ldc, long sC, int batch, cudaStream_t s, long kchunk,
           int lower_only);
-int cholesky_inplace(double* A, int n, int* d_status, double* d_maxdiag, double tol, cudaStream_t s);
+// work: cholesky_bytes(n), at most forward_substitution_bytes(_, n)
+size_t cholesky_bytes(int n);
+int cholesky_inplace(double* A, int n, int* d_status, double* d_maxdiag, double tol, void* work, cudaStream_t s);
 // work: forward_substitution_bytes(ncol, naux)
 size_t forward_substitution_bytes(long ncol, int naux);
 int forward_substitution(double* R, long ld, long ncol, const double* L, int naux, void* work, cudaStream_t s);

@@ -113,7 +113,11 @@ int dgemm(bool ta, bool tb, int M, int N, int K, double alpha, const double* A, 
 }
 
 // ---- Cholesky ----------------------------------------------------------------------
-constexpr int CH_NB = 64;
+// Right-looking in blocks of 32: one warp factors the diagonal block in registers, one lane per
+// row solves the panel below it and writes its digits, and the trailing update runs on digit
+// products.  The chain of 3 launches per block bounds it (n / 32 blocks): small blocks keep
+// the serial FP64 part of each link short.
+constexpr int CH_NB = 32;
 
 __global__ void chol_init_kernel(const double* __restrict__ A, int n, double* maxdiag, int* status) {
   __shared__ double sh[32];
@@ -131,63 +135,80 @@ __global__ void chol_init_kernel(const double* __restrict__ A, int n, double* ma
   }
 }
 
-// Factor the b x b diagonal block at (k0, k0) in shared memory (right-looking, one CTA).
-__global__ void __launch_bounds__(256) chol_diag_kernel(double* __restrict__ A, int n, int k0, int b,
-                                                        const double* maxdiag, int* status, double tol) {
-  __shared__ double T[CH_NB][CH_NB + 1];
-  __shared__ int fail;
+// Factor the b x b diagonal block at (k0, k0): lane i holds row i (right-looking).
+__global__ void __launch_bounds__(32) chol_diag_kernel(double* __restrict__ A, int n, int k0, int b,
+                                                       const double* maxdiag, int* status, double tol) {
   if (*status >= 0) return;
-  for (int e = threadIdx.x; e < b * b; e += blockDim.x) {
-    int i = e / b, j = e % b;
-    T[i][j] = A[(size_t)(k0 + i) * n + k0 + j];
-  }
-  if (threadIdx.x == 0) fail = -1;
-  __syncthreads();
-  double thr = tol * *maxdiag;
-  for (int j = 0; j < b; ++j) {
-    if (threadIdx.x == 0) {
-      double piv = T[j][j];
-      if (!(piv > thr)) fail = j;
-      else T[j][j] = sqrt(piv);
+  const int i = threadIdx.x;
+  double row[CH_NB];
+#pragma unroll
+  for (int j = 0; j < CH_NB; ++j) row[j] = (i < b && j <= i) ? A[(size_t)(k0 + i) * n + k0 + j] : 0.0;
+  const double thr = tol * *maxdiag;
+  int fail = -1;
+#pragma unroll
+  for (int j = 0; j < CH_NB; ++j) {
+    if (j < b && fail < 0) {
+      const double piv = __shfl_sync(0xffffffffu, row[j], j);
+      if (!(piv > thr)) {
+        fail = j;
+      } else {
+        const double l = sqrt(piv);
+        row[j] = i == j ? l : row[j] / l;  // rows above j hold zeros there
+#pragma unroll
+        for (int c = j + 1; c < CH_NB; ++c) {
+          const double lc = __shfl_sync(0xffffffffu, row[j], c);
+          if (c <= i) row[c] = fma(-row[j], lc, row[c]);
+        }
+      }
     }
-    __syncthreads();
-    if (fail >= 0) break;
-    double ljj = T[j][j];
-    for (int i = j + 1 + threadIdx.x; i < b; i += blockDim.x) T[i][j] /= ljj;
-    __syncthreads();
-    int rem = b - j - 1;
-    for (int e = threadIdx.x; e < rem * rem; e += blockDim.x) {
-      int i = j + 1 + e / rem, c = j + 1 + e % rem;
-      if (c <= i) T[i][c] -= T[i][j] * T[c][j];
-    }
-    __syncthreads();
   }
   if (fail >= 0) {
-    if (threadIdx.x == 0) atomicCAS(status, -1, k0 + fail);
+    if (i == 0) atomicCAS(status, -1, k0 + fail);
     return;
   }
-  for (int e = threadIdx.x; e < b * b; e += blockDim.x) {
-    int i = e / b, j = e % b;
-    A[(size_t)(k0 + i) * n + k0 + j] = (j <= i) ? T[i][j] : 0.0;
-  }
+#pragma unroll
+  for (int j = 0; j < CH_NB; ++j)
+    if (i < b && j < b) A[(size_t)(k0 + i) * n + k0 + j] = row[j];
 }
 
-// Panel below the diagonal block: L[i, k0:k0+b] = A[i, k0:k0+b] L_kk^-T, one lane per row.
-__global__ void chol_panel_kernel(double* __restrict__ A, int n, int k0, int b, const int* status) {
-  __shared__ double Lk[CH_NB][CH_NB + 1];
+// Panel below the diagonal block: L[i, k0:k0+32] = A[i, k0:k0+32] L_kk^-T, one lane per row, few
+// lanes per CTA to spread the FP64 work over the SMs; the row's digits for the trailing update.
+__global__ void __launch_bounds__(32) chol_panel_kernel(double* __restrict__ A, int n, int k0, const int* status,
+                                                        __nv_bfloat16* __restrict__ out, unsigned* __restrict__ key) {
+  __shared__ double Lk[CH_NB][CH_NB];
+  __shared__ double rinv[CH_NB];
   if (*status >= 0) return;
-  for (int e = threadIdx.x; e < b * b; e += blockDim.x) {
-    int i = e / b, j = e % b;
-    Lk[i][j] = A[(size_t)(k0 + i) * n + k0 + j];
-  }
+  for (int e = threadIdx.x; e < CH_NB * CH_NB; e += blockDim.x)
+    Lk[e / CH_NB][e % CH_NB] = A[(size_t)(k0 + e / CH_NB) * n + k0 + e % CH_NB];
+  rinv[threadIdx.x] = 1.0 / A[(size_t)(k0 + threadIdx.x) * n + k0 + threadIdx.x];
   __syncthreads();
-  int i = k0 + b + blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  double* row = A + (size_t)i * n + k0;
-  for (int j = 0; j < b; ++j) {
-    double x = row[j];
-    for (int m = 0; m < j; ++m) x -= row[m] * Lk[j][m];
-    row[j] = x / Lk[j][j];
+  const int r = blockIdx.x * blockDim.x + threadIdx.x, rows = n - k0 - CH_NB;
+  if (r >= rows) return;
+  double* a = A + (size_t)(k0 + CH_NB + r) * n + k0;
+  double x[CH_NB];
+#pragma unroll
+  for (int j = 0; j < CH_NB; ++j) x[j] = a[j];
+  unsigned t = 0;
+#pragma unroll
+  for (int j = 0; j < CH_NB; ++j) {
+    double v = x[j];
+#pragma unroll
+    for (int m = 0; m < j; ++m) v = fma(-Lk[j][m], x[m], v);
+    const double q = v * rinv[j];  // pivots are positive and normal: one correction rounds the quotient
+    x[j] = fma(fma(-Lk[j][j], q, v), rinv[j], q);
+    t = max(t, digits::high_key(x[j]));
+  }
+#pragma unroll
+  for (int j = 0; j < CH_NB; ++j) a[j] = x[j];
+  key[r] = t;
+  const bool bad = digits::key_bad(t);
+  const int f = digits::key_field(t);
+#pragma unroll
+  for (int j = 0; j < CH_NB; j += 8) {
+    double y[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) y[u] = bad ? 0.0 : x[j + u];
+    digits::store_digits8(y, f, out + (size_t)r * CH_NB + j, (size_t)rows * CH_NB);
   }
 }
 
@@ -198,24 +219,38 @@ __global__ void zero_upper_kernel(double* __restrict__ A, int n) {
   if (j > i) A[e] = 0.0;
 }
 
-int cholesky_inplace(double* A, int n, int* d_status, double* d_maxdiag, double tol, cudaStream_t s) {
+// A wait of the tensor-core updates gave up: no row may pass for a result.
+__global__ void poison_kernel(const int* __restrict__ err, double* __restrict__ R, long n) {
+  if (*err)
+    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
+      R[i] = __longlong_as_double(0x7ff8000000000000LL);
+}
+
+size_t cholesky_bytes(int n) { return 256 + (n > CH_NB ? digit_operand_bytes(n, CH_NB) : 0); }
+
+int cholesky_inplace(double* A, int n, int* d_status, double* d_maxdiag, double tol, void* work, cudaStream_t s) {
+  int* err = (int*)work;
+  DF_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
   chol_init_kernel<<<1, 1024, 0, s>>>(A, n, d_maxdiag, d_status);
   DF_LAUNCHED("chol_init_kernel");
   for (int k0 = 0; k0 < n; k0 += CH_NB) {
     int b = min(CH_NB, n - k0);
-    chol_diag_kernel<<<1, 256, 0, s>>>(A, n, k0, b, d_maxdiag, d_status, tol);
+    chol_diag_kernel<<<1, 32, 0, s>>>(A, n, k0, b, d_maxdiag, d_status, tol);
     DF_LAUNCHED("chol_diag_kernel");
     int rest = n - k0 - b;
     if (rest <= 0) break;
-    chol_panel_kernel<<<(rest + 127) / 128, 128, 0, s>>>(A, n, k0, b, d_status);
+    const DigitOperand l = digit_operand((char*)work + 256, rest, CH_NB);
+    chol_panel_kernel<<<(rest + 31) / 32, 32, 0, s>>>(A, n, k0, d_status, l.p, l.key);
     DF_LAUNCHED("chol_panel_kernel");
     int k1 = k0 + b;
-    DF_TRY(dgemm(false, true, rest, rest, b, -1.0, A + (size_t)k1 * n + k0, n, 0, A + (size_t)k1 * n + k0, n, 0, 1.0,
-                 A + (size_t)k1 * n + k1, n, 0, 1, s, 0, 1));
+    const DigitSource src{A + (size_t)k1 * n + k0, n, 1};
+    DF_TRY(digit_gemm(l, l, src, src, -1.0, 1.0, A + (size_t)k1 * n + k1, n, 0, 1, DIGIT_LOWER, err, s));
   }
   long nn = (long)n * n;
   zero_upper_kernel<<<(unsigned)((nn + 255) / 256), 256, 0, s>>>(A, n);
   DF_LAUNCHED("zero_upper_kernel");
+  poison_kernel<<<1, 256, 0, s>>>(err, A, n);
+  DF_LAUNCHED("poison_kernel");
   return DF_OK;
 }
 
@@ -281,13 +316,6 @@ __global__ void trsm_diag_generic_kernel(double* __restrict__ R, long ld, long n
   }
 }
 
-// A wait of the tensor-core updates gave up: no row may pass for a result.
-__global__ void poison_kernel(const int* __restrict__ err, double* __restrict__ R, long n) {
-  if (*err)
-    for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x)
-      R[i] = __longlong_as_double(0x7ff8000000000000LL);
-}
-
 // Two levels of blocks.  A block of 32 rows is solved in FP64 (FP64 work grows with the block);
 // its digits update the rest of the 128 rows around it; the 128 solved rows together update all
 // rows below, so that those are read and written once per 128 rows.  Columns go through in
@@ -296,7 +324,7 @@ constexpr int FS_NB = 32, FS_NBO = 128;
 constexpr long FS_COLS = 65536;
 
 size_t forward_substitution_bytes(long ncol, int naux) {
-  if (naux <= FS_NB) return 256;
+  if (naux <= FS_NB) return 256;  // (also enough for cholesky_bytes(naux), which comes first)
   return digit_operand_bytes(std::min(ncol, FS_COLS), FS_NBO) + digit_operand_bytes(naux, FS_NBO) + 256;
 }
 
@@ -356,8 +384,7 @@ int forward_substitution(double* R, long ld, long ncol, const double* L, int nau
 using namespace dfscf;
 
 extern "C" size_t df_metric_chol_work_bytes(int naux) {
-  (void)naux;
-  return 512;
+  return naux > 0 ? 512 + cholesky_bytes(naux) : 512;
 }
 
 extern "C" int df_metric_chol(const double* aux_xyz, const double* aux_exp, int naux, double* L, double* M_out,
@@ -371,7 +398,7 @@ extern "C" int df_metric_chol(const double* aux_xyz, const double* aux_exp, int 
   double* d_maxdiag = (double*)((char*)work + 256);
   DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, L, s));
   if (M_out) DF_CUDA(cudaMemcpyAsync(M_out, L, sizeof(double) * naux * naux, cudaMemcpyDeviceToDevice, s));
-  DF_TRY(cholesky_inplace(L, naux, d_status, d_maxdiag, 1e-14, s));
+  DF_TRY(cholesky_inplace(L, naux, d_status, d_maxdiag, 1e-14, (char*)work + 512, s));
   int h_status = -1;
   DF_CUDA(cudaMemcpyAsync(&h_status, d_status, sizeof(int), cudaMemcpyDeviceToHost, s));
   DF_CUDA(cudaStreamSynchronize(s));

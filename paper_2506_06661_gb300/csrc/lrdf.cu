@@ -196,7 +196,7 @@ extern "C" int df_lrdf_build(const double* ao_xyz, const double* ao_exp, int nao
   double* pair_tab = a.take<double>(5 * (size_t)npair_of(nao));
   void* subst = a.take<char>(forward_substitution_bytes(B_ld(nao), naux));
   DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, L, s, omega));
-  DF_TRY(cholesky_inplace(L, naux, status, maxdiag, 1e-14, s));
+  DF_TRY(cholesky_inplace(L, naux, status, maxdiag, 1e-14, subst, s));
   int h = -1;
   DF_CUDA(cudaMemcpyAsync(&h, status, sizeof(int), cudaMemcpyDeviceToHost, s));
   DF_CUDA(cudaStreamSynchronize(s));

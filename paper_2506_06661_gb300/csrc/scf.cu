@@ -833,7 +833,7 @@ static int setup_launch(ScfMol& M) {
   DF_LAUNCHED("axpy_kernel");
   DF_TRY(launch_enuc(mol->xyz, mol->charges, mol->natm, W.enuc, s));
   DF_TRY(launch_int2c(mol->aux_xyz, mol->aux_exp, naux, W.L, s));
-  DF_TRY(cholesky_inplace(W.L, naux, W.chol_status, W.maxdiag, 1e-14, s));
+  DF_TRY(cholesky_inplace(W.L, naux, W.chol_status, W.maxdiag, 1e-14, W.subst, s));
   DF_TRY(build_B(mol->ao_xyz, mol->ao_exp, nao, mol->aux_xyz, mol->aux_exp, naux, W.L, M.opt.precision, W.B,
                  W.pair_tab, W.subst, s));
   DF_CUDA(cudaMemcpyAsync(W.T1, W.S, sizeof(double) * nn, cudaMemcpyDeviceToDevice, s));
