@@ -26,3 +26,41 @@ __device__ __forceinline__ double boys_f0(double t) {
   if (t > 40.0) return half_sqrt_pi / s;
   return half_sqrt_pi * erf(s) / s;
 }
+
+// ---- tabulated F0 ------------------------------------------------------------------------
+// FP64 issues at 2 lanes/clk/SM here, and erf, the square roots and the divisions of one Coulomb
+// integral take about 140 FP64 instructions.  The integral kernels below 40 therefore use the
+// Taylor series F0(t0 + d) = sum_j (-d)^j F_j(t0) / j! around the nearest t0 = k / 32 (degree 6:
+// the remainder is under 2^-55 of F0), and one reciprocal square root above.  The table (1281
+// rows of 8 doubles, 82 KB) stays in L1; a kernel fills it before the integrals, as
+// it takes 3 us.
+constexpr int BOYS_ROWS = 40 * 32 + 1, BOYS_STRIDE = 8;
+constexpr size_t BOYS_TABLE = (size_t)BOYS_ROWS * BOYS_STRIDE;
+
+// 1 / sqrt(a) to about 1 ulp in 5 FP64 instructions: the hardware's 2^-20 estimate and one step of
+// third order (Householder): y (1 + e/2 + 3 e^2/8), e = 1 - a y^2.
+__device__ __forceinline__ double rsqrt_fast(double a) {
+  const unsigned h = (unsigned)__double2hiint(a);
+  if (h - 0x00100000u >= 0x7fd00000u) return 1.0 / sqrt(a);  // not a positive normal number below 2^1023
+  double y;
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double e = fma(-(a * y), y, 1.0);
+  return fma(y * e, fma(0.375, e, 0.5), y);
+}
+
+__device__ __forceinline__ double boys_f0_table(double t, const double* __restrict__ table) {
+  if ((unsigned)__double2hiint(t) >= 0x40440000u) {  // 40 and above, NaN
+    return 0.88622692545275801365 * rsqrt_fast(t);
+  }
+  const double m = fma(t, 32.0, 6755399441055744.0);  // 1.5 2^52: rounds to an integer
+  const double d = fma(m - 6755399441055744.0, -0.03125, t);
+  const double2* c = reinterpret_cast<const double2*>(table + (size_t)__double2loint(m) * BOYS_STRIDE);
+  const double2 c01 = __ldg(c), c23 = __ldg(c + 1), c45 = __ldg(c + 2);
+  double r = __ldg(reinterpret_cast<const double*>(c + 3));
+  r = fma(r, d, c45.y);
+  r = fma(r, d, c45.x);
+  r = fma(r, d, c23.y);
+  r = fma(r, d, c23.x);
+  r = fma(r, d, c01.y);
+  return fma(r, d, c01.x);
+}

@@ -152,7 +152,7 @@ void fit_layout(int nao, int naux, bool jac, Arena* a, Sizer* z, FitWork* w) {
 #define TAKE(T_, ptr, count) \
   if (a) ptr = a->take<T_>(count); else z->take<T_>(count);
   TAKE(double, w->L, (size_t)naux * naux);
-  TAKE(double, w->pair_tab, 5 * (size_t)npair_of(nao));
+  TAKE(double, w->pair_tab, pair_tab_doubles(nao));
   TAKE(double, w->T, big);
   // the Jacobian also substitutes into the naux x naux identity
   TAKE(char, w->subst, std::max(forward_substitution_bytes(ld, naux), forward_substitution_bytes(naux, naux)));
@@ -202,7 +202,7 @@ extern "C" int df_fit_residual(const double* ao_xyz, const double* ao_exp, int n
   const long ld = B_ld(nao), npair = npair_of(nao);
   DF_REQUIRE(ld < (1L << 31), DF_ERR_ARG, "df_fit_residual: too many orbital pairs");
   // metric and its Cholesky factor (pivot check as in df_metric_chol)
-  DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, w.L, s));
+  DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, w.L, pair_tab_boys(w.pair_tab, nao), s));
   DF_TRY(cholesky_inplace(w.L, naux, w.status, w.maxdiag, 1e-14, w.subst, s));
   int h_status = -1;
   DF_CUDA(cudaMemcpyAsync(&h_status, w.status, sizeof(int), cudaMemcpyDeviceToHost, s));

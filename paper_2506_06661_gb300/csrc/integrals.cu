@@ -69,23 +69,78 @@ __global__ void int1e_kernel(const double* __restrict__ xyz, const double* __res
 // long-range operator erf(omega r)/r of the paper's LRDF split: the reduced exponent
 // rho = cd/(c+d) becomes rho f in the Boys argument and the prefactor gains sqrt(f),
 // f = omega^2 / (rho + omega^2).
-__global__ void int2c_kernel(const double* __restrict__ xyz, const double* __restrict__ ex, int naux, double omega,
-                             double* __restrict__ M) {
-  int c = blockIdx.y;
-  int d = blockIdx.x * blockDim.x + threadIdx.x;
-  if (d >= naux) return;
-  double ec = ex[c], ed = ex[d];
-  double dx = xyz[3 * c] - xyz[3 * d], dy = xyz[3 * c + 1] - xyz[3 * d + 1], dz = xyz[3 * c + 2] - xyz[3 * d + 2];
-  double r2 = dx * dx + dy * dy + dz * dz;
-  double pre = norm_s(ec) * norm_s(ed) * 2.0 * kPi * kPi * sqrt(kPi) / (ec * ed * sqrt(ec + ed));
-  double rho = ec * ed / (ec + ed);
-  if (omega > 0.0) {
-    const double f = omega * omega / (rho + omega * omega);
-    pre *= sqrt(f);
-    rho *= f;
+// One lane per column d and 16 rows c, whose factors N_c / c are formed once per CTA.
+constexpr int I2C_ROWS = 16;
+__global__ void __launch_bounds__(128) int2c_kernel(const double* __restrict__ xyz, const double* __restrict__ ex,
+                                                    int naux, double omega, const double* __restrict__ table,
+                                                    double* __restrict__ M) {
+  __shared__ double sc[I2C_ROWS][5];  // exponent, centre, N_c / c
+  const int c0 = blockIdx.y * I2C_ROWS, nc = min(I2C_ROWS, naux - c0);
+  if ((int)threadIdx.x < nc) {
+    const int c = c0 + threadIdx.x;
+    const double e = ex[c];
+    sc[threadIdx.x][0] = e;
+    sc[threadIdx.x][1] = xyz[3 * c];
+    sc[threadIdx.x][2] = xyz[3 * c + 1];
+    sc[threadIdx.x][3] = xyz[3 * c + 2];
+    sc[threadIdx.x][4] = norm_s(e) / e;
   }
-  M[(size_t)c * naux + d] = pre * boys_f0(rho * r2);
+  __syncthreads();
+  const int d = blockIdx.x * blockDim.x + threadIdx.x;
+  if (d >= naux) return;
+  const double ed = ex[d], x = xyz[3 * d], y = xyz[3 * d + 1], z = xyz[3 * d + 2];
+  const double nd = norm_s(ed) / ed, k = 2.0 * kPi * kPi * sqrt(kPi);
+  for (int i = 0; i < nc; ++i) {
+    const double ec = sc[i][0], dx = sc[i][1] - x, dy = sc[i][2] - y, dz = sc[i][3] - z;
+    const double r2 = dx * dx + dy * dy + dz * dz;
+    const double q = rsqrt_fast(ec + ed);
+    double pre = (sc[i][4] * nd) * (k * q), rho = ec * ed * (q * q);  // the same bits for (c, d) and (d, c)
+    if (omega > 0.0) {
+      const double f = omega * omega / (rho + omega * omega);
+      pre *= sqrt(f);
+      rho *= f;
+    }
+    M[DF_IX((size_t)(c0 + i) * naux + d, (size_t)naux * naux)] = pre * boys_f0_table(rho * r2, table);
+  }
 }
+
+// Row k of the Boys table: (-1)^j F_j(t) / j!, j = 0..6, at t = k / 32.  Below t = 10, F_6 from its
+// series e^-t sum_i (2t)^i / (13 15 .. (13 + 2i)) (all terms positive) and downward recursion
+// F_{j-1} = (2t F_j + e^-t) / (2j - 1); above, upward from F_0.
+__global__ void boys_table_kernel(double* __restrict__ table) {
+  const int k = blockIdx.x * blockDim.x + threadIdx.x;
+  if (k >= BOYS_ROWS) return;
+  const double t = k * 0.03125, et = exp(-t);
+  double F[7];
+  if (t < 10.0) {
+    double r = 1.0;
+#pragma unroll
+    for (int i = 47; i >= 1; --i) r = fma(2.0 * t * (1.0 / (13 + 2 * i)), r, 1.0);
+    F[6] = et * r * (1.0 / 13.0);
+#pragma unroll
+    for (int j = 6; j >= 1; --j) F[j - 1] = fma(2.0 * t, F[j], et) * (1.0 / (2 * j - 1));
+  } else {
+    F[0] = boys_f0(t);
+    const double h = 0.5 / t;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) F[j + 1] = ((2 * j + 1) * F[j] - et) * h;
+  }
+  double f = 1.0;
+#pragma unroll
+  for (int j = 0; j < 7; ++j) {
+    table[(size_t)k * BOYS_STRIDE + j] = F[j] * f;
+    f *= -1.0 / (j + 1);
+  }
+  table[(size_t)k * BOYS_STRIDE + 7] = 0.0;
+}
+
+static int launch_boys_table(double* table, cudaStream_t s) {
+  boys_table_kernel<<<(BOYS_ROWS + 31) / 32, 32, 0, s>>>(table);
+  DF_LAUNCHED("boys_table_kernel");
+  return DF_OK;
+}
+
+size_t boys_table_doubles() { return BOYS_TABLE; }
 
 // Per packed pair mn: product exponent p, centre P and K_mn = N_m N_n e^{-mu R^2} 2 pi^{5/2} / p.
 __global__ void pair_table_kernel(const double* __restrict__ xyz, const double* __restrict__ ex, long npair,
@@ -106,33 +161,48 @@ __global__ void pair_table_kernel(const double* __restrict__ xyz, const double* 
 }
 
 // (Q|mn) = K_mn N_Q / (c sqrt(p + c)) F0(p c / (p + c) |P - C|^2), written row Q of R
-// (row stride ld, padding columns [npair, ld) set to zero).  One lane per (Q, mn).
-__global__ void int3c_kernel(const double* __restrict__ pp, const double* __restrict__ px,
-                             const double* __restrict__ py, const double* __restrict__ pz,
-                             const double* __restrict__ pk, long npair, long ld,
-                             const double* __restrict__ axyz, const double* __restrict__ aex, int q0, double omega,
-                             double* __restrict__ R) {
-  int q = q0 + blockIdx.y;
-  long ij = (long)blockIdx.x * blockDim.x + threadIdx.x;
+// (row stride ld, padding columns [npair, ld) set to zero).  One lane per pair mn and 8 rows Q:
+// the pair is loaded once, and FP64 work is about 28 instructions per integral.
+constexpr int I3C_ROWS = 8;
+__global__ void __launch_bounds__(256) int3c_kernel(const double* __restrict__ pp, const double* __restrict__ px,
+                                                    const double* __restrict__ py, const double* __restrict__ pz,
+                                                    const double* __restrict__ pk, long npair, long ld,
+                                                    const double* __restrict__ axyz, const double* __restrict__ aex,
+                                                    int naux, int q0, double omega, const double* __restrict__ table,
+                                                    double* __restrict__ R) {
+  __shared__ double sq[I3C_ROWS][5];
+  q0 += blockIdx.y * I3C_ROWS;
+  const int nq = min(I3C_ROWS, naux - q0);
+  if ((int)threadIdx.x < nq) {
+    const int q = q0 + threadIdx.x;
+    const double c = aex[q];
+    sq[threadIdx.x][0] = c;
+    sq[threadIdx.x][1] = axyz[3 * q];
+    sq[threadIdx.x][2] = axyz[3 * q + 1];
+    sq[threadIdx.x][3] = axyz[3 * q + 2];
+    sq[threadIdx.x][4] = norm_s(c) / c;
+  }
+  __syncthreads();
+  const long ij = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (ij >= ld) return;
-  double* row = R + (size_t)q * ld;
+  double* row = R + (size_t)q0 * ld + ij;
   if (ij >= npair) {
-    row[ij] = 0.0;
+    for (int i = 0; i < nq; ++i) row[(size_t)i * ld] = 0.0;
     return;
   }
-  double c = aex[q];
-  double cx = axyz[3 * q], cy = axyz[3 * q + 1], cz = axyz[3 * q + 2];
-  double p = pp[ij];
-  double dx = px[ij] - cx, dy = py[ij] - cy, dz = pz[ij] - cz;
-  double inv = 1.0 / (p + c);
-  double rho = p * c * inv;
-  double pre = pk[ij] * norm_s(c) / c * sqrt(inv);
-  if (omega > 0.0) {  // long-range operator, as in int2c_kernel
-    const double f = omega * omega / (rho + omega * omega);
-    pre *= sqrt(f);
-    rho *= f;
+  const double p = pp[ij], x = px[ij], y = py[ij], z = pz[ij], k = pk[ij];
+  for (int i = 0; i < nq; ++i) {
+    const double c = sq[i][0], dx = x - sq[i][1], dy = y - sq[i][2], dz = z - sq[i][3];
+    const double v = rsqrt_fast(p + c);
+    double rho = p * c * (v * v), pre = k * sq[i][4] * v;
+    if (omega > 0.0) {  // long-range operator, as in int2c_kernel
+      const double f = omega * omega / (rho + omega * omega);
+      pre *= sqrt(f);
+      rho *= f;
+    }
+    row[DF_IX((size_t)i * ld, (size_t)(naux - q0) * ld)] =
+        pre * boys_f0_table(rho * (dx * dx + dy * dy + dz * dz), table);
   }
-  row[ij] = pre * boys_f0(rho * (dx * dx + dy * dy + dz * dz));
 }
 
 __global__ void enuc_kernel(const double* __restrict__ xyz, const double* __restrict__ z, int natm,
@@ -158,9 +228,11 @@ int launch_int1e(const double* ao_xyz, const double* ao_exp, int nao, const doub
   return DF_OK;
 }
 
-int launch_int2c(const double* xyz, const double* ex, int naux, double* M, cudaStream_t s, double omega) {
-  dim3 grid((naux + 127) / 128, naux);
-  int2c_kernel<<<grid, 128, 0, s>>>(xyz, ex, naux, omega, M);
+int launch_int2c(const double* xyz, const double* ex, int naux, double* M, double* table, cudaStream_t s,
+                 double omega) {
+  DF_TRY(launch_boys_table(table, s));
+  dim3 grid((naux + 127) / 128, (naux + I2C_ROWS - 1) / I2C_ROWS);
+  int2c_kernel<<<grid, 128, 0, s>>>(xyz, ex, naux, omega, table, M);
   DF_LAUNCHED("int2c_kernel");
   return DF_OK;
 }
@@ -183,9 +255,11 @@ int launch_int3c(const double* ao_xyz, const double* ao_exp, int nao, const doub
   double* pz = py + npair;
   double* pk = pz + npair;
   DF_TRY(launch_pair_table(ao_xyz, ao_exp, nao, pair_tab, s));
-  for (int q0 = 0; q0 < naux; q0 += 32768) {
-    dim3 grid((unsigned)((ld + 255) / 256), (unsigned)min(32768, naux - q0));
-    int3c_kernel<<<grid, 256, 0, s>>>(pp, px, py, pz, pk, npair, ld, aux_xyz, aux_exp, q0, omega, R);
+  double* table = pair_tab_boys(pair_tab, nao);
+  DF_TRY(launch_boys_table(table, s));
+  for (int q0 = 0; q0 < naux; q0 += 32768 * I3C_ROWS) {
+    dim3 grid((unsigned)((ld + 255) / 256), (unsigned)((min(32768 * I3C_ROWS, naux - q0) + I3C_ROWS - 1) / I3C_ROWS));
+    int3c_kernel<<<grid, 256, 0, s>>>(pp, px, py, pz, pk, npair, ld, aux_xyz, aux_exp, naux, q0, omega, table, R);
     DF_LAUNCHED("int3c_kernel");
   }
   return DF_OK;

@@ -559,8 +559,8 @@ extern "C" size_t df_B_bytes(int nao, int naux, int precision) {
 }
 
 extern "C" size_t df_build_B_work_bytes(int nao, int naux) {
-  if (nao <= 0 || naux <= 0) return nao > 0 ? align_up(sizeof(double) * 5 * (size_t)npair_of(nao), 256) : 0;
-  return align_up(sizeof(double) * 5 * (size_t)npair_of(nao), 256) + forward_substitution_bytes(B_ld(nao), naux);
+  if (nao <= 0 || naux <= 0) return nao > 0 ? align_up(sizeof(double) * pair_tab_doubles(nao), 256) : 0;
+  return align_up(sizeof(double) * pair_tab_doubles(nao), 256) + forward_substitution_bytes(B_ld(nao), naux);
 }
 
 extern "C" int df_build_B(const double* ao_xyz, const double* ao_exp, int nao, const double* aux_xyz,
@@ -576,7 +576,7 @@ extern "C" int df_build_B(const double* ao_xyz, const double* ao_exp, int nao, c
              "df_build_B: workspace of %zu bytes < %zu", work_bytes, df_build_B_work_bytes(nao, naux));
   DF_REQUIRE(precision == DF_FP64 || naux <= 65535, DF_ERR_ARG, "df_build_B: naux > 65535 in mixed mode");
   return build_B(ao_xyz, ao_exp, nao, aux_xyz, aux_exp, naux, L, precision, B, (double*)work,
-                 (char*)work + align_up(sizeof(double) * 5 * (size_t)npair_of(nao), 256), s);
+                 (char*)work + align_up(sizeof(double) * pair_tab_doubles(nao), 256), s);
 }
 
 extern "C" int df_B_get_packed(const void* B, int nao, int naux, int P, double* row, cudaStream_t s) {

@@ -12,10 +12,17 @@ namespace dfscf {
 int launch_int1e(const double* ao_xyz, const double* ao_exp, int nao, const double* nuc_xyz, const double* nuc_z,
                  int natm, double* S, double* T, double* V, cudaStream_t s);
 // Per packed orbital pair: exponent p, centre (x, y, z) and factor K_ab = N_a N_b e^{-mu R^2}
-// 2 pi^{5/2} / p, as five arrays of npair doubles in pair_tab.
+// 2 pi^{5/2} / p, as five arrays of npair doubles in pair_tab (pair_tab_doubles(nao) in launch_int3c).
 int launch_pair_table(const double* ao_xyz, const double* ao_exp, int nao, double* pair_tab, cudaStream_t s);
-// omega > 0: the long-range operator erf(omega r)/r instead of 1/r (LRDF)
-int launch_int2c(const double* xyz, const double* ex, int naux, double* M, cudaStream_t s, double omega = 0.0);
+// Doubles of a pair table with the Boys table behind it (pair_tab_boys; 16-byte aligned).
+size_t boys_table_doubles();
+inline size_t pair_tab_boys_offset(int nao) { return align_up(5 * (size_t)npair_of(nao), 2); }
+inline size_t pair_tab_doubles(int nao) { return pair_tab_boys_offset(nao) + boys_table_doubles(); }
+inline double* pair_tab_boys(double* pair_tab, int nao) { return pair_tab + pair_tab_boys_offset(nao); }
+// omega > 0: the long-range operator erf(omega r)/r instead of 1/r (LRDF); table: scratch of
+// boys_table_doubles()
+int launch_int2c(const double* xyz, const double* ex, int naux, double* M, double* table, cudaStream_t s,
+                 double omega = 0.0);
 int launch_int3c(const double* ao_xyz, const double* ao_exp, int nao, const double* aux_xyz, const double* aux_exp,
                  int naux, double* R, long ld, double* pair_tab, cudaStream_t s, double omega = 0.0);
 int launch_enuc(const double* xyz, const double* z, int natm, double* out, cudaStream_t s);

@@ -384,7 +384,7 @@ int forward_substitution(double* R, long ld, long ncol, const double* L, int nau
 using namespace dfscf;
 
 extern "C" size_t df_metric_chol_work_bytes(int naux) {
-  return naux > 0 ? 512 + cholesky_bytes(naux) : 512;
+  return 512 + sizeof(double) * align_up(boys_table_doubles(), 32) + (naux > 0 ? cholesky_bytes(naux) : 0);
 }
 
 extern "C" int df_metric_chol(const double* aux_xyz, const double* aux_exp, int naux, double* L, double* M_out,
@@ -396,9 +396,10 @@ extern "C" int df_metric_chol(const double* aux_xyz, const double* aux_exp, int 
   *bad_pivot = -1;
   int* d_status = (int*)work;
   double* d_maxdiag = (double*)((char*)work + 256);
-  DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, L, s));
+  DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, L, (double*)((char*)work + 512), s));
   if (M_out) DF_CUDA(cudaMemcpyAsync(M_out, L, sizeof(double) * naux * naux, cudaMemcpyDeviceToDevice, s));
-  DF_TRY(cholesky_inplace(L, naux, d_status, d_maxdiag, 1e-14, (char*)work + 512, s));
+  DF_TRY(cholesky_inplace(L, naux, d_status, d_maxdiag, 1e-14,
+                          (char*)work + 512 + sizeof(double) * align_up(boys_table_doubles(), 32), s));
   int h_status = -1;
   DF_CUDA(cudaMemcpyAsync(&h_status, d_status, sizeof(int), cudaMemcpyDeviceToHost, s));
   DF_CUDA(cudaStreamSynchronize(s));

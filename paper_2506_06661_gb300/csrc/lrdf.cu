@@ -173,7 +173,7 @@ extern "C" size_t df_lrdf_build_work_bytes(int nao, int naux) {
   z.take<double>((size_t)naux * naux);
   z.take<int>(1);
   z.take<double>(1);
-  z.take<double>(5 * (size_t)npair_of(nao));
+  z.take<double>(pair_tab_doubles(nao));
   z.take<char>(forward_substitution_bytes(B_ld(nao), naux));
   return z.used;
 }
@@ -193,9 +193,9 @@ extern "C" int df_lrdf_build(const double* ao_xyz, const double* ao_exp, int nao
   double* L = a.take<double>((size_t)naux * naux);
   int* status = a.take<int>(1);
   double* maxdiag = a.take<double>(1);
-  double* pair_tab = a.take<double>(5 * (size_t)npair_of(nao));
+  double* pair_tab = a.take<double>(pair_tab_doubles(nao));
   void* subst = a.take<char>(forward_substitution_bytes(B_ld(nao), naux));
-  DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, L, s, omega));
+  DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, L, pair_tab_boys(pair_tab, nao), s, omega));
   DF_TRY(cholesky_inplace(L, naux, status, maxdiag, 1e-14, subst, s));
   int h = -1;
   DF_CUDA(cudaMemcpyAsync(&h, status, sizeof(int), cudaMemcpyDeviceToHost, s));

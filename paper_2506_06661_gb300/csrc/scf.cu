@@ -623,7 +623,7 @@ static void scf_layout(int nao, int naux, int nocc, int precision, Arena* a, Siz
   w->guess_bytes = nao % 5 == 0 ? guess_density_work_bytes(nao / 5) : 0;
   w->guess_ws = nullptr;
   if (w->guess_bytes) TAKE(char, w->guess_ws, w->guess_bytes);
-  TAKE(double, w->pair_tab, 5 * (size_t)npair_of(nao));
+  TAKE(double, w->pair_tab, pair_tab_doubles(nao));
   TAKE(char, w->subst, forward_substitution_bytes(B_ld(nao), naux));
   TAKE(double, w->S, nn);
   TAKE(double, w->h, nn);
@@ -832,7 +832,7 @@ static int setup_launch(ScfMol& M) {
   axpy_kernel<<<blocks_for(nn), 256, 0, s>>>(W.h, W.V, nn, 1.0);
   DF_LAUNCHED("axpy_kernel");
   DF_TRY(launch_enuc(mol->xyz, mol->charges, mol->natm, W.enuc, s));
-  DF_TRY(launch_int2c(mol->aux_xyz, mol->aux_exp, naux, W.L, s));
+  DF_TRY(launch_int2c(mol->aux_xyz, mol->aux_exp, naux, W.L, pair_tab_boys(W.pair_tab, nao), s));
   DF_TRY(cholesky_inplace(W.L, naux, W.chol_status, W.maxdiag, 1e-14, W.subst, s));
   DF_TRY(build_B(mol->ao_xyz, mol->ao_exp, nao, mol->aux_xyz, mol->aux_exp, naux, W.L, M.opt.precision, W.B,
                  W.pair_tab, W.subst, s));
