@@ -17,6 +17,7 @@
 // Parameters are one float array: for each layer, W [out][in] then b [out].
 #include <cuda_bf16.h>
 
+#include <algorithm>
 #include <cstdint>
 #include <cstring>
 
@@ -40,8 +41,6 @@ __host__ __device__ constexpr size_t w_offset(int l) {
 __host__ __device__ constexpr size_t b_offset(int l) { return w_offset(l) + (size_t)layer_in(l) * layer_out(l); }
 constexpr size_t NPARAM = w_offset(NLAYER);
 
-__device__ __forceinline__ float to_f(float x) { return x; }
-__device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
 template <typename T> __device__ __forceinline__ T from_f(float x);
 template <> __device__ __forceinline__ float from_f<float>(float x) { return x; }
 template <> __device__ __forceinline__ __nv_bfloat16 from_f<__nv_bfloat16>(float x) { return __float2bfloat16_rn(x); }
@@ -53,30 +52,39 @@ __device__ __forceinline__ float rbf(float r, int k) {
 }
 
 // ---- SIMT GEMM with FP32 accumulation ---------------------------------------------------------
-// C[M][N] = alpha * op(A) op(B) + beta * C;  op(A)(m,k) = TA ? A[k*lda+m] : A[m*lda+k];
-// op(B)(k,n) = TB ? B[n*ldb+k] : B[k*ldb+n].  64x64 tiles, 256 lanes with 4x4 outputs.
-template <bool TA, bool TB, typename T>
-__global__ void __launch_bounds__(256) sgemm_kernel(int M, int N, int K, float alpha, const T* __restrict__ A, int lda,
-                                                    const T* __restrict__ B, int ldb, float beta, float* __restrict__ C,
-                                                    int ldc) {
+// op(A) op(B) over K;  op(A)(m,k) = TA ? A[k*lda+m] : A[m*lda+k];  op(B)(k,n) = TB ? B[n*ldb+k] :
+// B[k*ldb+n].  64x64 tiles, 256 lanes with 4x4 outputs.  What becomes of a product c:
+//   PARTIAL   C[z][m][n] = c of the K range z (kchunk terms): the weight gradients are 256 x 256
+//             or less with K = the batch, 16 tiles in all, so K is split over the other SMs
+//             (4096 pairs: 383 us a layer unsplit, 13 us with its reduction)
+//   BIAS_ACT  Z = c + b[n], H = SiLU(Z) (act) or Z
+//   SILU_GRAD C = c silu'(Z), silu'(z) = s (1 + z (1 - s)), s = sigmoid(z)
+enum Epilogue { PARTIAL, BIAS_ACT, SILU_GRAD };
+
+template <bool TA, bool TB, Epilogue E>
+__global__ void __launch_bounds__(256) sgemm_kernel(int M, int N, int K, const float* __restrict__ A, int lda,
+                                                    const float* __restrict__ B, int ldb, float* __restrict__ C,
+                                                    int kchunk, const float* __restrict__ bias, int act,
+                                                    const float* __restrict__ Zin, float* __restrict__ H) {
   __shared__ float As[16][65];
   __shared__ float Bs[16][65];
   int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   int m0 = blockIdx.y * 64, n0 = blockIdx.x * 64;
+  const int kb = E == PARTIAL ? (int)blockIdx.z * kchunk : 0, ke = E == PARTIAL ? min(K, kb + kchunk) : K;
   float acc[4][4] = {};
-  for (int k0 = 0; k0 < K; k0 += 16) {
+  for (int k0 = kb; k0 < ke; k0 += 16) {
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
       int idx = threadIdx.x + 256 * r;
       int mm, kk;
       if (TA) { kk = idx >> 6; mm = idx & 63; } else { mm = idx >> 4; kk = idx & 15; }
       int gm = m0 + mm, gk = k0 + kk;
-      As[kk][mm] = (gm < M && gk < K) ? to_f(TA ? A[(size_t)gk * lda + gm] : A[(size_t)gm * lda + gk]) : 0.f;
+      As[kk][mm] = (gm < M && gk < ke) ? (TA ? A[(size_t)gk * lda + gm] : A[(size_t)gm * lda + gk]) : 0.f;
       int nn;
       if (TB) { nn = idx >> 4; kk = idx & 15; } else { kk = idx >> 6; nn = idx & 63; }
       int gn = n0 + nn;
       gk = k0 + kk;
-      Bs[kk][nn] = (gn < N && gk < K) ? to_f(TB ? B[(size_t)gn * ldb + gk] : B[(size_t)gk * ldb + gn]) : 0.f;
+      Bs[kk][nn] = (gn < N && gk < ke) ? (TB ? B[(size_t)gn * ldb + gk] : B[(size_t)gk * ldb + gn]) : 0.f;
     }
     __syncthreads();
 #pragma unroll
@@ -101,33 +109,48 @@ __global__ void __launch_bounds__(256) sgemm_kernel(int M, int N, int K, float a
     for (int j = 0; j < 4; ++j) {
       int gn = n0 + tx + 16 * j;
       if (gn >= N) continue;
-      float* c = C + (size_t)gm * ldc + gn;
-      *c = beta == 0.f ? alpha * acc[i][j] : fmaf(alpha, acc[i][j], beta * *c);
+      const size_t at = (size_t)gm * N + gn;
+      if (E == PARTIAL) {
+        C[(size_t)blockIdx.z * M * N + at] = acc[i][j];
+      } else if (E == BIAS_ACT) {
+        const float z = acc[i][j] + bias[gn];
+        C[at] = z;
+        H[at] = act ? z / (1.f + __expf(-z)) : z;
+      } else {
+        const float z = Zin[at], s = 1.f / (1.f + __expf(-z));
+        C[at] = acc[i][j] * (s * (1.f + z * (1.f - s)));
+      }
     }
   }
 }
 
-template <bool TA, bool TB, typename T>
-static int sgemm(int M, int N, int K, float alpha, const T* A, int lda, const T* B, int ldb, float beta, float* C,
-                 int ldc, cudaStream_t s) {
+template <bool TA, bool TB, Epilogue E>
+static int sgemm(int M, int N, int K, const float* A, int lda, const float* B, int ldb, float* C, int splits,
+                 const float* bias, int act, const float* Zin, float* H, cudaStream_t s) {
   if (M <= 0 || N <= 0) return DF_OK;
-  dim3 grid((N + 63) / 64, (M + 63) / 64);
+  const int kchunk = ((K + splits - 1) / splits + 15) / 16 * 16;
+  dim3 grid((N + 63) / 64, (M + 63) / 64, splits);
   DF_REQUIRE(grid.y <= 65535, DF_ERR_ARG, "mlp: batch too large for one GEMM (%d rows)", M);
-  sgemm_kernel<TA, TB, T><<<grid, 256, 0, s>>>(M, N, K, alpha, A, lda, B, ldb, beta, C, ldc);
+  sgemm_kernel<TA, TB, E><<<grid, 256, 0, s>>>(M, N, K, A, lda, B, ldb, C, kchunk, bias, act, Zin, H);
   DF_LAUNCHED("sgemm_kernel");
   return DF_OK;
 }
 
-// Z += b (broadcast over rows), H = act(Z) in type T (SiLU when act != 0).
-template <typename T>
-__global__ void bias_act_kernel(float* __restrict__ Z, const float* __restrict__ b, int rows, int cols, int act,
-                                T* __restrict__ H) {
-  long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= (long)rows * cols) return;
-  float z = Z[i] + b[i % cols];
-  Z[i] = z;
-  float h = act ? z / (1.f + __expf(-z)) : z;
-  H[i] = from_f<T>(h);
+// K ranges of a weight gradient of fo x fi over n pairs: two CTAs per SM, 64 pairs or more each.
+constexpr int MAX_SPLITS = 64;
+__host__ __device__ constexpr int tiles64(int x) { return (x + 63) / 64; }
+static int grad_splits(int fo, int fi, int n) {
+  const int want = (2 * 152 + tiles64(fo) * tiles64(fi) - 1) / (tiles64(fo) * tiles64(fi));
+  return std::max(1, std::min(std::min(want, MAX_SPLITS), (n + 63) / 64));
+}
+
+// The splits in order: the same sum on every run.
+__global__ void sum_partials_kernel(const float* __restrict__ part, int splits, int count, float* __restrict__ out) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= count) return;
+  float s = 0.f;
+  for (int z = 0; z < splits; ++z) s += part[(size_t)z * count + i];
+  out[i] = s;
 }
 
 // G = 2 (out - Y) mask / (nvalid * 15); loss partial sums atomically into loss[0].
@@ -144,15 +167,6 @@ __global__ void mse_grad_kernel(const float* __restrict__ out, const float* __re
   }
   l = warp_sumf(l);
   if ((threadIdx.x & 31) == 0 && loss) atomicAdd(loss, l);
-}
-
-// dZ = dA * silu'(Z), silu'(z) = s (1 + z (1 - s)), s = sigmoid(z).
-__global__ void silu_backward_kernel(const float* __restrict__ Z, float* __restrict__ dA, long n) {
-  long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  float z = Z[i];
-  float s = 1.f / (1.f + __expf(-z));
-  dA[i] *= s * (1.f + z * (1.f - s));
 }
 
 // db[c] = sum_r G[r][c]
@@ -288,6 +302,7 @@ struct Work {
   float* G;           // gradient of the current layer's pre-activation
   float* dA;          // gradient w.r.t. the previous activation
   float* grad;        // parameter gradient (NPARAM)
+  float* part;        // K ranges of a weight gradient
   float* loss;
   __nv_bfloat16* Wp;  // BF16 weights of the tensor-core inference, zero-padded per layer
   int* err;           // bounded wait of the inference kernel gave up
@@ -303,6 +318,12 @@ static void layout(int n, Arena* a, Sizer* z, Work* w) {
   TAKE(float, w->G, (size_t)n * NHID);
   TAKE(float, w->dA, (size_t)n * NHID);
   TAKE(float, w->grad, NPARAM);
+  {
+    size_t most = 0;
+    for (int l = 0; l < NLAYER; ++l)
+      most = std::max(most, (size_t)grad_splits(layer_out(l), layer_in(l), n) * layer_out(l) * layer_in(l));
+    TAKE(float, w->part, most);
+  }
   TAKE(float, w->loss, 1);
   TAKE(__nv_bfloat16, w->Wp, (size_t)(2 * NHID * NHID + 128 * NHID + 16 * NHID));
   TAKE(int, w->err, 1);
@@ -326,9 +347,8 @@ static int forward_fp32(const float* P, const float* X, int n, Work& w, cudaStre
   const float* in = X;
   for (int l = 0; l < NLAYER; ++l) {
     int fi = layer_in(l), fo = layer_out(l);
-    DF_TRY((sgemm<false, true, float>(n, fo, fi, 1.f, in, fi, P + w_offset(l), fi, 0.f, w.Z[l], fo, s)));
-    bias_act_kernel<float><<<nb((long)n * fo), 256, 0, s>>>(w.Z[l], P + b_offset(l), n, fo, l < NLAYER - 1, w.H[l]);
-    DF_LAUNCHED("bias_act_kernel");
+    DF_TRY((sgemm<false, true, BIAS_ACT>(n, fo, fi, in, fi, P + w_offset(l), fi, w.Z[l], 1, P + b_offset(l),
+                                         l < NLAYER - 1, nullptr, w.H[l], s)));
     in = w.H[l];
   }
   return DF_OK;
@@ -537,14 +557,19 @@ static int loss_grad(const float* P, const float* X, const float* Y, const float
     int fi = layer_in(l), fo = layer_out(l);
     const float* Ain = l == 0 ? X : w.H[l - 1];
     // dW = G^T A_in  [fo][fi];  db = column sums of G
-    DF_TRY((sgemm<true, false, float>(fo, fi, n, 1.f, w.G, fo, Ain, fi, 0.f, w.grad + w_offset(l), fi, s)));
+    const int splits = grad_splits(fo, fi, n);
+    float* part = splits > 1 ? w.part : w.grad + w_offset(l);
+    DF_TRY((sgemm<true, false, PARTIAL>(fo, fi, n, w.G, fo, Ain, fi, part, splits, nullptr, 0, nullptr, nullptr, s)));
+    if (splits > 1) {
+      sum_partials_kernel<<<nb((long)fo * fi), 256, 0, s>>>(part, splits, fo * fi, w.grad + w_offset(l));
+      DF_LAUNCHED("sum_partials_kernel");
+    }
     column_sum_kernel<<<fo, 256, 0, s>>>(w.G, n, fo, w.grad + b_offset(l));
     DF_LAUNCHED("column_sum_kernel");
     if (l == 0) break;
     // dA = G W  [n][fi]; then G = dA * silu'(Z_{l-1})
-    DF_TRY((sgemm<false, false, float>(n, fi, fo, 1.f, w.G, fo, P + w_offset(l), fi, 0.f, w.dA, fi, s)));
-    silu_backward_kernel<<<nb((long)n * fi), 256, 0, s>>>(w.Z[l - 1], w.dA, (long)n * fi);
-    DF_LAUNCHED("silu_backward_kernel");
+    DF_TRY((sgemm<false, false, SILU_GRAD>(n, fi, fo, w.G, fo, P + w_offset(l), fi, w.dA, 1, nullptr, 0, w.Z[l - 1],
+                                           nullptr, s)));
     std::swap(w.G, w.dA);
   }
   return DF_OK;
