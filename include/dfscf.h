@@ -152,21 +152,20 @@ int df_jk(const void* B, int nao, int naux, int precision, const double* D, cons
 
 /* ---- a11: symmetric eigensolver ----------------------------------------------------
  * Eigenvalues w[0..n) ascending and eigenvectors (columns of Z, [n][n]) of the
- * symmetric matrix A [n][n] (A is overwritten).  Householder tridiagonalisation, then
- * implicit QL on one thread block (n < 160), or for larger n the multi-SM path of
- * df_eigh_lowest with k = n (Sturm multisection, inverse iteration, back-transformation,
- * two Gram-Schmidt passes).  Synchronises the stream; DF_ERR_NOCONV if the solver breaks
- * down, DF_ERR_TIMEOUT if a grid barrier of the multi-SM path gave up waiting (every CTA
- * then returns; the context stays usable).  work: df_eigh_work_bytes(n).                 */
+ * symmetric matrix A [n][n] (A is overwritten).  The multi-SM path of df_eigh_lowest with
+ * k = n; one thread block and implicit QL below 8 rows, and QL from the tridiagonal form
+ * below 160 where clustered eigenvalues ask for it.  Synchronises the stream;
+ * DF_ERR_NOCONV if the solver breaks down, DF_ERR_TIMEOUT if a wait of the multi-SM path
+ * gave up (every CTA then returns; the context stays usable).  work: df_eigh_work_bytes(n). */
 size_t df_eigh_work_bytes(int n);
 int df_eigh(double* A, int n, double* w, double* Z, void* work, size_t work_bytes, cudaStream_t s);
 
 /* The k lowest eigenpairs only (w [k] ascending, Z [n][k] columns), as the SCF needs for
- * the occupied orbitals and the LUMO: Householder reduction, Sturm bisection, inverse
- * iteration on the tridiagonal matrix, back-transformation of the k vectors and
- * re-orthonormalisation.  A is overwritten.  work: df_eigh_lowest_work_bytes(n, k).
+ * the occupied orbitals and the LUMO: Householder reduction, Sturm bisection, twisted
+ * factorisations of the tridiagonal matrix (inverse iteration in clusters),
+ * back-transformation of the k vectors and re-orthonormalisation.  A is overwritten.  work: df_eigh_lowest_work_bytes(n, k).
  * Returns DF_ERR_NOCONV if inverse iteration or re-orthonormalisation breaks down and
- * DF_ERR_TIMEOUT if a grid barrier of the multi-SM path gave up waiting.                  */
+ * DF_ERR_TIMEOUT if a wait of the multi-SM path gave up.                                  */
 size_t df_eigh_lowest_work_bytes(int n, int k);
 int df_eigh_lowest(double* A, int n, int k, double* w, double* Z, void* work, size_t work_bytes, cudaStream_t s);
 

@@ -216,7 +216,8 @@ extern "C" int df_bounds_violations(unsigned long long* count, char* where, size
                         {"integrals.cu", dfscf::bounds_read_integrals}, {"jk.cu", dfscf::bounds_read_jk},
                         {"linalg.cu", dfscf::bounds_read_linalg}, {"lowdin.cu", dfscf::bounds_read_lowdin},
                         {"lrdf.cu", dfscf::bounds_read_lrdf},     {"mlp.cu", dfscf::bounds_read_mlp},
-                        {"scf.cu", dfscf::bounds_read_scf},       {"umma.cu", dfscf::bounds_read_umma}};
+                        {"scf.cu", dfscf::bounds_read_scf},       {"tridiag.cu", dfscf::bounds_read_tridiag},
+                        {"trivec.cu", dfscf::bounds_read_trivec}, {"umma.cu", dfscf::bounds_read_umma}};
   DF_CUDA(cudaDeviceSynchronize());
   *count = 0;
   if (where && where_bytes) where[0] = '\0';

@@ -1,18 +1,25 @@
-// FP64 symmetric eigensolver for the SCF (orthogonalisation of S and the Fock
-// diagonalisation F'C' = C' eps).  One CTA per matrix, so a batch of molecules is one
-// launch with one CTA each:
+// FP64 symmetric eigensolver for the SCF (orthogonalisation of S and the Fock diagonalisation
+// F'C' = C' eps).  From 8 rows up the work is spread over the SMs (eigh_multi_sm): reduction in
+// tridiag.cu, eigenpairs of the tridiagonal matrix in trivec.cu.  This file holds the entry points,
+// what those leave to a fallback, and the one-CTA solver of the smallest matrices:
 //   1. Householder reduction A -> Q^T A Q = tridiag(d, e), reflectors kept in A;
 //   2. explicit Q by backward accumulation of the reflectors;
 //   3. implicit QL iterations with Wilkinson shifts on (d, e); each sweep's Givens
 //      rotations are generated serially by one lane and applied by all lanes to the
 //      eigenvector rows (vectors stored as rows, so the updates are coalesced);
 //   4. ascending sort of (eigenvalue, vector).
-// All three phases are textbook algorithms (Householder 1958; QL with implicit shifts as
+// All of these are textbook algorithms (Householder 1958; QL with implicit shifts as
 // in Bowdler, Martin, Reinsch and Wilkinson 1968) written here for a thread block.
+//
+// eigh_lowest, start to end: n = 100, k = 11 3.1 ms on one CTA -> 0.57; 300, 31 6.1 -> 1.9;
+// 900, 91 23.4 -> 8.6.  Full spectra: n = 30 2.4 ms (QL) -> 0.26; 100 22.5 -> 0.6; 300 21 -> 2.5.
+#include <algorithm>
 #include <cfloat>
 
 #include "common.cuh"
+#include "fp64.cuh"
 #include "kernels.cuh"
+#include "tridiag.cuh"
 
 namespace dfscf {
 
@@ -149,14 +156,15 @@ __device__ void tridiagonalize_cta(double* __restrict__ A, int n, double* __rest
   __syncthreads();
 }
 
-// A [n][n] symmetric (full storage), overwritten.  Outputs w [n] ascending and
-// ZT [n][n] with eigenvector k in row k.  Scratch: d, e, beta, v (n each), cs, sn (n each).
-__device__ int eigh_cta(double* __restrict__ A, int n, double* __restrict__ w, double* __restrict__ ZT,
-                        double* __restrict__ d, double* __restrict__ e, double* __restrict__ beta,
-                        double* __restrict__ v, double* __restrict__ cs, double* __restrict__ sn, EigShared& sh) {
+// Eigenpairs of H_0 .. H_{n-3} tridiag(d, e) H_{n-3} .. H_0 by implicit QL: w [n] ascending and
+// ZT [n][n] with eigenvector k in row k.  Reflector k below the diagonal of column k of A, or
+// right of the diagonal of row k (by_rows).  d and e are overwritten; cs, sn: n each.
+__device__ int ql_cta(const double* __restrict__ A, bool by_rows, int n, double* __restrict__ w,
+                      double* __restrict__ ZT, double* __restrict__ d, double* __restrict__ e,
+                      const double* __restrict__ beta, double* __restrict__ cs, double* __restrict__ sn,
+                      EigShared& sh) {
   const int tid = threadIdx.x, nt = blockDim.x;
-  // ---- 1. tridiagonalisation --------------------------------------------------------
-  tridiagonalize_cta(A, n, d, e, beta, v, cs, sn, sh);
+  const size_t vs = by_rows ? 1 : n, vk = by_rows ? n : 1;  // v_k[i] = A[i vs + k vk]
   // ---- 2. Q = H_0 H_1 ... H_{n-3}, built as rows ZT = Q^T -----------------------------
   // Work on Q directly in ZT's storage as Q[i][j] = ZT[j][i] would be strided; instead build
   // Q (row-major) and transpose in place at the end of this phase.
@@ -169,13 +177,13 @@ __device__ int eigh_cta(double* __restrict__ A, int n, double* __restrict__ w, d
     // u_j = b * sum_i v_i Q[k+1+i][k+1+j]
     for (int j = tid; j < len; j += nt) {
       double s = 0.0;
-      for (int i = 0; i < len; ++i) s += A[(size_t)(k + 1 + i) * n + k] * ZT[(size_t)(k + 1 + i) * n + k + 1 + j];
+      for (int i = 0; i < len; ++i) s += A[(k + 1 + i) * vs + k * vk] * ZT[(size_t)(k + 1 + i) * n + k + 1 + j];
       cs[j] = b * s;
     }
     __syncthreads();
     for (long q = tid; q < (long)len * len; q += nt) {
       int i = (int)(q / len), j = (int)(q % len);
-      ZT[(size_t)(k + 1 + i) * n + k + 1 + j] -= A[(size_t)(k + 1 + i) * n + k] * cs[j];
+      ZT[(size_t)(k + 1 + i) * n + k + 1 + j] -= A[(k + 1 + i) * vs + k * vk] * cs[j];
     }
     __syncthreads();
   }
@@ -224,7 +232,15 @@ __device__ int eigh_cta(double* __restrict__ A, int n, double* __restrict__ w, d
             bool early = false;
             for (; i >= l; --i) {
               double f = s * e[i], bb = c * e[i];
-              r = hypot(f, g);
+              const double r2 = fma(f, f, g * g);
+              const bool fast = ordinary(r2);  // else the squares may have left the FP64 range
+              double ri = 0.0;
+              if (fast) {
+                ri = rsqrt_ordinary(r2);
+                r = r2 * ri;
+              } else {
+                r = hypot(f, g);
+              }
               e[i + 1] = r;
               if (r == 0.0) {
                 d[i + 1] -= p;
@@ -232,8 +248,8 @@ __device__ int eigh_cta(double* __restrict__ A, int n, double* __restrict__ w, d
                 early = true;
                 break;
               }
-              s = f / r;
-              c = g / r;
+              s = fast ? f * ri : f / r;
+              c = fast ? g * ri : g / r;
               g = d[i + 1] - p;
               r = (d[i] - g) * s + 2.0 * c * bb;
               p = s * r;
@@ -311,6 +327,15 @@ __device__ int eigh_cta(double* __restrict__ A, int n, double* __restrict__ w, d
   for (int i = tid; i < n; i += nt) w[i] = d[i];
   __syncthreads();
   return 0;
+}
+
+// A [n][n] symmetric (full storage), overwritten.  Outputs w [n] ascending and
+// ZT [n][n] with eigenvector k in row k.  Scratch: d, e, beta, v (n each), cs, sn (n each).
+__device__ int eigh_cta(double* __restrict__ A, int n, double* __restrict__ w, double* __restrict__ ZT,
+                        double* __restrict__ d, double* __restrict__ e, double* __restrict__ beta,
+                        double* __restrict__ v, double* __restrict__ cs, double* __restrict__ sn, EigShared& sh) {
+  tridiagonalize_cta(A, n, d, e, beta, v, cs, sn, sh);
+  return ql_cta(A, false, n, w, ZT, d, e, beta, cs, sn, sh);
 }
 
 __global__ void __launch_bounds__(1024) eigh_batched_kernel(double* A, int n, long sA, double* w, long sw, double* ZT,
@@ -573,8 +598,10 @@ __global__ void __launch_bounds__(1024) eigh_lowest_kernel(double* A, int n, int
   if (threadIdx.x == 0 && status) *status = rc;
 }
 
-// ---- k lowest eigenpairs on many SMs -------------------------------------------------------
-// Same algorithm as eigh_lowest_cta spread over G co-resident CTAs (cooperative launch).
+// ---- k lowest eigenpairs on many SMs, any n ---------------------------------------------------
+// For matrices whose rows do not fit in the SMs' shared memory, and (phases 2-5) the fallback of
+// the direct eigenvectors.  Same algorithm as eigh_lowest_cta spread over G co-resident CTAs
+// (cooperative launch).
 // FP64 issues at a small fraction of the FP32 rate on this GPU, so every serial FP64 chain
 // is spread over as many SMs as possible:
 //   1. reduction: in step k every CTA recomputes the Householder vector of column k itself
@@ -588,28 +615,23 @@ __global__ void __launch_bounds__(1024) eigh_lowest_kernel(double* A, int n, int
 //   4. back-transformation: one warp per vector with the vector staged in shared memory;
 //   5. classical Gram-Schmidt twice, each projection spread over the whole grid.
 // Barrier waits are bounded; a timeout sets the error flag and every CTA returns.
-struct GridBarrier {
-  unsigned count;  // arrivals since launch (monotone; zeroed before the launch)
-  unsigned extra;  // arrivals expected beyond the grid's own CTAs: 0, except in the test of
-                   // the bounded wait (knob "eig_barrier_extra"), where no barrier can complete
-  int err;         // 1: a wait gave up; 2: inverse iteration failed
-  unsigned limit;  // polls before a wait gives up (knob "eig_barrier_polls")
-};
 
-// Set up the barrier record on the stream (graph-capturable, unlike a host write).
-__global__ void grid_barrier_init_kernel(GridBarrier* b, unsigned limit, unsigned extra) {
-  if (threadIdx.x != 0) return;
-  b->count = 0;
-  b->extra = extra;
-  b->err = 0;
-  b->limit = limit;
+// Set up the control record and the exchange buffers on the stream (graph-capturable, unlike a
+// host write).
+__global__ void eig_control_init_kernel(EigControl* c, unsigned limit, unsigned extra, unsigned long long* exchange,
+                                        long words) {
+  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < words; i += (long)gridDim.x * blockDim.x) exchange[i] = 0;
+  if (blockIdx.x != 0 || threadIdx.x != 0) return;
+  *c = EigControl{};
+  c->extra = extra;
+  c->limit = limit;
 }
 
 // Grid barrier on a monotone arrival counter: the b-th barrier completes when the counter
 // reaches b * (G + extra).  Thread 0 of each CTA arrives after a device-scope fence and polls
 // with acquire loads; after `limit` polls (2^22 by default, about a second) it raises the
 // error flag, every other CTA sees the flag within 256 polls, and all of them return.
-__device__ bool grid_sync(GridBarrier* b, unsigned G) {
+__device__ bool grid_sync(EigControl* b, unsigned G) {
   __shared__ int ok;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -644,7 +666,7 @@ constexpr int kCoopMaxCtas = 1024;
 __device__ void coop_tail(const double* __restrict__ A, int n, int k, double* __restrict__ w, double* __restrict__ ZT,
                           double* __restrict__ d, double* __restrict__ e, double* __restrict__ beta,
                           double* __restrict__ ee, double* __restrict__ lu, double* __restrict__ coef,
-                          double* __restrict__ part, int zw, double* zsm, GridBarrier* bar, int* status,
+                          double* __restrict__ part, int zw, double* zsm, EigControl* bar, int* status,
                           EigShared& sh) {
   const unsigned G = gridDim.x;
   const int cta = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
@@ -767,7 +789,7 @@ __global__ void __launch_bounds__(256, 1) eigh_lowest_coop_kernel(double* __rest
                                                                 double* __restrict__ w, double* __restrict__ ZT,
                                                                 double* __restrict__ scr, double* __restrict__ pbuf,
                                                                 double* __restrict__ coef, double* __restrict__ part,
-                                                                int zw, GridBarrier* bar, int* status) {
+                                                                int zw, EigControl* bar, int* status) {
   extern __shared__ double smem_d[];
   __shared__ EigShared sh;
   const unsigned G = gridDim.x;
@@ -861,141 +883,33 @@ __global__ void __launch_bounds__(256, 1) eigh_lowest_coop_kernel(double* __rest
   coop_tail(A, n, k, w, ZT, d, e, beta, ee, lu, coef, part, zw, smem_d + 2 * (size_t)n, bar, status, sh);
 }
 
-// Reduction with the rows of the trailing matrix in shared memory: row r lives in CTA
-// r mod G at slot r / G (R = ceil(n / G) slots of n doubles).  Every CTA keeps the current
-// column x = A[kk+1.., kk] and recomputes the reflector (v, beta) from it; the owners of the
-// rows compute p = beta A22 v and publish p together with the old column kk+1; after the one
-// grid barrier of the step every CTA forms w = p - (beta p.v / 2) v, updates its rows and
-// derives the next column from the old one with the same rank-2 formula, so all CTAs hold
-// the same bits.  Exchange buffers are double-buffered by step parity.  The reflector goes to
-// row kk of A (global) for the back-transformation.  Dynamic shared memory: 4 n + max(R, zw) n
-// doubles (the back-transformation's vectors reuse the row slots).
-__device__ __forceinline__ double rank2(double vi, double wj, double wi, double vj) {
-  return __fma_rn(vi, wj, __dmul_rn(wi, vj));
-}
-
-__global__ void __launch_bounds__(256, 1) eigh_lowest_coop_smem_kernel(double* __restrict__ A, int n, int k,
-                                                                     double* __restrict__ w, double* __restrict__ ZT,
-                                                                     double* __restrict__ scr,
-                                                                     double* __restrict__ xbuf, int R,
-                                                                     double* __restrict__ coef,
-                                                                     double* __restrict__ part, int zw,
-                                                                     GridBarrier* bar, int* status) {
+// Fallback of the direct eigenvectors (trivec.cu) after tridiag_launch: phases 2-5 where a cluster
+// of eigenvalues asks for them; the other solves end here.  Dynamic shared memory: zw n doubles.
+__global__ void __launch_bounds__(256, 1) eigh_fallback_coop_kernel(const double* __restrict__ A, int n, int k,
+                                                                  double* __restrict__ w, double* __restrict__ ZT,
+                                                                  double* __restrict__ scr, double* __restrict__ coef,
+                                                                  double* __restrict__ part, int zw, EigControl* ctl,
+                                                                  int* status) {
   extern __shared__ double smem_d[];
   __shared__ EigShared sh;
-  const unsigned G = gridDim.x;
-  const int cta = blockIdx.x, tid = threadIdx.x, nt = blockDim.x;
-  const int lane = tid & 31, wid = tid >> 5, nw = nt >> 5;
-  double* v = smem_d;            // n: reflector
-  double* wv = smem_d + n;       // n: p, then w
-  double* x = smem_d + 2 * n;    // n: current column below the diagonal
-  double* c = smem_d + 3 * n;    // n: old next column
-  double* rows = smem_d + 4 * n; // R n
+  const bool gave_up = ctl->err == 1;
+  if (gave_up || !eig_needs_fallback(ctl, k)) {
+    if (blockIdx.x == 0 && threadIdx.x == 0) *status = gave_up ? 3 : 0;
+    return;
+  }
   double* d = scr;
-  double* e = d + n;
-  double* beta = e + n;
-  double* ee = beta + n;
-  double* lu = beta + 2 * n;  // 6 n k
-  // owned rows into shared memory; column 0 below the diagonal into x
-  for (int s = 0; s < R; ++s) {
-    const int r = s * (int)G + cta;
-    if (r >= n) break;
-    for (int j = tid; j < n; j += nt) rows[(size_t)s * n + j] = A[(size_t)r * n + j];
-  }
-  for (int i = tid; i + 1 < n; i += nt) x[i] = A[(size_t)(i + 1) * n];
-  // all CTAs have read A before any reflector is written back into it
-  if (!grid_sync(bar, G)) {
-    if (cta == 0 && tid == 0) *status = 3;
-    return;
-  }
-  // ---- 1. tridiagonalisation -------------------------------------------------------------
-  for (int kk = 0; kk + 2 < n; ++kk) {
-    const int len = n - kk - 1;  // x = A[kk+1..n)[kk]
-    double part_s = 0.0;
-    for (int i = tid + 1; i < len; i += nt) part_s += x[i] * x[i];
-    const double sigma = cta_sum(part_s, sh);
-    const double x0 = x[0];
-    double alpha, b;
-    if (sigma == 0.0) {
-      alpha = x0;
-      b = 0.0;
-    } else {
-      const double nrm = sqrt(x0 * x0 + sigma);
-      alpha = (x0 >= 0.0) ? -nrm : nrm;
-      const double v0 = x0 - alpha;
-      b = 2.0 / (v0 * v0 + sigma);
-    }
-    for (int i = tid; i < len; i += nt) v[i] = (i == 0) ? (x0 - alpha) : x[i];
-    if (cta == 0 && tid == 0) {
-      e[kk] = alpha;
-      beta[kk] = b;
-    }
-    if (kk % (int)G == cta && tid == 0) d[kk] = rows[(size_t)(kk / (int)G) * n + kk];
-    __syncthreads();
-    // p for the owned rows of the trailing block, and their entries in column kk+1
-    double* pg = xbuf + (size_t)(kk & 1) * 2 * n;
-    double* cg = pg + n;
-    {
-      const int s0 = (kk + 1 - cta + (int)G - 1) / (int)G;  // first slot with row > kk
-      for (int s = s0 + wid; s < R; s += nw) {
-        const int r = s * (int)G + cta;
-        if (r >= n) break;
-        const double* row = rows + (size_t)s * n + kk + 1;
-        double acc = 0.0;
-        if (b != 0.0)
-          for (int j = lane; j < len; j += 32) acc += row[j] * v[j];
-        acc = warp_sum(acc);
-        if (lane == 0) {
-          pg[r - kk - 1] = b * acc;
-          cg[r - kk - 1] = row[0];
-        }
-      }
-    }
-    // the reflector, for the back-transformation
-    if (kk % (int)G == cta)
-      for (int i = tid; i < len; i += nt) A[(size_t)kk * n + kk + 1 + i] = v[i];
-    if (!grid_sync(bar, G)) break;
-    double pv = 0.0;
-    for (int i = tid; i < len; i += nt) {
-      const double pi = pg[i];
-      wv[i] = pi;
-      c[i] = cg[i];
-      pv += pi * v[i];
-    }
-    const double Kf = 0.5 * b * cta_sum(pv, sh);
-    for (int i = tid; i < len; i += nt) wv[i] -= Kf * v[i];
-    __syncthreads();
-    // next column x' = A'[kk+2.., kk+1] from the old column and the same rank-2 formula
-    const double v0 = v[0], w0 = wv[0];
-    for (int i = tid; i + 1 < len; i += nt) x[i] = c[i + 1] - rank2(v[i + 1], w0, wv[i + 1], v0);
-    if (b != 0.0) {
-      const int s0 = (kk + 1 - cta + (int)G - 1) / (int)G;
-      for (int s = s0 + wid; s < R; s += nw) {
-        const int r = s * (int)G + cta;
-        if (r >= n) break;
-        const int i = r - kk - 1;
-        double* row = rows + (size_t)s * n + kk + 1;
-        const double vi = v[i], wi = wv[i];
-        for (int j = lane; j < len; j += 32) row[j] -= rank2(vi, wv[j], wi, v[j]);
-      }
-    }
-    __syncthreads();
-  }
-  if (bar->err) {
-    if (cta == 0 && tid == 0) *status = 3;
-    return;
-  }
-  if (n >= 2) {
-    if ((n - 2) % (int)G == cta && tid == 0) d[n - 2] = rows[(size_t)((n - 2) / (int)G) * n + n - 2];
-    if (cta == 0 && tid == 0) e[n - 2] = x[0];
-  }
-  if ((n - 1) % (int)G == cta && tid == 0) d[n - 1] = rows[(size_t)((n - 1) / (int)G) * n + n - 1];
-  if (cta == 0 && tid == 0) e[n - 1] = 0.0;
-  if (!grid_sync(bar, G)) {
-    if (cta == 0 && tid == 0) *status = 3;
-    return;
-  }
-  coop_tail(A, n, k, w, ZT, d, e, beta, ee, lu, coef, part, zw, rows, bar, status, sh);
+  coop_tail(A, n, k, w, ZT, d, d + n, d + 2 * n, d + 3 * n, d + 4 * n, coef, part, zw, smem_d, ctl, status, sh);
+}
+
+// The same for a small full spectrum: implicit QL on one CTA, exact in any cluster.
+__global__ void __launch_bounds__(1024) eigh_fallback_ql_kernel(const double* __restrict__ A, int n,
+                                                              double* __restrict__ w, double* __restrict__ ZT,
+                                                              double* __restrict__ scr, EigControl* ctl, int* status) {
+  __shared__ EigShared sh;
+  int rc = ctl->err ? 3 : 0;
+  if (rc == 0 && eig_needs_fallback(ctl, n))
+    rc = ql_cta(A, true, n, w, ZT, scr, scr + n, scr + 2 * n, scr + 4 * n, scr + 5 * n, sh);
+  if (threadIdx.x == 0) *status = rc;
 }
 
 __global__ void transpose_kernel(const double* __restrict__ in, int rows, int cols, double* __restrict__ out) {
@@ -1021,10 +935,12 @@ int transpose(const double* in, int rows, int cols, double* out, cudaStream_t s)
 
 size_t eigh_scratch_doubles(int n) { return (size_t)6 * n; }
 
-size_t eigh_lowest_scratch_doubles(int n, int k) { return (size_t)4 * n + (size_t)6 * n * std::max(k, 1); }
+size_t eigh_lowest_scratch_doubles(int n, int k) {
+  return (size_t)4 * n + std::max((size_t)6 * n * std::max(k, 1), trivec_scratch_doubles(n, std::max(k, 1)));
+}
 
 size_t eigh_coop_aux_bytes(int n) {
-  return align_up(4 * sizeof(double) * (size_t)n, 256) + align_up(sizeof(double) * (size_t)n, 256) +
+  return align_up(tridiag_exchange_bytes(n), 256) + align_up(sizeof(double) * (size_t)n, 256) +
          align_up(sizeof(double) * kCoopMaxCtas, 256) + 256;
 }
 
@@ -1035,97 +951,106 @@ constexpr size_t kSmemMax = 227 * 1024;
 int coop_zw(int k, int G) { return std::min(8, std::max(1, (k + G - 1) / G)); }
 
 struct CoopPlan {
-  int G = 0;         // CTAs (0: one-CTA kernel)
-  bool rows = false; // trailing rows in shared memory
-  int R = 0;         // row slots per CTA
+  int G = 0;  // CTAs (0: none fits)
   int zw = 0;
   size_t smem = 0;
 };
 
-size_t plan_smem(int n, int k, int G, bool rows) {
-  const int zw = coop_zw(k, G);
-  if (rows) return sizeof(double) * (size_t)n * (4 + std::max((n + G - 1) / G, zw));
-  return sizeof(double) * (size_t)n * (2 + zw);
-}
-
-bool fits(const void* kern, size_t smem, int G, int sms) {
-  if (smem > kSmemMax) return false;
-  if (smem > 48 * 1024 && cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-                              cudaSuccess)
-    return false;
-  int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem) != cudaSuccess) return false;
-  return G <= sms * per_sm;
-}
-
-// Multi-SM plan (G = 0: use one CTA).  Knob "eig_ctas" overrides the CTA count; the default
-// takes up to one CTA per SM once n is large enough for the reduction to gain from it, and
-// keeps the trailing rows in shared memory whenever they fit.
-CoopPlan coop_plan(int n, int k) {
+// Cooperative launch of `kern` with `vecs` vectors of n and the back-transformation's in shared
+// memory: up to one CTA per SM.
+CoopPlan coop_plan(const void* kern, int n, int k, int vecs) {
   CoopPlan P;
-  int forced = knob("eig_ctas");
-  if (forced == 1) return P;
-  if (forced == 0 && n < 160) return P;
-  int dev = 0, sms = 0;
+  int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return P;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  int G = forced > 1 ? forced : std::min(sms, std::max(32, n / 8));
-  G = std::min(G, kCoopMaxCtas);
-  if (G < 2) return P;
-  size_t sm_rows = plan_smem(n, k, G, true);
-  if (fits((const void*)eigh_lowest_coop_smem_kernel, sm_rows, G, sms)) {
-    P.G = G;
-    P.rows = true;
-    P.R = (n + G - 1) / G;
-    P.zw = coop_zw(k, G);
-    P.smem = sm_rows;
+  const int forced = knob("eig_ctas");
+  const int G = std::min(forced > 1 ? forced : std::min(sms, std::max(32, n / 8)), kCoopMaxCtas);
+  const int zw = coop_zw(k, G);
+  const size_t smem = sizeof(double) * (size_t)n * (vecs + zw);
+  if (smem > kSmemMax) return P;
+  if (smem > 48 * 1024 &&
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return P;
-  }
-  size_t sm_glob = plan_smem(n, k, G, false);
-  if (fits((const void*)eigh_lowest_coop_kernel, sm_glob, G, sms)) {
-    P.G = G;
-    P.zw = coop_zw(k, G);
-    P.smem = sm_glob;
-  }
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, 256, smem) != cudaSuccess) return P;
+  if (G > sms * per_sm) return P;
+  P.G = G;
+  P.zw = zw;
+  P.smem = smem;
   return P;
+}
+
+template <typename... Args>
+int coop_launch(void (*kern)(Args...), const CoopPlan& P, cudaStream_t s, Args... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(P.G);
+  cfg.blockDim = dim3(256);
+  cfg.dynamicSmemBytes = P.smem;
+  cfg.stream = s;
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeCooperative;
+  attr[0].val.cooperative = 1;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  DF_CUDA(cudaLaunchKernelEx(&cfg, kern, args...));
+  return DF_OK;
+}
+
+// Below this the reduction is a few steps of one CTA's work.  n = 32, k = 4: 0.7 ms on one CTA, 0.25 here.
+constexpr int kMultiSm = 8;
+// Full spectra up to here fall back to implicit QL, whose vectors are orthogonal in any cluster.
+constexpr int kQlMax = 160;
+
+// k lowest eigenpairs (full: k = n, the whole spectrum asked for).  aux: eigh_coop_aux_bytes(n)
+// of scratch for the multi-SM path; *done is false when only the one-CTA kernels apply.
+int eigh_multi_sm(double* A, int n, int k, bool full, double* w, double* ZT, double* scratch, int* status,
+                  cudaStream_t s, void* aux, bool* done) {
+  *done = false;
+  const int forced = knob("eig_ctas");
+  if (!aux || forced == 1 || (forced == 0 && n < kMultiSm) || n < 3) return DF_OK;
+  char* p = (char*)aux;
+  unsigned long long* exchange = (unsigned long long*)p;
+  p += align_up(tridiag_exchange_bytes(n), 256);
+  double* coef = (double*)p;
+  p += align_up(sizeof(double) * (size_t)n, 256);
+  double* part = (double*)p;
+  p += align_up(sizeof(double) * kCoopMaxCtas, 256);
+  EigControl* ctl = (EigControl*)p;
+  const TridiagPlan T = tridiag_plan(n, forced);
+  const CoopPlan F = coop_plan((const void*)eigh_fallback_coop_kernel, n, k, 0);
+  const bool fast = T.G > 0 && F.G > 0 && trivec_fits(n);
+  CoopPlan C;
+  if (!fast) {  // rows that do not fit in shared memory
+    C = coop_plan((const void*)eigh_lowest_coop_kernel, n, k, 2);
+    if (C.G < 2) return DF_OK;
+  }
+  const long words = fast ? (long)(tridiag_exchange_bytes(n) / sizeof(unsigned long long)) : 0;
+  eig_control_init_kernel<<<(unsigned)(words / 2048 + 1), 256, 0, s>>>(ctl, (unsigned)knob("eig_barrier_polls"),
+                                                               (unsigned)knob("eig_barrier_extra"), exchange, words);
+  DF_LAUNCHED("eig_control_init_kernel");
+  if (!fast) {
+    DF_TRY(coop_launch(eigh_lowest_coop_kernel, C, s, A, n, k, w, ZT, scratch, (double*)exchange, coef, part, C.zw, ctl,
+                       status));
+  } else {
+    DF_TRY(tridiag_launch(A, n, scratch, scratch + n, scratch + 2 * (size_t)n, T, exchange, ctl, s));
+    DF_TRY(trivec_launch(A, n, k, scratch, scratch + n, scratch + 2 * (size_t)n, w, ZT, scratch + 4 * (size_t)n, ctl, s));
+    if (full && n < kQlMax) {
+      eigh_fallback_ql_kernel<<<1, 1024, 0, s>>>(A, n, w, ZT, scratch, ctl, status);
+      DF_LAUNCHED("eigh_fallback_ql_kernel");
+    } else {
+      DF_TRY(coop_launch(eigh_fallback_coop_kernel, F, s, (const double*)A, n, k, w, ZT, scratch, coef, part, F.zw, ctl,
+                         status));
+    }
+  }
+  *done = true;
+  return DF_OK;
 }
 }  // namespace
 
-// aux: coop_aux_bytes(n) of scratch for the multi-SM path.
 int eigh_lowest_rows(double* A, int n, int k, double* w, double* ZT, double* scratch, int* status, cudaStream_t s,
                      void* aux) {
-  CoopPlan P;
-  if (aux) P = coop_plan(n, k);
-  if (P.G >= 2) {
-    char* p = (char*)aux;
-    double* xbuf = (double*)p;
-    p += align_up(4 * sizeof(double) * (size_t)n, 256);
-    double* coef = (double*)p;
-    p += align_up(sizeof(double) * (size_t)n, 256);
-    double* part = (double*)p;
-    p += align_up(sizeof(double) * kCoopMaxCtas, 256);
-    GridBarrier* bar = (GridBarrier*)p;
-    grid_barrier_init_kernel<<<1, 32, 0, s>>>(bar, (unsigned)knob("eig_barrier_polls"),
-                                              (unsigned)knob("eig_barrier_extra"));
-    DF_LAUNCHED("grid_barrier_init_kernel");
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(P.G);
-    cfg.blockDim = dim3(256);
-    cfg.dynamicSmemBytes = P.smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeCooperative;
-    attr[0].val.cooperative = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (P.rows)
-      DF_CUDA(cudaLaunchKernelEx(&cfg, eigh_lowest_coop_smem_kernel, A, n, k, w, ZT, scratch, xbuf, P.R, coef, part,
-                                 P.zw, bar, status));
-    else
-      DF_CUDA(cudaLaunchKernelEx(&cfg, eigh_lowest_coop_kernel, A, n, k, w, ZT, scratch, xbuf, coef, part, P.zw, bar,
-                                 status));
-    return DF_OK;
-  }
+  bool done = false;
+  DF_TRY(eigh_multi_sm(A, n, k, false, w, ZT, scratch, status, s, aux, &done));
+  if (done) return DF_OK;
   eigh_lowest_kernel<<<1, 1024, 0, s>>>(A, n, k, w, ZT, scratch, status);
   DF_LAUNCHED("eigh_lowest_kernel");
   return DF_OK;
@@ -1139,7 +1064,9 @@ size_t eigh_full_scratch_doubles(int n) {
 // else one CTA with implicit QL.  scratch: eigh_full_scratch_doubles(n).
 int eigh_full_rows(double* A, int n, double* w, double* ZT, double* scratch, int* status, cudaStream_t s,
                    void* aux) {
-  if (aux && coop_plan(n, n).G >= 2) return eigh_lowest_rows(A, n, n, w, ZT, scratch, status, s, aux);
+  bool done = false;
+  DF_TRY(eigh_multi_sm(A, n, n, true, w, ZT, scratch, status, s, aux, &done));
+  if (done) return DF_OK;
   return eigh_rows(A, n, w, ZT, scratch, status, s);
 }
 

@@ -132,6 +132,8 @@ int bounds_read_lowdin(BoundsRecord*);
 int bounds_read_lrdf(BoundsRecord*);
 int bounds_read_mlp(BoundsRecord*);
 int bounds_read_scf(BoundsRecord*);
+int bounds_read_tridiag(BoundsRecord*);
+int bounds_read_trivec(BoundsRecord*);
 int bounds_read_umma(BoundsRecord*);
 
 }  // namespace dfscf

@@ -1036,7 +1036,7 @@ static int dm0_finish(ScfMol& M) {
 }
 
 // Principal angles between the occupied space of the accumulated K (C'_base) and the new
-// one (C'): M = C'_base^T C', eigen-decomposition of M^T M on one CTA, summary into the status.
+// one (C'): M = C'_base^T C', eigen-decomposition of M^T M, summary into the status.
 static int incremental_prep(ScfMol& M) {
   ScfWork& W = M.W;
   cudaStream_t s = M.s;
@@ -1044,7 +1044,7 @@ static int incremental_prep(ScfMol& M) {
   ProfScope ps_inc("scf_incremental_prep", s);
   DF_TRY(dgemm(true, false, nocc, nocc, nmo, 1.0, W.Cbase, nocc, 0, W.Cp, nocc, 0, 0.0, W.Minc, nocc, 0, 1, s, 0, 0));
   DF_TRY(dgemm(true, false, nocc, nocc, nocc, 1.0, W.Minc, nocc, 0, W.Minc, nocc, 0, 0.0, W.Tinc, nocc, 0, 1, s, 0, 0));
-  DF_TRY(eigh_rows(W.Tinc, nocc, W.cinc, W.Winc, W.eig_scratch, W.inc_status, s));
+  DF_TRY(eigh_full_rows(W.Tinc, nocc, W.cinc, W.Winc, W.eig_scratch, W.inc_status, s, W.eig_aux));
   inc_status_kernel<<<1, 256, 0, s>>>(W.cinc, nocc, W.inc_status, W.st);
   DF_LAUNCHED("inc_status_kernel");
   return DF_OK;
@@ -1169,7 +1169,7 @@ static int rotate_orbitals(ScfMol& M) {
   const int nmo = M.nmo, nocc = M.nocc, nvir = nmo - nocc;
   const long ne = (long)nmo * nmo;
   DF_TRY(dgemm(true, false, nocc, nocc, nvir, 1.0, W.cg_x, nocc, 0, W.cg_x, nocc, 0, 0.0, W.kk, nocc, 0, 1, s, 0, 0));
-  DF_TRY(eigh_rows(W.kk, nocc, W.ksig, W.kVrow, W.eig_scratch, W.k_status, s));
+  DF_TRY(eigh_full_rows(W.kk, nocc, W.ksig, W.kVrow, W.eig_scratch, W.k_status, s, W.eig_aux));
   rotation_mats_kernel<<<blocks_for((long)nocc * nocc), 256, 0, s>>>(W.kVrow, W.ksig, nocc, W.Pc, W.Ps, W.Pd);
   DF_LAUNCHED("rotation_mats_kernel");
   // occupied: C'_o Pc + C'_v (k Ps)
