@@ -94,12 +94,83 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int M, int N, int K, double 
   }
 }
 
+// The same product in tiles of 16 x 8, one output per thread.  FP64 issues one warp instruction per
+// 64 clocks on each partition of an SM, so four warps fill it and a tile's time is its share of
+// the multiplications: 300^3 in 64 x 64 tiles put them on 25 of 152 SMs, 309 us; in 16 x 8 tiles
+// 722 CTAs spread over all of them (48 us are the FP64 units' own); in an SCF with 300 functions the
+// products took 309 and 236 us, now 24 and 24, with 100 functions 125, now 8.  The tiles of the
+// next 32 of K are on their way while this one's are multiplied.
+constexpr int GS_M = 16, GS_N = 8, GS_K = 32;
+template <bool TA, bool TB>
+__global__ void __launch_bounds__(128) dgemm_small_kernel(int M, int N, int K, double alpha, const double* __restrict__ A,
+                                                          long lda, long sA, const double* __restrict__ B, long ldb,
+                                                          long sB, double beta, double* __restrict__ C, long ldc,
+                                                          long sC) {
+  __shared__ double As[GS_K][GS_M + 1], Bs[GS_K][GS_N + 1];
+  A += (size_t)blockIdx.z * sA;
+  B += (size_t)blockIdx.z * sB;
+  C += (size_t)blockIdx.z * sC;
+  const int tid = threadIdx.x, tx = tid % GS_N, ty = tid / GS_N;
+  const int m0 = blockIdx.y * GS_M, n0 = blockIdx.x * GS_N;
+  double a[4], b[2], acc = 0.0;
+  auto fetch = [&](int k0) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int q = tid + 128 * r, mm = TA ? q % GS_M : q / GS_K, kk = TA ? q / GS_M : q % GS_K;
+      const long gm = m0 + mm, gk = k0 + kk;
+      a[r] = gm < M && gk < K ? (TA ? A[gk * lda + gm] : A[gm * lda + gk]) : 0.0;
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int q = tid + 128 * r, nn = TB ? q / GS_K : q % GS_N, kk = TB ? q % GS_K : q / GS_N;
+      const long gn = n0 + nn, gk = k0 + kk;
+      b[r] = gn < N && gk < K ? (TB ? B[gn * ldb + gk] : B[gk * ldb + gn]) : 0.0;
+    }
+  };
+  fetch(0);
+  for (int k0 = 0; k0 < K; k0 += GS_K) {
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      const int q = tid + 128 * r;
+      As[TA ? q / GS_M : q % GS_K][TA ? q % GS_M : q / GS_K] = a[r];
+    }
+#pragma unroll
+    for (int r = 0; r < 2; ++r) {
+      const int q = tid + 128 * r;
+      Bs[TB ? q % GS_K : q / GS_N][TB ? q / GS_K : q % GS_N] = b[r];
+    }
+    __syncthreads();
+    if (k0 + GS_K < K) fetch(k0 + GS_K);
+    if (k0 + GS_K <= K) {
+#pragma unroll
+      for (int kk = 0; kk < GS_K; ++kk) acc = fma(As[kk][ty], Bs[kk][tx], acc);
+    } else {
+      for (int kk = 0; kk < K - k0; ++kk) acc = fma(As[kk][ty], Bs[kk][tx], acc);
+    }
+  }
+  const int gm = m0 + ty, gn = n0 + tx;
+  if (gm >= M || gn >= N) return;
+  double* c = C + (size_t)gm * ldc + gn;
+  *c = beta == 0.0 ? alpha * acc : fma(alpha, acc, beta * *c);
+}
+
 int dgemm(bool ta, bool tb, int M, int N, int K, double alpha, const double* A, long lda, long sA, const double* B,
           long ldb, long sB, double beta, double* C, long ldc, long sC, int batch, cudaStream_t s, long kchunk,
           int lower_only) {
   if (M <= 0 || N <= 0 || batch <= 0) return DF_OK;
   dim3 grid((N + GB_N - 1) / GB_N, (M + GB_M - 1) / GB_M, batch);
   DF_REQUIRE(grid.y <= 65535 && grid.z <= 65535, DF_ERR_ARG, "dgemm: grid too large (M=%d batch=%d)", M, batch);
+  // Few large tiles leave SMs idle; up to about four per SM the small ones spread better, and their
+  // reads (3 bytes per multiplication from L2) are still far below what L2 gives.
+  const dim3 small((N + GS_N - 1) / GS_N, (M + GS_M - 1) / GS_M, batch);
+  if (kchunk == 0 && !lower_only && (long)grid.x * grid.y * grid.z <= 4 * 152 && small.y <= 65535) {
+    auto k = !ta && !tb ? dgemm_small_kernel<false, false>
+                        : !ta ? dgemm_small_kernel<false, true> : !tb ? dgemm_small_kernel<true, false> : dgemm_small_kernel<true, true>;
+    k<<<small, 128, 0, s>>>(M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC);
+    DF_LAUNCHED("dgemm_small_kernel");
+    return DF_OK;
+  }
   if (!ta && !tb)
     dgemm_kernel<false, false><<<grid, 256, 0, s>>>(M, N, K, alpha, A, lda, sA, B, ldb, sB, beta, C, ldc, sC, kchunk, lower_only);
   else if (!ta && tb)
