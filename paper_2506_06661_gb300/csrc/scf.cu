@@ -2363,9 +2363,9 @@ extern "C" int scf_run_batch(const df_molecule* mols, int nmol, const scf_opts* 
       progressed = true;
       rc = advance(k);
     }
-    if (rc == DF_OK && running == 0 && next < nmol) {
-      // nothing runs and the next molecule still does not fit: cannot happen while the
-      // workspace holds the largest molecule, but never spin on it
+    if (rc == DF_OK && !progressed && running == 0 && next < nmol) {
+      // nothing runs, nothing has just finished and the next molecule still does not fit: cannot
+      // happen while the workspace holds the largest molecule, but never spin on it
       set_error("scf_run_batch: molecule %d does not fit in the workspace", order[next]);
       rc = DF_ERR_NOMEM;
     }

@@ -90,3 +90,13 @@ def test_wait_that_runs_out_at_a_small_size():
             dfscf.lib().df_tune_set(name, v)
     torch.cuda.synchronize()
     _check(_sym(60, 1), 4)
+
+
+def test_batch_with_one_slot():
+    """Molecules one after another: the pass in which the last running one ends, before the next
+    has started, is not a workspace too small."""
+    import gen
+    mols = [gen.make_molecule(n, gen.molecules.box_for(n), n) for n in (8, 5, 6)]
+    batch = dfscf.scf_run_batch(mols, precision="fp64", slots=1)
+    for m, r in zip(mols, batch.results):
+        assert abs(r.energy - dfscf.scf_run(m, precision="fp64").energy) <= 1e-9
