@@ -2251,9 +2251,10 @@ extern "C" int scf_run_batch(const df_molecule* mols, int nmol, const scf_opts* 
     slot_off[k] = off;
     running++;
     DF_TRY(init_mol(*M, &mols[i], o, (char*)work + off, bytes[i], streams[k]));
-    // Each diagonalises on several SMs all the same: the cooperative grids are small (n / 5 CTAs) and
-    // launch when they fit.  8 molecules of 10 to 40 centres 439 -> 113 ms, 64 on 16 slots
-    // 1161 -> 679, 128 of 8 to 24 on 128 slots 467 -> 396, against one CTA each.
+    // With several molecules in flight each diagonalises on one CTA: many one-CTA
+    // eigensolvers fill the SMs in parallel, while cooperative grids from different streams
+    // (one CTA per SM each) would contend for co-residency.
+    if (slots > 1) M->W.eig_aux = nullptr;
     M->hst = hst + k;
     M->h_eps = heps + (size_t)(max_nao + 1) * k;
     M->h_ints = hints + 2 * k;
