@@ -56,6 +56,12 @@ __device__ __forceinline__ bool ll_load(const Word* p, unsigned tag, double& v) 
   return (unsigned)(lo >> 32) == tag && (unsigned)(hi >> 32) == tag;
 }
 
+__device__ __forceinline__ unsigned long long global_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
 // Barrier of one half of the CTA (1: the row warps, 2: the reflector warps) or of both (3).
 __device__ __forceinline__ void bar(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
 
@@ -176,12 +182,16 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
   const int nrows = (n - 1 - cta) / G + 1, last_row = (nrows - 1) * G + cta;
   bool lost = false;
   unsigned it = 0;
+  // A wait ends after `limit` polls, or two seconds: a poll takes a microsecond, and several when
+  // every CTA of a full grid polls.
+  const unsigned long long t0 = global_ns();
   auto tired = [&]() {
-    if (++it > limit) {
+    const bool look = (++it & 255u) == 0u;
+    if (it > limit || (look && global_ns() - t0 > 2000000000ull + 100000ull * (unsigned)n)) {
       atomicCAS(&ctl->err, 0, 1);
       return true;
     }
-    return (it & 255u) == 0u && *(volatile int*)&ctl->err != 0;
+    return look && *(volatile int*)&ctl->err != 0;
   };
   unsigned top = 0;  // high word of the largest |element|
   for (int s = 0; s < nrows; ++s)
