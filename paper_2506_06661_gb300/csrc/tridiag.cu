@@ -62,8 +62,13 @@ __device__ __forceinline__ unsigned long long global_ns() {
   return t;
 }
 
-// Barrier of one half of the CTA (1: the row warps, 2: the reflector warps) or of both (3).
-__device__ __forceinline__ void bar(int id, int threads) { asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory"); }
+// Barrier of one half of the CTA (1: the row warps, 2: the reflector warps) or of both (3).  The
+// instruction counts whole warps and wants them converged, and the lanes of a warp leave a polling
+// loop one by one: they meet first.
+__device__ __forceinline__ void bar(int id, int threads) {
+  __syncwarp();
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
 
 // One pass over S owned rows (slots s0 .. s0 + S - 1, global rows from r0 in steps of G): the
 // pending update, y = row . x, and the entry of column kk + 1.  The S sums are
