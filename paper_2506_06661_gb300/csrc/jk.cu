@@ -61,108 +61,36 @@ int recorded_B_planes(const void* B) {
 }
 
 // ---- BF16 planes of B ------------------------------------------------------------------
-// Rows (P, m) of the full symmetric B_P (over n) as `planes` row-scaled planes (planes.cuh), padding
-// (m or n >= nao) zero.  One CTA per P and 32 rows m; tiles of 32 x 64 of the packed rows go through
-// shared memory, read along rows left of the diagonal and along columns right of it, once for the row
-// maxima and (from L2) once for the planes.  The planes come from x as a 62-bit integer in units of
-// 2^-62 sigma: FP64 arithmetic, about 20 instructions an element, bounded the kernel that used it
-// (7.5 ms for 900 x 300 x 300 in 5 planes, 1.2 ms here).
+// Row (P, m) of the full symmetric B_P (over n) as `planes` row-scaled planes (planes.cuh;
+// residuals in FP64).  One CTA per row; padding (m or n >= nao) is zero.
 struct PlaneOut {
   __nv_bfloat16* p[kMixedPlanes];
   int planes;
 };
 
-// Round half to even of v / 2^s.
-__device__ __forceinline__ long long round_shift(long long v, int s) {
-  return (v + ((1ll << (s - 1)) - 1) + ((v >> s) & 1)) >> s;
-}
-
-// The planes of x in a row of exponent field f (sigma = 2^(f - 1022)).
-__device__ __forceinline__ void split_row_bits(double x, int f, __nv_bfloat16 (&q)[kPlanesMax]) {
-  const unsigned long long u = (unsigned long long)__double_as_longlong(x);
-  const int fx = (int)((u >> 52) & 0x7ffu);
-  if (fx == 0x7ff) {  // not finite: neither is what it contributes to
-#pragma unroll
-    for (int j = 0; j < kPlanesMax; ++j) q[j] = __float2bfloat16_rn(NAN);
-    return;
-  }
-  unsigned long long m = u & 0xfffffffffffffull;
-  if (fx) m |= 1ull << 52;
-  const int s = 9 - (f - max(fx, 1));  // m 2^s counts 2^-62 sigma
-  if (s >= 0) m <<= s;
-  else if (s > -55) m = (m + (1ull << (-s - 1))) >> (-s);
-  else m = 0;
-  long long v = (long long)u < 0 ? -(long long)m : (long long)m;  // |v| < 2^62
-  // sigma in FP32; beyond its range the planes are zero or infinite as FP32 conversions would have them
-  const int sf = f - 1022 + 127;
-  const float sig = sf <= 0 ? 0.0f : (sf >= 255 ? INFINITY : __int_as_float(sf << 23));
-  const long long n0 = round_shift(v, 55);
-  v -= n0 << 55;
-  const long long n1 = round_shift(v, 47);
-  v -= n1 << 47;
-  q[0] = __float2bfloat16_rn((float)(int)n0 * 0x1p-7f * sig);
-  q[1] = __float2bfloat16_rn((float)(int)n1 * 0x1p-15f * sig);
-#pragma unroll
-  for (int j = 2; j < kPlanesMax; ++j) {
-    const float r = __bfloat162float(__float2bfloat16_rn(__ll2float_rn(v)));  // an integer
-    q[j] = __float2bfloat16_rn(r * 0x1p-62f * sig);
-    v -= __float2ll_rn(r);
-  }
-}
-
-constexpr int PT = 32, PN = 64;
-__global__ void __launch_bounds__(256) b_to_planes_kernel(const double* __restrict__ B64, long ld, int nao, int npad,
+__global__ void __launch_bounds__(128) b_to_planes_kernel(const double* __restrict__ B64, long ld, int nao, int npad,
                                                           PlaneOut out) {
-  __shared__ double T[PT][PN + 1];
-  const int m0 = blockIdx.x * PT, P = blockIdx.y, tid = threadIdx.x;
-  const double* b = B64 + (size_t)P * ld;
-  auto load = [&](int n0) {
-    __syncthreads();
-    if (n0 <= m0 + PT - 1)  // left of the diagonal (n <= m): consecutive threads along n
-#pragma unroll
-      for (int e = tid; e < PT * PN; e += 256) {
-        const int i = e / PN, j = e % PN, m = m0 + i, n = n0 + j;
-        if (n <= m && m < nao) T[i][j] = b[DF_IX((size_t)m * (m + 1) / 2 + n, ld)];
-      }
-    if (n0 + PN - 1 > m0)  // right of it (n > m): consecutive threads along m
-#pragma unroll
-      for (int e = tid; e < PT * PN; e += 256) {
-        const int j = e / PT, i = e % PT, m = m0 + i, n = n0 + j;
-        if (n > m && n < nao) T[i][j] = b[DF_IX((size_t)n * (n + 1) / 2 + m, ld)];
-      }
-    __syncthreads();
+  __shared__ double sh[4];
+  const int m = blockIdx.x, P = blockIdx.y;
+  const double* row = B64 + (size_t)P * ld;
+  auto load = [&](int n) -> double {
+    if (m >= nao || n >= nao) return 0.0;
+    int a = max(m, n), b = min(m, n);
+    return row[DF_IX((size_t)a * (a + 1) / 2 + b, ld)];
   };
-  const int r = tid >> 3, u = tid & 7, m = m0 + r;  // 8 threads per row, 8 elements each
-  unsigned t = 0;
-  for (int n0 = 0; n0 < nao; n0 += PN) {
-    load(n0);
-    if (m < nao)
+  double amax = 0.0;
+  for (int n = threadIdx.x; n < npad; n += blockDim.x) amax = fmax(amax, fabs(load(n)));
+  for (int o = 16; o; o >>= 1) amax = fmax(amax, __shfl_xor_sync(0xffffffffu, amax, o));
+  if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = amax;
+  __syncthreads();
+  const double sig = row_scale(fmax(fmax(sh[0], sh[1]), fmax(sh[2], sh[3])));
+  const size_t o = ((size_t)P * npad + m) * npad;
+  for (int n = threadIdx.x; n < npad; n += blockDim.x) {
+    __nv_bfloat16 q[kPlanesMax];
+    split_row_value(load(n), sig, q);
 #pragma unroll
-      for (int j = 0; j < 8; ++j) {
-        const int c = u + 8 * j;
-        if (n0 + c < nao) {
-          const unsigned k = (unsigned)__double2hiint(T[r][c]) & 0x7fffffffu;
-          if (k < 0x7ff00000u) t = max(t, k);
-        }
-      }
-  }
-  for (int o = 4; o; o >>= 1) t = max(t, __shfl_xor_sync(0xffffffffu, t, o));
-  const int f = max((int)(t >> 20), 1);
-  for (int n0 = 0; n0 < npad; n0 += PN) {
-    if (n0 < nao) load(n0);
-    const int c0 = n0 + 8 * u;
-    __align__(16) __nv_bfloat16 w[kPlanesMax][8];
-#pragma unroll
-    for (int j = 0; j < 8; ++j) {
-      __nv_bfloat16 q[kPlanesMax];
-      split_row_bits(m < nao && c0 + j < nao ? T[r][8 * u + j] : 0.0, f, q);
-#pragma unroll
-      for (int p = 0; p < kPlanesMax; ++p) w[p][j] = q[p];
-    }
-    const size_t at = DF_IXW(((size_t)P * npad + m) * npad + c0, 8, (size_t)gridDim.y * npad * npad);
-#pragma unroll
-    for (int p = 0; p < kMixedPlanes; ++p)
-      if (p < out.planes) *reinterpret_cast<uint4*>(out.p[p] + at) = *reinterpret_cast<const uint4*>(w[p]);
+    for (int j = 0; j < kMixedPlanes; ++j)
+      if (j < out.planes) out.p[j][DF_IX(o + n, (size_t)gridDim.y * npad * npad)] = q[j];
   }
 }
 
@@ -612,7 +540,7 @@ int build_B(const double* ao_xyz, const double* ao_exp, int nao, const double* a
     po.planes = L.planes;
     for (int j = 0; j < L.planes; ++j) po.p[j] = (__nv_bfloat16*)((char*)Bbuf + L.offp[j]);
     record_B_planes(Bbuf, L.planes);
-    b_to_planes_kernel<<<dim3((unsigned)L.npad / PT, (unsigned)naux), 256, 0, s>>>(B64, L.ld, nao, L.npad, po);
+    b_to_planes_kernel<<<dim3((unsigned)L.npad, (unsigned)naux), 128, 0, s>>>(B64, L.ld, nao, L.npad, po);
     DF_LAUNCHED("b_to_planes_kernel");
   }
   return DF_OK;

@@ -59,22 +59,14 @@ struct DiisState {
 };
 
 // ---- elementwise / reduction kernels ----------------------------------------------------
-// Sums over nao^2 elements run on all SMs: each CTA leaves a partial sum, and the kernel that needs the
-// total adds them in order.  On one CTA the energy took 143 us at 300 functions and the DIIS
-// products 106 (eight FP64 instructions in turn on every element of a thread).
-constexpr int kEnergyParts = 152;
-constexpr int kGramParts = 16;
-
-// F = h + J - K; part[b] = partial sum of D (h + F), NaN when an element of F is not finite; clears
-// the DIIS error's maximum.
-__global__ void __launch_bounds__(256) fock_energy_kernel(const double* __restrict__ h, const double* __restrict__ J,
-                                                          const double* __restrict__ K, const double* __restrict__ D,
-                                                          long nn, double* __restrict__ F, double* __restrict__ part,
-                                                          ScfStatus* st) {
-  __shared__ double sh[8];
+// F = h + J - K; status.energy = 1/2 sum D (h + F) + enuc; nonfinite flag.
+__global__ void fock_energy_kernel(const double* __restrict__ h, const double* __restrict__ J,
+                                   const double* __restrict__ K, const double* __restrict__ D, long nn,
+                                   const double* __restrict__ enuc, double* __restrict__ F, ScfStatus* st) {
+  __shared__ double sh[32];
   double e = 0.0;
   int bad = 0;
-  for (long i = (long)blockIdx.x * blockDim.x + threadIdx.x; i < nn; i += (long)gridDim.x * blockDim.x) {
+  for (long i = threadIdx.x; i < nn; i += blockDim.x) {
     double f = h[i] + J[i] - K[i];
     F[i] = f;
     e += D[i] * (h[i] + f);
@@ -83,45 +75,17 @@ __global__ void __launch_bounds__(256) fock_energy_kernel(const double* __restri
   e = block_sum(e, sh);
   bad = __syncthreads_or(bad);
   if (threadIdx.x == 0) {
-    part[blockIdx.x] = bad ? NAN : e;
-    if (blockIdx.x == 0) st->emax = 0.0;
-  }
-}
-
-// status.energy = 1/2 sum of the parts + enuc, nonfinite flag (one warp).
-__device__ __forceinline__ void finish_energy(const double* __restrict__ part, const double* __restrict__ enuc,
-                                              ScfStatus* st) {
-  double e = 0.0;
-  for (int i = threadIdx.x; i < kEnergyParts; i += 32) e += part[i];
-  e = warp_sum(e);
-  if (threadIdx.x == 0) {
     st->energy = 0.5 * e + *enuc;
-    st->nonfinite = !isfinite(e);
+    st->nonfinite = bad || !isfinite(e);
   }
 }
 
-// out = T - T^T (T = F D S), i.e. F D S - S D F; its largest |element| into *top (cleared before; a NaN
-// counts as larger than any number).
-__global__ void __launch_bounds__(256) antisym_kernel(const double* __restrict__ T, int n, double* __restrict__ out,
-                                                      double* top) {
-  __shared__ unsigned long long sh;
-  if (threadIdx.x == 0) sh = 0;
-  __syncthreads();
-  const long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
-  unsigned long long m = 0;
-  if (q < (long)n * n) {
-    const int i = (int)(q / n), j = (int)(q % n);
-    const double v = T[q] - T[(size_t)j * n + i];
-    out[q] = v;
-    m = (unsigned long long)__double_as_longlong(v) & 0x7fffffffffffffffull;
-  }
-  for (int o = 16; o; o >>= 1) {
-    const unsigned long long t = __shfl_xor_sync(0xffffffffu, m, o);
-    m = t > m ? t : m;
-  }
-  if ((threadIdx.x & 31) == 0) atomicMax(&sh, m);
-  __syncthreads();
-  if (threadIdx.x == 0) atomicMax((unsigned long long*)top, sh);
+// out = T - T^T (T = F D S), i.e. F D S - S D F.
+__global__ void antisym_kernel(const double* __restrict__ T, int n, double* __restrict__ out) {
+  long q = (long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (q >= (long)n * n) return;
+  int i = (int)(q / n), j = (int)(q % n);
+  out[q] = T[q] - T[(size_t)j * n + i];
 }
 
 __global__ void absmax_kernel(const double* __restrict__ x, long n, double* out) {
@@ -192,128 +156,94 @@ __global__ void diis_store_kernel(const DiisState* __restrict__ d, const double*
   }
 }
 
-// part[j][p] = partial sums of <E[slot], E[j]> for valid slots j.
-__global__ void __launch_bounds__(256) diis_gram_kernel(const DiisState* __restrict__ d, const double* __restrict__ Eh,
-                                                        long nn, long ne, double* __restrict__ part) {
-  __shared__ double sh[8];
-  const int j = blockIdx.x;
+// G[slot][j] = G[j][slot] = <E[slot], E[j]> for valid slots j.
+__global__ void diis_gram_kernel(const DiisState* __restrict__ d, const double* __restrict__ Eh, long nn, long ne,
+                                 double* __restrict__ G) {
+  __shared__ double sh[32];
+  int j = blockIdx.x;
   if (j >= d->space || !d->valid[j]) return;
-  const double* a = Eh + (size_t)d->slot * nn;
+  int slot = d->slot;
+  const double* a = Eh + (size_t)slot * nn;
   const double* b = Eh + (size_t)j * nn;
   double s = 0.0;
-  for (long i = (long)blockIdx.y * blockDim.x + threadIdx.x; i < ne; i += (long)gridDim.y * blockDim.x)
-    s = fma(a[i], b[i], s);
+  for (long i = threadIdx.x; i < ne; i += blockDim.x) s += a[i] * b[i];
   s = block_sum(s, sh);
-  if (threadIdx.x == 0) part[j * kGramParts + blockIdx.y] = s;
+  if (threadIdx.x == 0) {
+    G[slot * DIIS_MAX + j] = s;
+    G[j * DIIS_MAX + slot] = s;
+  }
 }
 
-// The new row and column of G from the partial sums, then the bordered Pulay system over the valid
-// slots: one row per lane, Gaussian elimination with partial pivoting (rows stay in place, a mask
-// marks the used ones).  With fewer than two vectors, or when no pivot exceeds 1e-14 of the largest
-// entry, the newest vector gets coefficient 1; in the singular case the history restarts from
-// the newest vector.  The chain of FP64 instructions bounds it; on one lane it took 56 us for 8 vectors.
-__global__ void __launch_bounds__(32) diis_solve_kernel(DiisState* d, double* __restrict__ G,
-                                                        const double* __restrict__ part, double* __restrict__ coef,
-                                                        ScfStatus* st) {
-  __shared__ int order[DIIS_MAX];
-  const int lane = threadIdx.x, slot = d->slot;
-  const unsigned full = 0xffffffffu;
-  const bool valid = lane < d->space && d->valid[min(lane, DIIS_MAX - 1)];
-  const unsigned slots = __ballot_sync(full, valid);
-  const int m = __popc(slots), dim = m + 1;
-  if (valid) {
-    order[__popc(slots & ((1u << lane) - 1))] = lane;
-    double g = 0.0;
-    for (int q = 0; q < kGramParts; ++q) g += part[lane * kGramParts + q];
-    G[slot * DIIS_MAX + lane] = g;
-    G[lane * DIIS_MAX + slot] = g;
-  }
-  if (lane < DIIS_MAX) coef[lane] = 0.0;
-  if (lane == 0) st->singular = 0;
-  __syncwarp();
+// Solve the bordered Pulay system over the valid slots (one lane).  With fewer than two
+// vectors, or when no pivot exceeds 1e-14 of the largest entry, the newest vector gets
+// coefficient 1; in the singular case the history restarts from the newest vector.
+__global__ void diis_solve_kernel(DiisState* d, const double* __restrict__ G, double* __restrict__ coef,
+                                  ScfStatus* st) {
+  if (threadIdx.x != 0) return;
+  int order[DIIS_MAX];
+  int m = 0;
+  for (int k = 0; k < d->space; ++k)
+    if (d->valid[k]) order[m++] = k;
+  for (int i = 0; i < DIIS_MAX; ++i) coef[i] = 0.0;
+  st->singular = 0;
   if (m < 2) {
-    if (lane == 0) coef[slot] = 1.0;
+    coef[d->slot] = 1.0;
     return;
   }
-  // row `lane` of the system: valid slot number `lane`, or the border
-  const int mine = lane < m ? order[lane] : 0;
-  double scale = lane < m ? fabs(G[mine * DIIS_MAX + mine]) : 0.0;
-  for (int o = 16; o; o >>= 1) scale = fmax(scale, __shfl_xor_sync(full, scale, o));
-  const double inv = scale > 0.0 ? 1.0 / scale : 1.0;
-  double A[DIIS_MAX + 1], rhs = lane == m ? -1.0 : 0.0, amax = 0.0;
-#pragma unroll
-  for (int k = 0; k <= DIIS_MAX; ++k) {
-    double v = 0.0;
-    if (k < m) v = lane < m ? G[mine * DIIS_MAX + order[k]] * inv : (lane == m ? -1.0 : 0.0);
-    else if (k == m) v = lane < m ? -1.0 : 0.0;
-    A[k] = v;
-    amax = fmax(amax, fabs(v));
+  double A[DIIS_MAX + 1][DIIS_MAX + 2];
+  int dim = m + 1;
+  double scale = 0.0;
+  for (int i = 0; i < m; ++i) scale = fmax(scale, fabs(G[order[i] * DIIS_MAX + order[i]]));
+  if (!(scale > 0.0)) scale = 1.0;
+  for (int i = 0; i < m; ++i) {
+    for (int j = 0; j < m; ++j) A[i][j] = G[order[i] * DIIS_MAX + order[j]] / scale;
+    A[i][m] = -1.0;
+    A[m][i] = -1.0;
+    A[i][dim] = 0.0;
   }
-  for (int o = 16; o; o >>= 1) amax = fmax(amax, __shfl_xor_sync(full, amax, o));
-  amax = fmax(amax, 1.0);
-  bool used = lane >= dim, ok = true;
-  int place = -1;  // the column this lane's row is the pivot of
-  double rp = 0.0;
-#pragma unroll
-  for (int c = 0; c <= DIIS_MAX; ++c) {
-    if (c >= dim || !ok) continue;
-    // largest |A[c]| of the rows left, the lowest lane among equals
-    unsigned long long key = used ? 0ull : (unsigned long long)__double_as_longlong(fabs(A[c]));
-    unsigned long long top = key;
-    for (int o = 16; o; o >>= 1) {
-      const unsigned long long t = __shfl_xor_sync(full, top, o);
-      top = t > top ? t : top;
-    }
-    const double pmax = __longlong_as_double((long long)top);
-    if (!(pmax > 1e-14 * amax) || !isfinite(pmax)) {
+  A[m][m] = 0.0;
+  A[m][dim] = -1.0;
+  double amax = 0.0;
+  for (int i = 0; i < dim; ++i)
+    for (int j = 0; j < dim; ++j) amax = fmax(amax, fabs(A[i][j]));
+  bool ok = true;
+  for (int c = 0; c < dim && ok; ++c) {
+    int p = c;
+    for (int r = c + 1; r < dim; ++r)
+      if (fabs(A[r][c]) > fabs(A[p][c])) p = r;
+    if (!(fabs(A[p][c]) > 1e-14 * amax)) {
       ok = false;
-      continue;
+      break;
     }
-    const int p = __ffs(__ballot_sync(full, !used && key == top)) - 1;
-    const double pv = __shfl_sync(full, A[c], p), r = 1.0 / pv, f = A[c] * r;
-    if (lane == p) {
-      used = true;
-      place = c;
-      rp = r;
-    }
-    const bool change = !used;
-#pragma unroll
-    for (int k = c; k <= DIIS_MAX; ++k)
-      if (k < dim) {
-        const double row = __shfl_sync(full, A[k], p);
-        if (change) A[k] = fma(-f, row, A[k]);
+    if (p != c)
+      for (int k = 0; k <= dim; ++k) {
+        double t = A[c][k];
+        A[c][k] = A[p][k];
+        A[p][k] = t;
       }
-    const double row = __shfl_sync(full, rhs, p);
-    if (change) rhs = fma(-f, row, rhs);
+    for (int r = c + 1; r < dim; ++r) {
+      double f = A[r][c] / A[c][c];
+      for (int k = c; k <= dim; ++k) A[r][k] -= f * A[c][k];
+    }
   }
   if (ok) {
     double x[DIIS_MAX + 1];
-#pragma unroll
-    for (int c = DIIS_MAX; c >= 0; --c) {
-      x[c] = 0.0;
-      if (c >= dim) continue;
-      const int p = __ffs(__ballot_sync(full, place == c)) - 1;
-      x[c] = __shfl_sync(full, rhs * rp, p);
-      rhs = fma(-A[c], x[c], rhs);
+    for (int r = dim - 1; r >= 0; --r) {
+      double s = A[r][dim];
+      for (int k = r + 1; k < dim; ++k) s -= A[r][k] * x[k];
+      x[r] = s / A[r][r];
     }
-    bool finite = true;
-    double own = 0.0;
-#pragma unroll
-    for (int c = 0; c < DIIS_MAX; ++c) {
-      if (c < m && !isfinite(x[c])) finite = false;
-      if (c == lane) own = x[c];
+    for (int i = 0; i < m; ++i) {
+      if (!isfinite(x[i])) ok = false;
+      coef[order[i]] = x[i];
     }
-    if (lane < m) coef[mine] = own;
-    ok = finite;
   }
   if (!ok) {
-    __syncwarp();
-    if (lane < DIIS_MAX) coef[lane] = lane == slot ? 1.0 : 0.0;
-    if (lane < d->space) d->valid[lane] = lane == slot;
-    if (lane == 0) {
-      d->nvalid = 1;
-      st->singular = 1;
-    }
+    for (int i = 0; i < DIIS_MAX; ++i) coef[i] = 0.0;
+    coef[d->slot] = 1.0;
+    for (int k = 0; k < DIIS_MAX; ++k) d->valid[k] = (k == d->slot);
+    d->nvalid = 1;
+    st->singular = 1;
   }
 }
 
@@ -349,10 +279,9 @@ __global__ void occ_columns_kernel(const double* __restrict__ ZT, int nmo, int n
 }
 
 // HOMO / LUMO of the last diagonalisation, its eigensolver status and the tensor-core
-// exchange's timeout flag (tc_err may be null: an FP64 iteration) and the energy into the status block.
+// exchange's timeout flag (tc_err may be null: an FP64 iteration) into the status block.
 __global__ void orbital_status_kernel(const double* __restrict__ eps, int nmo, int nocc, const int* eig_status,
-                                      const int* tc_err, const double* part, const double* enuc, ScfStatus* st) {
-  finish_energy(part, enuc, st);
+                                      const int* tc_err, ScfStatus* st) {
   if (threadIdx.x != 0) return;
   st->homo = nocc > 0 ? eps[nocc - 1] : 0.0;
   st->lumo = nocc < nmo ? eps[nocc] : 0.0;
@@ -645,8 +574,7 @@ __global__ void add_identity_kernel(double* __restrict__ A, int n) {
 
 // HOMO / LUMO estimates (diagonal of F_mo) and statuses after a Newton step.
 __global__ void soscf_status_kernel(const double* __restrict__ Fmo, int nmo, int nocc, const int* k_status,
-                                    const int* tc_err, const double* part, const double* enuc, ScfStatus* st) {
-  finish_energy(part, enuc, st);
+                                    const int* tc_err, ScfStatus* st) {
   if (threadIdx.x != 0) return;
   double homo = -INFINITY, lumo = INFINITY;
   for (int i = 0; i < nocc; ++i) homo = fmax(homo, Fmo[(size_t)i * nmo + i]);
@@ -661,7 +589,6 @@ static unsigned blocks_for(long n, int t = 256) { return (unsigned)((n + t - 1) 
 
 // ---- per-molecule workspace --------------------------------------------------------------
 struct ScfWork {
-  double* part;  // partial sums: energy [kEnergyParts], DIIS products [DIIS_MAX][kGramParts]
   double *L, *pair_tab, *S, *h, *V, *X, *F, *Fo, *Cp, *J, *K, *D, *Dprev, *Cocc, *Cprev, *Cchunk, *T1, *T2, *E, *Fp,
       *ZT, *eps, *Fhist, *Ehist, *G, *coef, *eig_scratch, *enuc, *maxdiag;
   int *eig_status, *chol_status, *idx;
@@ -722,7 +649,6 @@ static void scf_layout(int nao, int naux, int nocc, int precision, Arena* a, Siz
   TAKE(double, w->Ehist, DIIS_MAX * nn);
   TAKE(double, w->G, DIIS_MAX * DIIS_MAX);
   TAKE(double, w->coef, DIIS_MAX);
-  TAKE(double, w->part, kEnergyParts + DIIS_MAX * kGramParts);
   TAKE(double, w->eig_scratch, eigh_full_scratch_doubles(nao));
   TAKE(double, w->enuc, 1);
   TAKE(double, w->maxdiag, 1);
@@ -1693,7 +1619,7 @@ static int iteration_tail(ScfMol& M, int prec) {
   const long nn = (long)nao * nao, ne = (long)nmo * nmo;
   {
     ProfScope ps("scf_fock_energy", s);
-    fock_energy_kernel<<<kEnergyParts, 256, 0, s>>>(W.h, W.J, W.K, W.D, nn, W.F, W.part, W.st);
+    fock_energy_kernel<<<1, 1024, 0, s>>>(W.h, W.J, W.K, W.D, nn, W.enuc, W.F, W.st);
     DF_LAUNCHED("fock_energy_kernel");
   }
   {
@@ -1707,27 +1633,27 @@ static int iteration_tail(ScfMol& M, int prec) {
       // a starting density need not lie in the span of X C': AO-basis commutator
       DF_TRY(dgemm(false, false, nao, nao, nao, 1.0, W.F, nao, 0, W.D, nao, 0, 0.0, W.T1, nao, 0, 1, s, 0, 0));
       DF_TRY(dgemm(false, false, nao, nao, nao, 1.0, W.T1, nao, 0, W.S, nao, 0, 0.0, W.T2, nao, 0, 1, s, 0, 0));
-      antisym_kernel<<<blocks_for(nn), 256, 0, s>>>(W.T2, nao, W.T1, &W.st->emax);
+      antisym_kernel<<<blocks_for(nn), 256, 0, s>>>(W.T2, nao, W.T1);
       DF_LAUNCHED("antisym_kernel");
       DF_TRY(dgemm(false, false, nao, nmo, nao, 1.0, W.T1, nao, 0, W.X, nmo, 0, 0.0, W.T2, nmo, 0, 1, s, 0, 0));
       DF_TRY(dgemm(true, false, nmo, nmo, nao, 1.0, W.X, nmo, 0, W.T2, nmo, 0, 0.0, W.E, nmo, 0, 1, s, 0, 0));
-      absmax_kernel<<<1, 1024, 0, s>>>(W.E, ne, &W.st->emax);  // of X^T e X, not of e
-      DF_LAUNCHED("absmax_kernel");
     } else {
       DF_TRY(dgemm(false, false, nmo, nocc, nmo, 1.0, W.Fo, nmo, 0, W.Cp, nocc, 0, 0.0, W.T1, nocc, 0, 1, s, 0, 0));
       DF_TRY(dgemm(false, true, nmo, nmo, nocc, 2.0, W.T1, nocc, 0, W.Cp, nocc, 0, 0.0, W.T2, nmo, 0, 1, s, 0, 0));
-      antisym_kernel<<<blocks_for(ne), 256, 0, s>>>(W.T2, nmo, W.E, &W.st->emax);
+      antisym_kernel<<<blocks_for(ne), 256, 0, s>>>(W.T2, nmo, W.E);
       DF_LAUNCHED("antisym_kernel");
     }
+    absmax_kernel<<<1, 1024, 0, s>>>(W.E, ne, &W.st->emax);
+    DF_LAUNCHED("absmax_kernel");
   }
   ProfScope ps_diis("scf_diis_and_diagonalize", s);
   diis_select_kernel<<<1, 32, 0, s>>>(W.diis);
   DF_LAUNCHED("diis_select_kernel");
   diis_store_kernel<<<blocks_for(ne), 256, 0, s>>>(W.diis, W.Fo, W.E, W.Fhist, W.Ehist, nn, ne);
   DF_LAUNCHED("diis_store_kernel");
-  diis_gram_kernel<<<dim3(DIIS_MAX, kGramParts), 256, 0, s>>>(W.diis, W.Ehist, nn, ne, W.part + kEnergyParts);
+  diis_gram_kernel<<<DIIS_MAX, 256, 0, s>>>(W.diis, W.Ehist, nn, ne, W.G);
   DF_LAUNCHED("diis_gram_kernel");
-  diis_solve_kernel<<<1, 32, 0, s>>>(W.diis, W.G, W.part + kEnergyParts, W.coef, W.st);
+  diis_solve_kernel<<<1, 32, 0, s>>>(W.diis, W.G, W.coef, W.st);
   DF_LAUNCHED("diis_solve_kernel");
   diis_combine_kernel<<<blocks_for(ne), 256, 0, s>>>(W.diis, W.Fhist, nn, ne, W.coef, W.Fp);
   DF_LAUNCHED("diis_combine_kernel");
@@ -1735,7 +1661,7 @@ static int iteration_tail(ScfMol& M, int prec) {
   DF_TRY(diagonalize_orth(nao, nmo, nocc, W, s));
   if (M.inc) DF_TRY(incremental_prep(M));
   orbital_status_kernel<<<1, 32, 0, s>>>(W.eps, nmo, nocc, W.eig_status, prec == DF_MIXED ? W.jk.mk.err : nullptr,
-                                         W.part, W.enuc, W.st);
+                                         W.st);
   DF_LAUNCHED("orbital_status_kernel");
   DF_CUDA(cudaMemcpyAsync(M.hst, W.st, sizeof(ScfStatus), cudaMemcpyDeviceToHost, s));
   return DF_OK;
@@ -1749,17 +1675,18 @@ static int iteration_tail_soscf(ScfMol& M, int prec) {
   cudaStream_t s = M.s;
   const int nao = M.nao, nmo = M.nmo, nocc = M.nocc;
   const long nn = (long)nao * nao, ne = (long)nmo * nmo;
-  fock_energy_kernel<<<kEnergyParts, 256, 0, s>>>(W.h, W.J, W.K, W.D, nn, W.F, W.part, W.st);
+  fock_energy_kernel<<<1, 1024, 0, s>>>(W.h, W.J, W.K, W.D, nn, W.enuc, W.F, W.st);
   DF_LAUNCHED("fock_energy_kernel");
   DF_TRY(to_orth(W.F, nao, nmo, W, W.Fo, s));
   DF_TRY(dgemm(false, false, nmo, nocc, nmo, 1.0, W.Fo, nmo, 0, W.Cp, nocc, 0, 0.0, W.T1, nocc, 0, 1, s, 0, 0));
   DF_TRY(dgemm(false, true, nmo, nmo, nocc, 2.0, W.T1, nocc, 0, W.Cp, nocc, 0, 0.0, W.T2, nmo, 0, 1, s, 0, 0));
-  antisym_kernel<<<blocks_for(ne), 256, 0, s>>>(W.T2, nmo, W.E, &W.st->emax);
+  antisym_kernel<<<blocks_for(ne), 256, 0, s>>>(W.T2, nmo, W.E);
   DF_LAUNCHED("antisym_kernel");
+  absmax_kernel<<<1, 1024, 0, s>>>(W.E, ne, &W.st->emax);
+  DF_LAUNCHED("absmax_kernel");
   DF_TRY(soscf_step(M));
   if (M.inc) DF_TRY(incremental_prep(M));
-  soscf_status_kernel<<<1, 32, 0, s>>>(W.Fmo, nmo, nocc, W.k_status, prec == DF_MIXED ? W.jk.mk.err : nullptr,
-                                       W.part, W.enuc, W.st);
+  soscf_status_kernel<<<1, 32, 0, s>>>(W.Fmo, nmo, nocc, W.k_status, prec == DF_MIXED ? W.jk.mk.err : nullptr, W.st);
   DF_LAUNCHED("soscf_status_kernel");
   DF_CUDA(cudaMemcpyAsync(M.hst, W.st, sizeof(ScfStatus), cudaMemcpyDeviceToHost, s));
   return DF_OK;
