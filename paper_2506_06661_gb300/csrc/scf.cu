@@ -787,7 +787,6 @@ struct ScfMol {
   bool soscf_pending = false; // switch before the next launch
   double d_best = INFINITY;
   int d_stall = 0;
-  std::vector<double> d_hist;  // best error after each iteration
   enum KPhase { KP_FULL, KP_BASE, KP_INCR, KP_FINAL } kp = KP_FULL;
   int rebases = 0;
   double inc_best = INFINITY;
@@ -1918,15 +1917,8 @@ static bool scf_iter_finish(ScfMol& M) {
   } else {
     M.d_stall++;
   }
-  // Near a saddle point DIIS can also creep on, now and then by 10%, for a number of iterations
-  // that the last bits decide (92, 103 and 127 for one molecule under three orders of summation):
-  // less than a factor of 10 on the best error in 40 iterations is a stall too.
-  M.d_hist.push_back(M.d_best);
-  const size_t nd = M.d_hist.size();
-  const bool creeping = nd > 40 && M.d_best > 0.1 * M.d_hist[nd - 41];
   const bool accurate_fock = M.prec == DF_FP64 || (M.inc && M.kp == ScfMol::KP_INCR);
-  if (M.soscf_on && !M.soscf && !M.soscf_pending && accurate_fock && (M.d_stall >= 12 || creeping) &&
-      M.d_best < 0.1) {
+  if (M.soscf_on && !M.soscf && !M.soscf_pending && accurate_fock && M.d_stall >= 12 && M.d_best < 0.1) {
     M.soscf_pending = true;
     M.inc_stall = 0;
   }
