@@ -892,7 +892,10 @@ __global__ void __launch_bounds__(256, 1) eigh_fallback_coop_kernel(const double
                                                                   int* status) {
   extern __shared__ double smem_d[];
   __shared__ EigShared sh;
-  const bool gave_up = ctl->err == 1;
+  __shared__ int gave_up;
+  // one thread reads the flag, which CTAs that are ahead may raise, for its whole CTA
+  if (threadIdx.x == 0) gave_up = *(volatile int*)&ctl->err == 1;
+  __syncthreads();
   if (gave_up || !eig_needs_fallback(ctl, k)) {
     if (blockIdx.x == 0 && threadIdx.x == 0) *status = gave_up ? 3 : 0;
     return;

@@ -447,9 +447,13 @@ __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const dou
   __shared__ double sh[4];
   __shared__ unsigned shm[4];
   __shared__ unsigned long long best;
-  __shared__ int pick[5];
-  if (ctl->err | ctl->bad) return;
+  __shared__ int pick[5], leave;
   const int tid = threadIdx.x, t = (int)blockIdx.x;
+  // Other CTAs of this grid may raise ctl->bad at any time: one thread reads it for all, or part of
+  // the CTA would leave and the rest work on shared memory that was never written.
+  if (tid == 0) leave = ctl->err | *(volatile int*)&ctl->bad;
+  __syncthreads();
+  if (leave) return;
   Row* T = (Row*)smem_d;
   double* p = smem_d + 2 * (size_t)n;
   double* s = p + n;
