@@ -18,8 +18,8 @@
  *   - all matrices are row-major; all array arguments are DEVICE pointers unless the
  *     parameter is documented as host memory;
  *   - the caller owns every buffer.  Calls that need scratch take (work, work_bytes);
- *     the matching *_work_bytes() query gives the size.  The library never allocates
- *     device memory;
+ *     the matching *_work_bytes() query gives the size, for a `work` of any alignment.
+ *     The library never allocates device memory;
  *   - every call is asynchronous on stream `s` unless documented otherwise; results are
  *     valid once the stream has synchronised;
  *   - every call returns DF_OK or one of the error codes below and, on error, records a

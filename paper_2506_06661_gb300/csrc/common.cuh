@@ -32,13 +32,21 @@ constexpr double kPi = 3.14159265358979323846;
 inline size_t align_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 inline long npair_of(int nao) { return (long)nao * (nao + 1) / 2; }
 
+// Callers may pass a workspace of any alignment; the kernels make 16-byte accesses and TMA copies
+// to it.  The size queries add kWorkAlign bytes, and what is laid out starts at the first multiple.
+constexpr size_t kWorkAlign = 256;
+inline char* aligned_work(void* work) { return (char*)(((uintptr_t)work + kWorkAlign - 1) / kWorkAlign * kWorkAlign); }
+
 // Bump allocator over a caller-owned workspace; every slice is 256-byte aligned.
 struct Arena {
   char* base;
   size_t size;
   size_t used = 0;
   bool overflow = false;
-  Arena(void* b, size_t s) : base((char*)b), size(s) {}
+  Arena(void* b, size_t s) : base(aligned_work(b)), size(s) {
+    const size_t pad = (size_t)(base - (char*)b);
+    size = s > pad ? s - pad : 0;
+  }
   template <typename T>
   T* take(size_t count) {
     size_t off = align_up(used, 256);
@@ -54,7 +62,7 @@ struct Arena {
 
 // Size-only twin of Arena used by the *_work_bytes queries.
 struct Sizer {
-  size_t used = 0;
+  size_t used = kWorkAlign;
   template <typename T>
   void take(size_t count) {
     used = align_up(used, 256) + align_up(count * sizeof(T), 256);

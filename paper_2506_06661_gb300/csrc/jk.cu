@@ -559,8 +559,9 @@ extern "C" size_t df_B_bytes(int nao, int naux, int precision) {
 }
 
 extern "C" size_t df_build_B_work_bytes(int nao, int naux) {
-  if (nao <= 0 || naux <= 0) return nao > 0 ? align_up(sizeof(double) * pair_tab_doubles(nao), 256) : 0;
-  return align_up(sizeof(double) * pair_tab_doubles(nao), 256) + forward_substitution_bytes(B_ld(nao), naux);
+  if (nao <= 0) return 0;
+  return kWorkAlign + align_up(sizeof(double) * pair_tab_doubles(nao), 256) +
+         (naux > 0 ? forward_substitution_bytes(B_ld(nao), naux) : 0);
 }
 
 extern "C" int df_build_B(const double* ao_xyz, const double* ao_exp, int nao, const double* aux_xyz,
@@ -575,6 +576,7 @@ extern "C" int df_build_B(const double* ao_xyz, const double* ao_exp, int nao, c
   DF_REQUIRE(work && work_bytes >= df_build_B_work_bytes(nao, naux), DF_ERR_NOMEM,
              "df_build_B: workspace of %zu bytes < %zu", work_bytes, df_build_B_work_bytes(nao, naux));
   DF_REQUIRE(precision == DF_FP64 || naux <= 65535, DF_ERR_ARG, "df_build_B: naux > 65535 in mixed mode");
+  work = aligned_work(work);
   return build_B(ao_xyz, ao_exp, nao, aux_xyz, aux_exp, naux, L, precision, B, (double*)work,
                  (char*)work + align_up(sizeof(double) * pair_tab_doubles(nao), 256), s);
 }

@@ -455,7 +455,7 @@ int forward_substitution(double* R, long ld, long ncol, const double* L, int nau
 using namespace dfscf;
 
 extern "C" size_t df_metric_chol_work_bytes(int naux) {
-  return 512 + sizeof(double) * align_up(boys_table_doubles(), 32) + (naux > 0 ? cholesky_bytes(naux) : 0);
+  return kWorkAlign + 512 + sizeof(double) * align_up(boys_table_doubles(), 32) + (naux > 0 ? cholesky_bytes(naux) : 0);
 }
 
 extern "C" int df_metric_chol(const double* aux_xyz, const double* aux_exp, int naux, double* L, double* M_out,
@@ -465,6 +465,7 @@ extern "C" int df_metric_chol(const double* aux_xyz, const double* aux_exp, int 
   DF_REQUIRE(work && work_bytes >= df_metric_chol_work_bytes(naux), DF_ERR_NOMEM,
              "df_metric_chol: workspace of %zu bytes is smaller than %zu", work_bytes, df_metric_chol_work_bytes(naux));
   *bad_pivot = -1;
+  work = aligned_work(work);
   int* d_status = (int*)work;
   double* d_maxdiag = (double*)((char*)work + 256);
   DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, L, (double*)((char*)work + 512), s));

@@ -229,8 +229,8 @@ extern "C" int df_lrdf_jk(const void* B_lr, const double* ao_xyz, const double* 
   Arena a(work, work_bytes);
   LrWork w{};
   lr_layout(nao, &a, nullptr, &w);
-  void* jkw = (char*)work + align_up(a.used, 256);
-  const size_t jkw_bytes = work_bytes - align_up(a.used, 256);
+  void* jkw = a.base + align_up(a.used, 256);
+  const size_t jkw_bytes = a.size - align_up(a.used, 256);
   // long-range part: ordinary DF J/K on the long-range tensor
   DF_TRY(df_jk(B_lr, nao, naux, DF_FP64, D, C, nocc, J, K, jkw, jkw_bytes, s));
   clear_error();

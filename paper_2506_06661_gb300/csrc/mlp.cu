@@ -691,8 +691,8 @@ extern "C" int guess_density(const float* params, const double* xyz, int natm, i
   double* Dt = a.take<double>((size_t)nao * nao);
   double* T = a.take<double>((size_t)nao * nao);
   double* scale = a.take<double>(1);
-  size_t rest = work_bytes - a.used;
-  void* mw = (char*)work + a.used;
+  size_t rest = a.size - a.used;
+  void* mw = a.base + a.used;
   env_kernel<<<natm, 32, 0, s>>>(xyz, natm, env);
   DF_LAUNCHED("env_kernel");
   pair_feature_kernel<float><<<(unsigned)np, 96, 0, s>>>(xyz, natm, env, feat, mask);
