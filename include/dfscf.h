@@ -103,7 +103,8 @@ int df_nuclear_repulsion(const double* nuc_xyz, const double* nuc_z, int natm, d
  * (Section "Density fitting", metric equation).  L is [naux][naux], lower triangle
  * filled, strict upper triangle set to zero.  Optionally M is also written to M_out
  * ([naux][naux], may be NULL).
- * Synchronises the stream once to read the pivot status.  If a pivot is <= 1e-14 times
+ * Synchronises the stream once to read the pivot status (DF_ERR_TIMEOUT, before any pivot,
+ * if a wait of the tensor-core updates gave up; L is then incomplete).  If a pivot is <= 1e-14 times
  * the largest diagonal element of M, returns DF_ERR_NOT_SPD and stores the 0-based
  * pivot index in the HOST int *bad_pivot (otherwise *bad_pivot = -1).
  * work: df_metric_chol_work_bytes(naux) bytes.                                         */
@@ -123,7 +124,9 @@ int df_metric_chol(const double* aux_xyz, const double* aux_exp, int naux, doubl
  *        npad = df_nao_pad(nao), padding zero; NP is the knob "mixed_planes" when
  *        df_B_bytes is called, and df_build_B must see the same value.  A later mixed
  *        df_jk needs NP at least its own "mixed_planes" (checked: DF_ERR_ARG otherwise).
- * L is the factor from df_metric_chol.  work: df_build_B_work_bytes(...) bytes.         */
+ * L is the factor from df_metric_chol.  Outside a stream capture the call synchronises the
+ * stream once and returns DF_ERR_TIMEOUT if a wait of the tensor-core whitening gave up (row 0
+ * of B is then NaN).  work: df_build_B_work_bytes(...) bytes.                              */
 long df_B_ld(int nao);
 int df_nao_pad(int nao);
 size_t df_B_bytes(int nao, int naux, int precision);
@@ -141,10 +144,10 @@ int df_B_get_packed(const void* B, int nao, int naux, int P, double* row, cudaSt
  * D: [nao][nao] symmetric density; C: [nao][nocc] occupied coefficients.  For an RHF
  * density D = 2 C C^T the Fock matrix is F = h + J - K.  J or K may be NULL to skip it
  * (then D or C may be NULL too).  precision DF_MIXED requires B built with DF_MIXED.
- * The tensor-core kernels of the mixed exchange bound every wait; if one gives up, K is
- * filled with NaN and, unless the stream is being captured into a graph, df_jk (which then
- * synchronises the stream once to read the flag) returns DF_ERR_TIMEOUT.  A mixed df_jk
- * outside a capture therefore returns with the stream drained.
+ * The tensor-core kernels of the exchange (both precisions) bound every wait; if one gives
+ * up, K is filled with NaN and, unless the stream is being captured into a graph, df_jk
+ * (which then synchronises the stream once to read the flag) returns DF_ERR_TIMEOUT.  A
+ * df_jk with K outside a capture therefore returns with the stream drained.
  * work: df_jk_work_bytes(nao, naux, nocc, precision) bytes.                           */
 size_t df_jk_work_bytes(int nao, int naux, int nocc, int precision);
 int df_jk(const void* B, int nao, int naux, int precision, const double* D, const double* C,
@@ -368,7 +371,7 @@ int df_congruence(const double* M, const double* A, int n, double* out, void* wo
  * differentiates automatically).  For an even-tempered set alpha_P = a beta^k_P on every
  * centre, theta = (ln a, ln beta) gives dalpha[P] = (alpha_P, k_P alpha_P).  *delta (HOST,
  * may be NULL) receives Delta.  Synchronises the stream (pivot check of the metric's
- * Cholesky factor: DF_ERR_NOT_SPD).  The Jacobian needs O(naux^2 npair) work and
+ * Cholesky factor: DF_ERR_NOT_SPD; DF_ERR_TIMEOUT as in df_build_B).  The Jacobian needs O(naux^2 npair) work and
  * 4 naux npair doubles of workspace: meant for small molecules or single atoms, as in the
  * paper's basis optimisation.  work: df_fit_residual_work_bytes(nao, naux, jac != NULL).   */
 size_t df_fit_residual_work_bytes(int nao, int naux, int with_jacobian);
@@ -382,12 +385,12 @@ int df_fit_residual(const double* ao_xyz, const double* ao_exp, int nao, const d
  * T = L^-1 (Q|mn)^LR, the short-range part computed exactly:
  *     (mn|kl) ~ (mn|kl)^SR + sum_P T_{P,mn} T_{P,kl}.
  * df_lrdf_build writes T (omega > 0) into B in the DF_FP64 layout of df_build_B
- * (df_B_bytes(nao, naux, DF_FP64) bytes), synchronising once for the metric's pivot check
- * (DF_ERR_NOT_SPD).  df_lrdf_jk returns J[D] and K[C C^T] (either may be NULL) as the
+ * (df_B_bytes(nao, naux, DF_FP64) bytes), synchronising for the metric's pivot check
+ * (DF_ERR_NOT_SPD) and at the end (DF_ERR_TIMEOUT as in df_build_B).  df_lrdf_jk returns J[D] and K[C C^T] (either may be NULL) as the
  * long-range DF part (df_jk on T) plus the short-range four-centre part, summed directly over
  * orbital pairs (quartets whose pair factors multiply to less than 1e-16 of the largest are
  * skipped).  The short-range sums cost O(npair^2) for J and O(nao^4) for K: meant for
- * molecules of up to a few hundred basis functions.  Both synchronise the stream once.
+ * molecules of up to a few hundred basis functions.  Both synchronise the stream.
  * works: df_lrdf_build_work_bytes(nao, naux), df_lrdf_jk_work_bytes(nao, naux, nocc).       */
 size_t df_lrdf_build_work_bytes(int nao, int naux);
 int df_lrdf_build(const double* ao_xyz, const double* ao_exp, int nao, const double* aux_xyz, const double* aux_exp,
@@ -459,7 +462,10 @@ int df_j_noalloc(const void* B, int nao, int naux, const double* D, double* J, c
  * Two more knobs bound the multi-SM eigensolver's grid barriers:
  * "eig_barrier_polls" (256..2^30 polls before a wait gives up with DF_ERR_TIMEOUT; default 2^22, about a second) and "eig_barrier_extra"
  * (0 or 1; 1 makes every barrier wait for one arrival that never comes, so that a test can
- * watch the bounded wait run out; leave it 0).  Host-side process-wide state: change
+ * watch the bounded wait run out; leave it 0).  "tc_give_up" (0..2) is the tensor-core
+ * kernels' test hook: 1 raises the error word of the metric's and the whitening's kernels before
+ * their launches, 2 that of the exchange, so that they skip their work and the call must report
+ * DF_ERR_TIMEOUT; leave it 0.  Host-side process-wide state: change
  * knobs only between calls and re-query *_work_bytes afterwards (split counts size the
  * workspaces).  df_tune_set returns DF_ERR_ARG for an unknown name or an out-of-range value;
  * df_tune_get returns -1 for an unknown name; df_tune_reset puts every knob back to its

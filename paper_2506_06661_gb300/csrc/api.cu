@@ -147,12 +147,31 @@ static Knob g_knobs[] = {
     {"eig_barrier_polls", 1 << 22, 256, 1 << 30},  // polls before a grid-barrier wait of the eigensolver gives up
     {"eig_barrier_extra", 0, 0, 1},  // test hook: 1 = every eigensolver grid barrier waits for one arrival
                                      // that never comes, so its bounded wait runs out
+    {"tc_give_up", 0, 0, 2},         // test hook: 1 = the metric and the whitening, 2 = the exchange find the error
+                                     // word of their tensor-core kernels raised, as a wait that gave up leaves it
 };
 
 int knob(const char* name) {
   for (auto& k : g_knobs)
     if (strcmp(k.name, name) == 0) return k.value;
   return 0;
+}
+
+int reset_tc_errors(int* err, int n, TcUser user, cudaStream_t s) {
+  DF_CUDA(cudaMemsetAsync(err, knob("tc_give_up") == user ? 1 : 0, sizeof(int) * (size_t)n, s));
+  return DF_OK;
+}
+
+int check_tc_errors(const int* err, int n, const char* who, cudaStream_t s) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  DF_CUDA(cudaStreamIsCapturing(s, &cs));
+  if (cs != cudaStreamCaptureStatusNone) return DF_OK;
+  int h[2] = {0, 0};
+  DF_REQUIRE(n <= 2, DF_ERR_ARG, "%s: too many error words", who);
+  DF_CUDA(cudaMemcpyAsync(h, err, sizeof(int) * (size_t)n, cudaMemcpyDeviceToHost, s));
+  DF_CUDA(cudaStreamSynchronize(s));
+  DF_REQUIRE(!(h[0] | h[1]), DF_ERR_TIMEOUT, "%s: a bounded wait of the tensor-core kernels gave up", who);
+  return DF_OK;
 }
 
 }  // namespace dfscf

@@ -206,7 +206,7 @@ extern "C" int df_fit_residual(const double* ao_xyz, const double* ao_exp, int n
   DF_TRY(cholesky_inplace(w.L, naux, w.status, w.maxdiag, 1e-14, w.subst, s));
   int h_status = -1;
   DF_CUDA(cudaMemcpyAsync(&h_status, w.status, sizeof(int), cudaMemcpyDeviceToHost, s));
-  DF_CUDA(cudaStreamSynchronize(s));
+  DF_TRY(check_tc_errors((const int*)w.subst, 1, "df_fit_residual", s));
   DF_REQUIRE(h_status < 0, DF_ERR_NOT_SPD, "df_fit_residual: auxiliary metric not positive definite at pivot %d",
              h_status);
   // T = L^-1 (P|mn), then sigma and Delta
@@ -217,6 +217,7 @@ extern "C" int df_fit_residual(const double* ao_xyz, const double* ao_exp, int n
   const double* pz = py + npair;
   const double* pk = pz + npair;
   DF_TRY(forward_substitution(w.T, ld, ld, w.L, naux, w.subst, s));
+  DF_TRY(check_tc_errors((const int*)w.subst, 1, "df_fit_residual", s));
   residual_kernel<<<(unsigned)((npair + 255) / 256), 256, 0, s>>>(pp, pk, npair, w.T, ld, naux, sigma);
   DF_LAUNCHED("residual_kernel");
   delta_kernel<<<1, 1024, 0, s>>>(sigma, nao, w.delta);
@@ -226,6 +227,7 @@ extern "C" int df_fit_residual(const double* ao_xyz, const double* ao_exp, int n
     identity_kernel<<<(unsigned)(((long)naux * naux + 255) / 256), 256, 0, s>>>(w.Linv, naux);
     DF_LAUNCHED("identity_kernel");
     DF_TRY(forward_substitution(w.Linv, naux, naux, w.L, naux, w.subst, s));
+    DF_TRY(check_tc_errors((const int*)w.subst, 1, "df_fit_residual", s));
     DF_TRY(dgemm(true, false, naux, (int)ld, naux, 1.0, w.Linv, naux, 0, w.T, ld, 0, 0.0, w.C, ld, 0, 1, s, 0, 0));
     dim3 g3((unsigned)((ld + 255) / 256), (unsigned)naux);
     int3c_dexp_kernel<<<g3, 256, 0, s>>>(pp, px, py, pz, pk, npair, ld, aux_xyz, aux_exp, w.dv);

@@ -402,6 +402,9 @@ JKWork jk_work_layout(int nao, int naux, int nocc, int precision, Arena* a, Size
   w.nsplit_j = nsplit_j;
 #define TAKE(T, ptr, count) \
   if (a) ptr = a->take<T>(count); else z->take<T>(count);
+  TAKE(int, w.err, 2);
+  w.fk.err = w.err;
+  w.mk.err = w.err + 1;
   TAKE(double, w.Dw, ld);
   TAKE(double, w.d, naux);
   TAKE(double, w.Jpart, (size_t)nsplit_j * ld);
@@ -413,7 +416,6 @@ JKWork jk_work_layout(int nao, int naux, int nocc, int precision, Arena* a, Size
     TAKE(char, w.fk.Xd, digit_operand_bytes(nao, (long)w.fk.px * oc));
     TAKE(double, w.fk.X, (size_t)nao * w.fk.px * oc);
     TAKE(double, w.fk.Kpart, (size_t)w.fk.nsplit * nao * nao);
-    TAKE(int, w.fk.err, 1);
   }
   if (precision == DF_MIXED) mixed_k_work_layout(nao, naux, nocc, a, z, &w.mk);
 #undef TAKE
@@ -476,7 +478,6 @@ int build_J(const void* Bbuf, const BLayout& L, int nao, int naux, int precision
 
 int build_K_fp64(const double* B64, long ld, int nao, int naux, const double* C, int nocc, double* K,
                  const Fp64KWork& w, cudaStream_t s) {
-  DF_CUDA(cudaMemsetAsync(w.err, 0, sizeof(int), s));
   const DigitOperand ct = digit_operand(w.Ct, nocc, nao);
   DF_TRY(slice_matrix(C, nocc, true, ct, s));
   for (int x0 = 0; x0 < naux; x0 += w.px) {
@@ -577,8 +578,9 @@ extern "C" int df_build_B(const double* ao_xyz, const double* ao_exp, int nao, c
              "df_build_B: workspace of %zu bytes < %zu", work_bytes, df_build_B_work_bytes(nao, naux));
   DF_REQUIRE(precision == DF_FP64 || naux <= 65535, DF_ERR_ARG, "df_build_B: naux > 65535 in mixed mode");
   work = aligned_work(work);
-  return build_B(ao_xyz, ao_exp, nao, aux_xyz, aux_exp, naux, L, precision, B, (double*)work,
-                 (char*)work + align_up(sizeof(double) * pair_tab_doubles(nao), 256), s);
+  char* subst = (char*)work + align_up(sizeof(double) * pair_tab_doubles(nao), 256);
+  DF_TRY(build_B(ao_xyz, ao_exp, nao, aux_xyz, aux_exp, naux, L, precision, B, (double*)work, subst, s));
+  return check_tc_errors((const int*)subst, 1, "df_build_B", s);
 }
 
 extern "C" int df_B_get_packed(const void* B, int nao, int naux, int P, double* row, cudaStream_t s) {
@@ -610,20 +612,9 @@ extern "C" int df_jk(const void* B, int nao, int naux, int precision, const doub
   Arena a(work, work_bytes);
   JKWork w = jk_work_layout(nao, naux, nocc, precision, &a, nullptr, false);
   DF_REQUIRE(!a.overflow, DF_ERR_NOMEM, "df_jk: workspace overflow");
+  if (K) DF_TRY(reset_tc_errors(w.err, 2, TC_EXCHANGE, s));
   DF_TRY(run_jk(B, nao, naux, precision, D, C, nocc, J, K, w, s));
-  if (K && precision == DF_MIXED) {
-    // The tensor-core kernels flag a bounded wait that gave up (K is then NaN).  Outside a
-    // stream capture the flag is read back here, which synchronises the stream.
-    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-    DF_CUDA(cudaStreamIsCapturing(s, &cs));
-    if (cs == cudaStreamCaptureStatusNone) {
-      int err = 0;
-      DF_CUDA(cudaMemcpyAsync(&err, w.mk.err, sizeof(int), cudaMemcpyDeviceToHost, s));
-      DF_CUDA(cudaStreamSynchronize(s));
-      DF_REQUIRE(err == 0, DF_ERR_TIMEOUT, "df_jk: a bounded wait of the tensor-core exchange gave up; K is NaN");
-    }
-  }
-  return DF_OK;
+  return K ? check_tc_errors(w.err, 2, "df_jk", s) : DF_OK;
 }
 
 DF_BOUNDS_READER(bounds_read_jk)

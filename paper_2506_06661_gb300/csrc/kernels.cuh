@@ -38,6 +38,14 @@ int cholesky_inplace(double* A, int n, int* d_status, double* d_maxdiag, double 
 size_t forward_substitution_bytes(long ncol, int naux);
 int forward_substitution(double* R, long ld, long ncol, const double* L, int naux, void* work, cudaStream_t s);
 
+// Error words of the tensor-core kernels (digit products, split-BF16 GEMMs): a bounded wait that
+// gives up raises its word, and every later launch with that word skips its work.  reset before the
+// launches of a call; check reads them back (synchronising; not inside a stream capture) and
+// returns DF_ERR_TIMEOUT.  cholesky_inplace and forward_substitution keep theirs at the start of work.
+enum TcUser { TC_SETUP = 1, TC_EXCHANGE = 2 };  // values of the test hook "tc_give_up"
+int reset_tc_errors(int* err, int n, TcUser user, cudaStream_t s);
+int check_tc_errors(const int* err, int n, const char* who, cudaStream_t s);
+
 // ---- eigensolver (eig.cu) ------------------------------------------------------------
 size_t eigh_scratch_doubles(int n);
 int eigh_rows(double* A, int n, double* w, double* ZT, double* scratch, int* status, cudaStream_t s);
@@ -90,6 +98,7 @@ struct Fp64KWork {
 };
 
 struct JKWork {
+  int* err;  // error words of the FP64 and of the mixed exchange (reset_tc_errors before run_jk)
   double* Dw;
   double* d;
   double* Jpart;

@@ -301,7 +301,7 @@ size_t cholesky_bytes(int n) { return 256 + (n > CH_NB ? digit_operand_bytes(n, 
 
 int cholesky_inplace(double* A, int n, int* d_status, double* d_maxdiag, double tol, void* work, cudaStream_t s) {
   int* err = (int*)work;
-  DF_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
+  DF_TRY(reset_tc_errors(err, 1, TC_SETUP, s));
   chol_init_kernel<<<1, 1024, 0, s>>>(A, n, d_maxdiag, d_status);
   DF_LAUNCHED("chol_init_kernel");
   for (int k0 = 0; k0 < n; k0 += CH_NB) {
@@ -404,7 +404,7 @@ int forward_substitution(double* R, long ld, long ncol, const double* L, int nau
   char* xmem = (char*)work + 256;
   char* lmem = xmem + digit_operand_bytes(cmax, FS_NBO);
   int* err = (int*)work;
-  if (naux > FS_NB) DF_CUDA(cudaMemsetAsync(err, 0, sizeof(int), s));
+  DF_TRY(reset_tc_errors(err, 1, TC_SETUP, s));
   // R[r0.., :] -= L[r0.., k0..k0+b) R[k0..k0+b, :] over nr rows and the columns of chunk c0 (digits
   // of R's rows k0.. in x)
   auto update = [&](int r0, int nr, int k0, int b, long c0, const DigitOperand& x, const DigitOperand& l) -> int {
@@ -470,11 +470,11 @@ extern "C" int df_metric_chol(const double* aux_xyz, const double* aux_exp, int 
   double* d_maxdiag = (double*)((char*)work + 256);
   DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, L, (double*)((char*)work + 512), s));
   if (M_out) DF_CUDA(cudaMemcpyAsync(M_out, L, sizeof(double) * naux * naux, cudaMemcpyDeviceToDevice, s));
-  DF_TRY(cholesky_inplace(L, naux, d_status, d_maxdiag, 1e-14,
-                          (char*)work + 512 + sizeof(double) * align_up(boys_table_doubles(), 32), s));
+  void* chol = (char*)work + 512 + sizeof(double) * align_up(boys_table_doubles(), 32);
+  DF_TRY(cholesky_inplace(L, naux, d_status, d_maxdiag, 1e-14, chol, s));
   int h_status = -1;
   DF_CUDA(cudaMemcpyAsync(&h_status, d_status, sizeof(int), cudaMemcpyDeviceToHost, s));
-  DF_CUDA(cudaStreamSynchronize(s));
+  DF_TRY(check_tc_errors((const int*)chol, 1, "df_metric_chol", s));  // (synchronises) before the pivot, which it may spoil
   if (h_status >= 0) {
     *bad_pivot = h_status;
     set_error("df_metric_chol: metric not positive definite at pivot %d", h_status);

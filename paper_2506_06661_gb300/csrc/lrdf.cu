@@ -199,13 +199,13 @@ extern "C" int df_lrdf_build(const double* ao_xyz, const double* ao_exp, int nao
   DF_TRY(cholesky_inplace(L, naux, status, maxdiag, 1e-14, subst, s));
   int h = -1;
   DF_CUDA(cudaMemcpyAsync(&h, status, sizeof(int), cudaMemcpyDeviceToHost, s));
-  DF_CUDA(cudaStreamSynchronize(s));
+  DF_TRY(check_tc_errors((const int*)subst, 1, "df_lrdf_build", s));
   DF_REQUIRE(h < 0, DF_ERR_NOT_SPD, "df_lrdf_build: long-range metric not positive definite at pivot %d", h);
   const long ld = B_ld(nao);
   double* B64 = (double*)B;
   DF_TRY(launch_int3c(ao_xyz, ao_exp, nao, aux_xyz, aux_exp, naux, B64, ld, pair_tab, s, omega));
   DF_TRY(forward_substitution(B64, ld, ld, L, naux, subst, s));
-  return DF_OK;
+  return check_tc_errors((const int*)subst, 1, "df_lrdf_build", s);
 }
 
 extern "C" size_t df_lrdf_jk_work_bytes(int nao, int naux, int nocc) {

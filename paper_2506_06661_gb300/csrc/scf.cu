@@ -279,14 +279,14 @@ __global__ void occ_columns_kernel(const double* __restrict__ ZT, int nmo, int n
 }
 
 // HOMO / LUMO of the last diagonalisation, its eigensolver status and the tensor-core
-// exchange's timeout flag (tc_err may be null: an FP64 iteration) into the status block.
+// exchange's error words of this iteration into the status block.
 __global__ void orbital_status_kernel(const double* __restrict__ eps, int nmo, int nocc, const int* eig_status,
                                       const int* tc_err, ScfStatus* st) {
   if (threadIdx.x != 0) return;
   st->homo = nocc > 0 ? eps[nocc - 1] : 0.0;
   st->lumo = nocc < nmo ? eps[nocc] : 0.0;
   st->eig_fail = *eig_status;
-  st->tc_timeout = tc_err ? *tc_err : 0;
+  st->tc_timeout = tc_err[0] | tc_err[1];
 }
 
 __global__ void axpy_kernel(double* __restrict__ y, const double* __restrict__ x, long n, double a) {
@@ -582,7 +582,7 @@ __global__ void soscf_status_kernel(const double* __restrict__ Fmo, int nmo, int
   st->homo = homo;
   st->lumo = nocc < nmo ? lumo : 0.0;
   st->eig_fail = *k_status;
-  st->tc_timeout = tc_err ? *tc_err : 0;
+  st->tc_timeout = tc_err[0] | tc_err[1];
 }
 
 static unsigned blocks_for(long n, int t = 256) { return (unsigned)((n + t - 1) / t); }
@@ -807,7 +807,8 @@ struct ScfMol {
   enum Phase { SETUP, GUESS_CHECK, READY, DM0_EIG, ITER, STAB, DONE } phase = SETUP;
   bool outputs_done = false;  // outputs already written for the current solution
   double* h_eps = nullptr;  // pinned: eigenvalues of S, then E_nuc (nao + 1 doubles); then of dm0
-  int* h_ints = nullptr;    // pinned: [0] eigensolver status, [1] Cholesky status
+  int* h_ints = nullptr;    // pinned: [0] eigensolver status, [1] Cholesky status, [2, 3] error words of the
+                            // tensor-core kernels (metric and B; then the stability analysis)
   double* h_dav = nullptr;  // pinned: read-backs of the stability analysis
   DavState dav;
   std::vector<int> dm0_ids; // eigenvalue indices of the dm0 split (source of an async copy)
@@ -834,8 +835,10 @@ static int setup_launch(ScfMol& M) {
   DF_TRY(launch_enuc(mol->xyz, mol->charges, mol->natm, W.enuc, s));
   DF_TRY(launch_int2c(mol->aux_xyz, mol->aux_exp, naux, W.L, pair_tab_boys(W.pair_tab, nao), s));
   DF_TRY(cholesky_inplace(W.L, naux, W.chol_status, W.maxdiag, 1e-14, W.subst, s));
+  DF_CUDA(cudaMemcpyAsync(M.h_ints + 2, W.subst, sizeof(int), cudaMemcpyDeviceToHost, s));  // its error word
   DF_TRY(build_B(mol->ao_xyz, mol->ao_exp, nao, mol->aux_xyz, mol->aux_exp, naux, W.L, M.opt.precision, W.B,
                  W.pair_tab, W.subst, s));
+  DF_CUDA(cudaMemcpyAsync(M.h_ints + 3, W.subst, sizeof(int), cudaMemcpyDeviceToHost, s));
   DF_CUDA(cudaMemcpyAsync(W.T1, W.S, sizeof(double) * nn, cudaMemcpyDeviceToDevice, s));
   DF_TRY(eig_rows(W.T1, nao, W.eps, W.ZT, W, s));
   DF_CUDA(cudaMemcpyAsync(M.h_eps, W.eps, sizeof(double) * nao, cudaMemcpyDeviceToHost, s));
@@ -920,6 +923,8 @@ static int setup_orthogonalize(ScfMol& M) {
   const int nao = M.nao, nocc = M.nocc;
   const long nn = (long)nao * nao;
   M.res.e_nuc = M.h_eps[nao];
+  DF_REQUIRE(!(M.h_ints[2] | M.h_ints[3]), DF_ERR_TIMEOUT,
+             "scf: a bounded wait of the tensor-core kernels gave up in the metric or in B");
   DF_REQUIRE(M.h_ints[1] < 0, DF_ERR_NOT_SPD, "scf: auxiliary metric not positive definite at pivot %d", M.h_ints[1]);
   DF_REQUIRE(M.h_ints[0] != 3, DF_ERR_TIMEOUT, "scf: a grid barrier of the eigensolver timed out on S");
   DF_REQUIRE(M.h_ints[0] == 0, DF_ERR_NOCONV, "scf: eigensolver failed on S");
@@ -990,6 +995,7 @@ static int dm0_launch(ScfMol& M) {
   const int nao = M.nao;
   const long nn = (long)nao * nao;
   DF_CUDA(cudaMemcpyAsync(W.Dprev, W.D, sizeof(double) * nn, cudaMemcpyDeviceToDevice, s));
+  DF_TRY(reset_tc_errors(W.jk.err, 2, TC_EXCHANGE, s));
   DF_TRY(run_jk(W.B, nao, M.naux, M.prec, W.D, nullptr, 0, W.J, nullptr, W.jk, s));
   DF_CUDA(cudaMemcpyAsync(W.T1, W.D, sizeof(double) * nn, cudaMemcpyDeviceToDevice, s));
   DF_TRY(eig_rows(W.T1, nao, W.eps, W.ZT, W, s));
@@ -1422,6 +1428,7 @@ static int dav_products(ScfMol& M) {
   DF_CUDA(cudaMemcpyAsync(M.h_dav + at, p.G + at, sizeof(double) * rows, cudaMemcpyDeviceToHost, M.s));
   DF_CUDA(cudaMemcpyAsync(M.h_dav + kDavidsonMax * kDavidsonMax, p.misc, 2 * sizeof(double), cudaMemcpyDeviceToHost,
                           M.s));
+  DF_CUDA(cudaMemcpyAsync(M.h_ints + 2, M.W.jk.err, sizeof(int) * 2, cudaMemcpyDeviceToHost, M.s));
   d.stage = DavState::RITZ;
   return DF_OK;
 }
@@ -1497,6 +1504,8 @@ static int dav_advance(ScfMol& M, bool* finished) {
     *finished = true;
     return DF_OK;
   }
+  DF_REQUIRE(!(M.h_ints[2] | M.h_ints[3]), DF_ERR_TIMEOUT,
+             "scf: a bounded wait of the tensor-core exchange gave up in the stability analysis");
   const double* hG = M.h_dav;
   const double rr_prev = M.h_dav[kDavidsonMax * kDavidsonMax];      // |r|^2 of the previous Ritz pair
   const double n2 = M.h_dav[kDavidsonMax * kDavidsonMax + 1];       // |t|^2 of the newest vector
@@ -1611,7 +1620,7 @@ static int escape_saddle(ScfMol& M) {
 
 // Everything after J and K: Fock, energy, DIIS error and extrapolation, diagonalisation,
 // status readback.  No host decisions: capturable.
-static int iteration_tail(ScfMol& M, int prec) {
+static int iteration_tail(ScfMol& M) {
   ScfWork& W = M.W;
   cudaStream_t s = M.s;
   const int nao = M.nao, nmo = M.nmo, nocc = M.nocc;
@@ -1659,8 +1668,7 @@ static int iteration_tail(ScfMol& M, int prec) {
   if (M.soscf_on) DF_CUDA(cudaMemcpyAsync(W.Fbar, W.Fp, sizeof(double) * ne, cudaMemcpyDeviceToDevice, s));
   DF_TRY(diagonalize_orth(nao, nmo, nocc, W, s));
   if (M.inc) DF_TRY(incremental_prep(M));
-  orbital_status_kernel<<<1, 32, 0, s>>>(W.eps, nmo, nocc, W.eig_status, prec == DF_MIXED ? W.jk.mk.err : nullptr,
-                                         W.st);
+  orbital_status_kernel<<<1, 32, 0, s>>>(W.eps, nmo, nocc, W.eig_status, W.jk.err, W.st);
   DF_LAUNCHED("orbital_status_kernel");
   DF_CUDA(cudaMemcpyAsync(M.hst, W.st, sizeof(ScfStatus), cudaMemcpyDeviceToHost, s));
   return DF_OK;
@@ -1669,7 +1677,7 @@ static int iteration_tail(ScfMol& M, int prec) {
 // Tail of a Newton iteration: Fock and energy, the orthogonal-basis error of the density
 // that was built (for the convergence test), then a Newton step instead of DIIS and the
 // diagonalisation.
-static int iteration_tail_soscf(ScfMol& M, int prec) {
+static int iteration_tail_soscf(ScfMol& M) {
   ScfWork& W = M.W;
   cudaStream_t s = M.s;
   const int nao = M.nao, nmo = M.nmo, nocc = M.nocc;
@@ -1685,7 +1693,7 @@ static int iteration_tail_soscf(ScfMol& M, int prec) {
   DF_LAUNCHED("absmax_kernel");
   DF_TRY(soscf_step(M));
   if (M.inc) DF_TRY(incremental_prep(M));
-  soscf_status_kernel<<<1, 32, 0, s>>>(W.Fmo, nmo, nocc, W.k_status, prec == DF_MIXED ? W.jk.mk.err : nullptr, W.st);
+  soscf_status_kernel<<<1, 32, 0, s>>>(W.Fmo, nmo, nocc, W.k_status, W.jk.err, W.st);
   DF_LAUNCHED("soscf_status_kernel");
   DF_CUDA(cudaMemcpyAsync(M.hst, W.st, sizeof(ScfStatus), cudaMemcpyDeviceToHost, s));
   return DF_OK;
@@ -1697,10 +1705,11 @@ static int iteration_body(ScfMol& M, int prec) {
   const long nn = (long)M.nao * M.nao;
   DF_CUDA(cudaMemcpyAsync(W.Dprev, W.D, sizeof(double) * nn, cudaMemcpyDeviceToDevice, M.s));
   DF_CUDA(cudaMemcpyAsync(W.Cprev, W.Cocc, sizeof(double) * M.nao * M.nocc, cudaMemcpyDeviceToDevice, M.s));
+  DF_TRY(reset_tc_errors(W.jk.err, 2, TC_EXCHANGE, M.s));
   DF_TRY(run_jk(W.B, M.nao, M.naux, prec, W.D, W.Cocc, M.nocc, W.J, W.K, W.jk, M.s));
   if (M.inc)  // a full build: the accumulated K now belongs to this density
     DF_CUDA(cudaMemcpyAsync(W.Cbase, W.Cp, sizeof(double) * M.nmo * M.nocc, cudaMemcpyDeviceToDevice, M.s));
-  return M.soscf ? iteration_tail_soscf(M, prec) : iteration_tail(M, prec);
+  return M.soscf ? iteration_tail_soscf(M) : iteration_tail(M);
 }
 
 // Body of an incremental iteration: J in FP64 as always; K += K[U+] - K[U-] with the
@@ -1713,6 +1722,7 @@ static int iteration_body_incremental(ScfMol& M) {
   const long nn = (long)nao * nao;
   DF_CUDA(cudaMemcpyAsync(W.Dprev, W.D, sizeof(double) * nn, cudaMemcpyDeviceToDevice, s));
   DF_CUDA(cudaMemcpyAsync(W.Cprev, W.Cocc, sizeof(double) * nao * nocc, cudaMemcpyDeviceToDevice, s));
+  DF_TRY(reset_tc_errors(W.jk.err, 2, TC_EXCHANGE, s));
   DF_TRY(run_jk(W.B, nao, M.naux, DF_MIXED, W.D, nullptr, 0, W.J, nullptr, W.jk, s));
   {
     ProfScope ps("scf_incremental_factors", s);
@@ -1730,13 +1740,13 @@ static int iteration_body_incremental(ScfMol& M) {
   kacc_kernel<<<blocks_for(nn), 256, 0, s>>>(W.K, W.T2, W.T1, nn);
   DF_LAUNCHED("kacc_kernel");
   DF_CUDA(cudaMemcpyAsync(W.Cbase, W.Cp, sizeof(double) * nmo * nocc, cudaMemcpyDeviceToDevice, s));
-  return M.soscf ? iteration_tail_soscf(M, DF_MIXED) : iteration_tail(M, DF_MIXED);
+  return M.soscf ? iteration_tail_soscf(M) : iteration_tail(M);
 }
 
 // Second half of the first iteration from a non-idempotent dm0 (after dm0_launch drained).
 static int scf_dm0_finish(ScfMol& M) {
   DF_TRY(dm0_finish(M));
-  DF_TRY(iteration_tail(M, M.prec));
+  DF_TRY(iteration_tail(M));
   M.first_dm0 = false;
   return DF_OK;
 }
@@ -1882,14 +1892,14 @@ static bool scf_iter_finish(ScfMol& M) {
   const ScfStatus& h = *M.hst;
   M.res.iterations++;
   if (M.prec == DF_FP64) M.res.fp64_iterations++;
+  if (h.tc_timeout) {  // first: the K it left is NaN
+    M.rc = DF_ERR_TIMEOUT;
+    set_error("scf: a bounded wait of the tensor-core exchange gave up at iteration %d", M.res.iterations);
+    return true;
+  }
   if (h.nonfinite || !std::isfinite(h.emax)) {
     M.rc = DF_ERR_NUMERIC;
     set_error("scf: non-finite Fock matrix at iteration %d", M.res.iterations);
-    return true;
-  }
-  if (h.tc_timeout) {
-    M.rc = DF_ERR_TIMEOUT;
-    set_error("scf: a bounded wait of the tensor-core exchange gave up at iteration %d", M.res.iterations);
     return true;
   }
   if (h.eig_fail == 3) {
@@ -2088,7 +2098,7 @@ int scf_run_on(const df_molecule* mol, const scf_opts& o, const double* dm0, dou
   int* hints = nullptr;
   DF_CUDA(cudaMallocHost(&hst, sizeof(ScfStatus)));
   DF_CUDA(cudaMallocHost(&heps, sizeof(double) * (mol->nao + 1)));
-  DF_CUDA(cudaMallocHost(&hints, sizeof(int) * 2));
+  DF_CUDA(cudaMallocHost(&hints, sizeof(int) * 4));
   double* hdav = nullptr;
   DF_CUDA(cudaMallocHost(&hdav, sizeof(double) * kDavHost));
   M.h_dav = hdav;
@@ -2228,7 +2238,7 @@ extern "C" int scf_run_batch(const df_molecule* mols, int nmol, const scf_opts* 
   int* hints = nullptr;
   DF_CUDA(cudaMallocHost(&hst, sizeof(ScfStatus) * slots));
   DF_CUDA(cudaMallocHost(&heps, sizeof(double) * (size_t)(max_nao + 1) * slots));
-  DF_CUDA(cudaMallocHost(&hints, sizeof(int) * 2 * slots));
+  DF_CUDA(cudaMallocHost(&hints, sizeof(int) * 4 * slots));
   double* hdav = nullptr;
   DF_CUDA(cudaMallocHost(&hdav, sizeof(double) * kDavHost * slots));
   std::vector<ScfMol*> slot_mol(slots, nullptr);
@@ -2257,7 +2267,7 @@ extern "C" int scf_run_batch(const df_molecule* mols, int nmol, const scf_opts* 
     if (slots > 1) M->W.eig_aux = nullptr;
     M->hst = hst + k;
     M->h_eps = heps + (size_t)(max_nao + 1) * k;
-    M->h_ints = hints + 2 * k;
+    M->h_ints = hints + 4 * k;
     M->h_dav = hdav + (size_t)kDavHost * k;
     M->dm0 = dm0s ? dm0s[i] : nullptr;
     M->D_out = D_outs ? D_outs[i] : nullptr;

@@ -687,10 +687,8 @@ void mixed_k_work_layout(int nao, int naux, int nocc, Arena* a, Sizer* z, MixedK
   }
   if (a) {
     w->Kpart = a->take<float>((size_t)nsplit * npad * npad);
-    w->err = a->take<int>(1);
   } else {
     z->take<float>((size_t)nsplit * npad * npad);
-    z->take<int>(1);
   }
 }
 
@@ -700,7 +698,6 @@ int build_K_mixed(const void* B, const BLayout& L, int nao, int naux, const doub
   DF_REQUIRE(nocc <= ncpad, DF_ERR_ARG, "mixed K: workspace sized for %d occupied columns, got %d", ncpad, nocc);
   DF_REQUIRE(ncpad <= 256, DF_ERR_ARG, "mixed K: more than 256 occupied orbitals per call is not supported");
   DF_REQUIRE(NP >= 3 && NP <= 5, DF_ERR_ARG, "mixed K: %d planes", NP);
-  DF_CUDA(cudaMemsetAsync(w.err, 0, sizeof(int), s));
   DF_CUDA(cudaMemsetAsync(w.xmax, 0, sizeof(unsigned) * (size_t)npad, s));
   PlanePtrs cpp{}, xpp{};
   for (int j = 0; j < NP; ++j) {
