@@ -445,7 +445,8 @@ int df_j_noalloc(const void* B, int nao, int naux, const double* D, double* J, c
  * eigensolver: 0 automatic, 1 a single CTA) and "mixed_planes" (3..5 BF16 planes per operand of
  * the mixed exchange: 6, 10 or 15 plane products; it also sizes a mixed B).
  * Tile shapes: "fp64_ht_cols" (0 automatic, 16 or 32 occupied columns per column group of the FP64
- * half-transform), "ht_n" (0: the widest tcgen05 half-transform tile that fits; else a cap, a multiple
+ * half-transform), "fp64_k_pb" and "fp64_k_px" (0 automatic, else auxiliary rows per half-transform and per
+ * SYRK launch of the FP64 exchange), "ht_n" (0: the widest tcgen05 half-transform tile that fits; else a cap, a multiple
  * of 16), "jpass1_rows" (1, 2, 4 or 8 auxiliary rows per CTA of J's first pass) and
  * "j_fp64_fma" (1: J's passes with FP64 FMAs instead of double-float products).
  * "mixed_incremental" (0 or 1), "soscf" (0 or 1) and "soscf_cg" (1..64) shape the SCF as

@@ -130,6 +130,8 @@ static Knob g_knobs[] = {
     {"syrk_split", 0, 0, 4096},      // K-dimension splits of the tcgen05 exchange SYRK
     {"syrk_pair", 0, 0, 1},          // exchange SYRK on CTA pairs (cta_group::2, 256 x 128 blocks); 0: one CTA per 128 x 128 tile
     {"fp64_syrk_split", 0, 0, 4096}, // K-dimension splits of the FP64 exchange SYRK
+    {"fp64_k_pb", 0, 0, 65535},      // auxiliary rows per half-transform launch of the FP64 exchange (0 auto)
+    {"fp64_k_px", 0, 0, 65535},      // auxiliary rows per SYRK launch of the FP64 exchange (0 auto)
     {"jpass2_rows", 256, 32, 512},   // auxiliary rows per CTA slice of J's second pass
     {"j_fp64_fma", 0, 0, 1},         // J passes: 0 double-float products on FP32 units, 1 FP64 FMAs
     {"jpass1_rows", 1, 1, 8},        // auxiliary rows per CTA of J's first pass (1, 2, 4 or 8)

@@ -362,16 +362,25 @@ __global__ void ksum_mirror_kernel(const double* __restrict__ Kpart, int nsplit,
   K[(size_t)n * nao + m] = s;
 }
 
-// Block sizes of the FP64 exchange.  Each half-transform launch should fill the GPU for a few
-// waves of 128-row tiles (pb), within 512 MB of B digits; each SYRK launch should have a long K
-// (px), within 1 GB of X and its digits.
+// Block sizes of the FP64 exchange.  Each half-transform launch should fill the GPU for whole waves
+// of 128-row tiles (pb), and each SYRK launch should have a long K (px), within 1 GB of X and its
+// digits and within 64 splits of 4096 stages.  The digits of a wave's rows of B take more than B itself in small
+// molecules, and every molecule of a batch holds them: two waves where they fit in 5/4 of B, else
+// one.  Four waves, two, one (MB of workspace, ms): 20 centres 52, 52, 37 MB, 0.18, 0.18, 0.19 ms;
+// 40 centres 280, 170, 116 MB, 0.61, 0.63, 0.67 ms; 63 centres 566, 389, 302 MB, 1.64, 1.70, 1.85
+// ms; 100 centres 1399, 1134, 997 MB, 7.9, 8.1, 8.0 ms; 200 centres 2164, 1605, 1381 MB, 66.7,
+// 69.4, 72.7 ms.
 static void fp64_k_blocks(int nao, int naux, int nocc, Fp64KWork* w) {
   const long coltiles = (nocc + 63) / 64;
-  const long rows = 4L * 152 * digits::BM / coltiles;
   const size_t bytes_b = digits::plane_bytes(nao, nao), bytes_x = (size_t)nao * nocc * (2 * digits::NS + 8);
-  long pb = std::min((rows + nao - 1) / nao, std::max(1L, (long)((512ul << 20) / bytes_b)));
-  pb = std::max(1L, std::min(pb, (long)naux));
+  const size_t bytes_B = sizeof(double) * (size_t)B_ld(nao) * naux;
+  auto waves = [&](long n) { return std::max(1L, std::min(n * 152 * digits::BM / coltiles / nao, (long)naux)); };
+  long pb = waves(2);
+  if ((size_t)pb * bytes_b > bytes_B / 4 * 5 || (size_t)pb * bytes_b > (640ul << 20)) pb = waves(1);
+  if (knob("fp64_k_pb") > 0) pb = std::min(knob("fp64_k_pb"), naux);
   long px = std::max(pb, (long)((1ul << 30) / bytes_x) / pb * pb);
+  px = std::min(px, std::max(1L, 64L * 4096 * digits::BK / nocc));
+  if (knob("fp64_k_px") > 0) px = std::max(pb, (long)knob("fp64_k_px"));
   w->pb = (int)pb;
   w->px = (int)std::min(px, (long)naux);
   // splits of the SYRK's K range: least waves x (stages + the cost of a tile's start and end)
@@ -392,9 +401,22 @@ static void fp64_k_blocks(int nao, int naux, int nocc, Fp64KWork* w) {
   if (forced > 0) w->nsplit = (int)std::max((nst + 4095) / 4096, std::min((long)forced, std::max(1L, nst / 2)));
 }
 
-// fp64_k: also carve the FP64 exchange buffers when precision is DF_MIXED (an SCF that
-// switches from mixed to FP64 iterations needs both).
-JKWork jk_work_layout(int nao, int naux, int nocc, int precision, Arena* a, Sizer* z, bool fp64_k) {
+static void fp64_k_work_layout(int nao, int naux, int nocc, Arena* a, Sizer* z, Fp64KWork* w) {
+  fp64_k_blocks(nao, naux, nocc, w);
+#define TAKE(T, ptr, count) \
+  if (a) ptr = a->take<T>(count); else z->take<T>(count);
+  TAKE(char, w->Ct, digit_operand_bytes(nocc, nao));
+  TAKE(char, w->Bp, digit_operand_bytes((long)w->pb * nao, nao));
+  TAKE(char, w->Xd, digit_operand_bytes(nao, (long)w->px * nocc));
+  TAKE(double, w->X, (size_t)nao * w->px * nocc);
+  TAKE(double, w->Kpart, (size_t)w->nsplit * nao * nao);
+#undef TAKE
+}
+
+// fp64_k: also lay out the FP64 exchange buffers when precision is DF_MIXED (an SCF that
+// switches from mixed to FP64 iterations needs both).  shared: bytes of scratch that the caller
+// needs only between K builds.  All of it is one region: nothing there outlives a build.
+JKWork jk_work_layout(int nao, int naux, int nocc, int precision, Arena* a, Sizer* z, bool fp64_k, size_t shared) {
   JKWork w{};
   long ld = B_ld(nao);
   int rows = max(32, min(JP2_MAX_ROWS, knob("jpass2_rows")));
@@ -408,17 +430,18 @@ JKWork jk_work_layout(int nao, int naux, int nocc, int precision, Arena* a, Size
   TAKE(double, w.Dw, ld);
   TAKE(double, w.d, naux);
   TAKE(double, w.Jpart, (size_t)nsplit_j * ld);
-  if (precision == DF_FP64 || fp64_k) {
-    const int oc = max(nocc, 1);
-    fp64_k_blocks(nao, naux, oc, &w.fk);
-    TAKE(char, w.fk.Ct, digit_operand_bytes(oc, nao));
-    TAKE(char, w.fk.Bp, digit_operand_bytes((long)w.fk.pb * nao, nao));
-    TAKE(char, w.fk.Xd, digit_operand_bytes(nao, (long)w.fk.px * oc));
-    TAKE(double, w.fk.X, (size_t)nao * w.fk.px * oc);
-    TAKE(double, w.fk.Kpart, (size_t)w.fk.nsplit * nao * nao);
-  }
-  if (precision == DF_MIXED) mixed_k_work_layout(nao, naux, nocc, a, z, &w.mk);
+  const bool f = nocc > 0 && (precision == DF_FP64 || fp64_k), m = precision == DF_MIXED;
+  Sizer zf{0}, zm{0};
+  if (f) fp64_k_work_layout(nao, naux, nocc, nullptr, &zf, &w.fk);
+  if (m) mixed_k_work_layout(nao, naux, nocc, nullptr, &zm, &w.mk);
+  const size_t bytes = std::max(std::max(zf.used, zm.used), shared);
+  if (bytes) TAKE(char, w.scratch, bytes);
 #undef TAKE
+  if (w.scratch) {
+    Arena af(w.scratch, bytes), am(w.scratch, bytes);
+    if (f) fp64_k_work_layout(nao, naux, nocc, &af, nullptr, &w.fk);
+    if (m) mixed_k_work_layout(nao, naux, nocc, &am, nullptr, &w.mk);
+  }
   return w;
 }
 

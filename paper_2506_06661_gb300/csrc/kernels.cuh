@@ -103,6 +103,7 @@ struct JKWork {
   double* d;
   double* Jpart;
   int nsplit_j;
+  char* scratch;  // the region of fk, of mk and of the caller's shared scratch
   Fp64KWork fk;
   MixedKWork mk;
 };
@@ -117,7 +118,7 @@ int mixed_planes();
 // checked before an exchange reads the planes; -1 if the address was never recorded.
 void record_B_planes(const void* B, int planes);
 int recorded_B_planes(const void* B);
-JKWork jk_work_layout(int nao, int naux, int nocc, int precision, Arena* a, Sizer* z, bool fp64_k);
+JKWork jk_work_layout(int nao, int naux, int nocc, int precision, Arena* a, Sizer* z, bool fp64_k, size_t shared = 0);
 int umma_prepare();
 void mixed_k_work_layout(int nao, int naux, int nocc, Arena* a, Sizer* z, MixedKWork* w);
 int build_K_mixed(const void* B, const BLayout& L, int nao, int naux, const double* C, int nocc, double* K,

@@ -624,7 +624,6 @@ static void scf_layout(int nao, int naux, int nocc, int precision, Arena* a, Siz
   w->guess_ws = nullptr;
   if (w->guess_bytes) TAKE(char, w->guess_ws, w->guess_bytes);
   TAKE(double, w->pair_tab, pair_tab_doubles(nao));
-  TAKE(char, w->subst, forward_substitution_bytes(B_ld(nao), naux));
   TAKE(double, w->S, nn);
   TAKE(double, w->h, nn);
   TAKE(double, w->V, nn);
@@ -708,7 +707,9 @@ static void scf_layout(int nao, int naux, int nocc, int precision, Arena* a, Siz
   TAKE(DiisState, w->diis, 1);
   if (a) w->B = a->take<char>(df_B_bytes(nao, naux, precision)); else z->take<char>(df_B_bytes(nao, naux, precision));
 #undef TAKE
-  w->jk = jk_work_layout(nao, naux, nocc, precision, a, z, true);
+  // the whitening is done before the first exchange build
+  w->jk = jk_work_layout(nao, naux, nocc, precision, a, z, true, forward_substitution_bytes(B_ld(nao), naux));
+  w->subst = w->jk.scratch;
 }
 
 static int eig_rows(double* A, int n, double* w, double* ZT, ScfWork& W, cudaStream_t s) {
