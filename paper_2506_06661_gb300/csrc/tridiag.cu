@@ -30,7 +30,7 @@ namespace dfscf {
 
 namespace {
 constexpr int HALF = 128;  // threads that work on the rows, and as many on the reflector
-constexpr size_t kSmemLimit = 226 * 1024;
+constexpr size_t kSmemLimit = 227 * 1024 - 160;  // beside the kernel's static shared memory
 
 constexpr unsigned kTopTag = 0x3fffffffu;  // tag of the exchange before the first step
 
@@ -162,25 +162,28 @@ __device__ __forceinline__ void all_rows(double* rows, int n, int s0, int s1, in
 #undef DF_PASS
 }
 
-// Dynamic shared memory: x, vb (two), wt, cn [n], R rows of n, red [4][R], cnew [R].  NC: columns
-// per thread whose packets are in flight together.
+// Dynamic shared memory: x, vb (two), wt, cn [n], R rows of n, red [4][R], cnew [R].  With vbs = 1
+// there is one vb and red and cnew lie in cn: the reflector half then waits for the pass over the
+// rows before it writes vb, and the row half for itself before it writes cn.  NC: columns per thread
+// whose packets are in flight together.
 template <int NC>
 __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict__ A, int n, double* __restrict__ d,
                                                              double* __restrict__ e, double* __restrict__ beta, int R,
-                                                             Packet* ex, EigControl* ctl) {
+                                                             int vbs, Packet* ex, EigControl* ctl) {
   extern __shared__ double smem_d[];
   __shared__ double sh_sigma[4], sh_pv[4], sh_ref[5];
   __shared__ int give_up;
   __shared__ unsigned sh_top;
+  if (NC < 8) vbs = 2;  // the plan takes one vb for large n only
   const int G = (int)gridDim.x, cta = (int)blockIdx.x, tid = threadIdx.x;
   const int t = tid & (HALF - 1), lane = tid & 31, wid = t >> 5;
   const bool reflector_half = tid >= HALF;
   double* x = smem_d;         // current column, rows kk + 1 ..
   double* vb2 = smem_d + n;   // the pending update is A -= vb wt^T + wt vb^T, vb = beta v; by parity
-  double* wt = smem_d + 3 * (size_t)n;
-  double* cn = smem_d + 4 * (size_t)n;  // the next column before this step's update
-  double* rows = smem_d + 5 * (size_t)n;
-  double* red = rows + (size_t)R * n;
+  double* wt = vb2 + vbs * (size_t)n;
+  double* cn = wt + n;  // the next column before this step's update
+  double* rows = cn + n;
+  double* red = vbs == 2 ? rows + (size_t)R * n : cn;
   double* cnew = red + 4 * R;
   const unsigned limit = ctl->limit, off_tag = ctl->extra ? 0x40000000u : 0u;
   const bool writer = cta == (n - 1) % G;  // the CTA that stays to the end writes the results
@@ -238,7 +241,7 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
   // of that row, who has read it above, published from it (row 0 is not read again).
   for (int i = tid; i < n; i += 2 * HALF) {
     x[i] = A[(size_t)i * n] * down;
-    vb2[n + i] = 0.0;  // no update is pending
+    vb2[(vbs - 1) * n + i] = 0.0;  // no update is pending
     wt[i] = 0.0;
   }
   if (writer && tid == 0) d[0] = A[0];
@@ -247,8 +250,8 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
   int s0 = 0;  // first slot with row > kk
   for (int kk = 0; kk + 2 < n; ++kk) {
     const int c1 = kk + 2, base = c1 & ~(HALF - 1);
-    const double* vb = vb2 + (size_t)((kk & 1) ^ 1) * n;  // of the step before
-    double* vbn = vb2 + (size_t)(kk & 1) * n;
+    const double* vb = vb2 + (vbs == 2 ? (size_t)((kk & 1) ^ 1) * n : 0);  // of the step before
+    double* vbn = vb2 + (vbs == 2 ? (size_t)(kk & 1) * n : 0);
     if (reflector_half) {
       // ---- reflector of x, while the other half works on the rows: v = x but for v0,
       // H = 1 - b v v^T
@@ -286,6 +289,7 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
         }
       }
       bar(2, HALF);
+      if (vbs == 1) bar(3, 2 * HALF);  // the row half has read vb
       const double b = sh_ref[1];
       for (int col = base + t; col < n; col += HALF)
         if (col >= c1) {
@@ -312,6 +316,7 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
       ll_store(&p->c, cnew[s], tag);
     }
     if (last_row <= kk + 1) return;  // nothing to publish any more
+    if (vbs == 1) bar(3, 2 * HALF);
     // ---- 2. A v = y - alpha c for the own columns > kk + 1 ----------------------------------------
     it = 0;
     double y0 = 0.0, d0 = 0.0, alpha = 0.0, pv = 0.0;  // y0, d0: row kk + 1 itself
@@ -369,7 +374,7 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
   }
   if (writer && tid == 0) {
     if (n >= 2) {
-      const double* vb = vb2 + (size_t)((n - 3) & 1) * n;  // of the last step
+      const double* vb = vb2 + (vbs == 2 ? (size_t)((n - 3) & 1) * n : 0);  // of the last step
       const double a = rows[(size_t)(nrows - 1) * n + n - 1];
       d[n - 1] = up * (n >= 3 ? fma(-2.0 * vb[n - 1], wt[n - 1], a) : a);
       e[n - 2] = up * x[n - 1];
@@ -378,11 +383,13 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
   }
 }
 
-size_t smem_of(int n, int R) { return sizeof(double) * ((size_t)n * (5 + R) + 5 * (size_t)R); }
+size_t smem_of(int n, int R, int vbs) {
+  return sizeof(double) * (vbs == 2 ? (size_t)n * (5 + R) + 5 * (size_t)R : std::max((size_t)n, 5 * (size_t)R) + (size_t)n * (3 + R));
+}
 }  // namespace
 
 namespace {
-using Kernel = void (*)(double*, int, double*, double*, double*, int, Packet*, EigControl*);
+using Kernel = void (*)(double*, int, double*, double*, double*, int, int, Packet*, EigControl*);
 Kernel kernel_of(int n) {
   return n <= HALF ? tridiag_kernel<1> : n <= 2 * HALF ? tridiag_kernel<2> : n <= 4 * HALF ? tridiag_kernel<4> : tridiag_kernel<8>;
 }
@@ -401,7 +408,10 @@ TridiagPlan tridiag_plan(int n, int forced) {
   int G = forced > 1 ? forced : std::min(sms, std::max(16, n / 5));
   G = std::min(G, n);
   const int R = (n + G - 1) / G;
-  const size_t smem = smem_of(n, R);
+  // Two vb until they are what keeps the rows out of shared memory (n from 1705 to 1814 on 152 SMs:
+  // 1800 rows, 181 vectors take 33.9 ms here and 83.7 ms on the general path).
+  const int vbs = n <= 4 * HALF || smem_of(n, R, 2) <= kSmemLimit ? 2 : 1;
+  const size_t smem = smem_of(n, R, vbs);
   if (smem > kSmemLimit) return P;
   if (cudaFuncSetAttribute(kernel_of(n), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel_of(n), 2 * HALF, smem) != cudaSuccess)
@@ -409,6 +419,7 @@ TridiagPlan tridiag_plan(int n, int forced) {
   if (G > sms * per_sm) return P;
   P.G = G;
   P.R = R;
+  P.vbs = vbs;
   P.smem = smem;
   return P;
 }
@@ -425,7 +436,7 @@ int tridiag_launch(double* A, int n, double* d, double* e, double* beta, const T
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  DF_CUDA(cudaLaunchKernelEx(&cfg, kernel_of(n), A, n, d, e, beta, P.R, (Packet*)exchange, ctl));
+  DF_CUDA(cudaLaunchKernelEx(&cfg, kernel_of(n), A, n, d, e, beta, P.R, P.vbs, (Packet*)exchange, ctl));
   return DF_OK;
 }
 

@@ -29,7 +29,7 @@ def clustered(n, m, gap, seed):
 
 
 def solve(A, k):
-    """Eigenpairs, and whether the direct vectors were given up."""
+    """Eigenpairs, whether the direct vectors were given up, and whether they were made at all."""
     lib, n = dfscf.lib(), len(A)
     dev = torch.as_tensor(A, device="cuda").clone()
     w = torch.empty(k, dtype=torch.float64, device="cuda")
@@ -50,7 +50,7 @@ def solve(A, k):
     words = work.view(torch.int32)[-1024:].cpu().numpy()
     at = np.flatnonzero(words == POLLS)
     assert len(at) == 1
-    return w.cpu().numpy(), Z.cpu().numpy(), bool(words[at[0] + 1])
+    return w.cpu().numpy(), Z.cpu().numpy(), bool(words[at[0] + 1]), bool(words[at[0] + 3:at[0] + 5].any())
 
 
 @pytest.mark.parametrize("n,m,k,direct", [(120, 20, 60, True), (120, 40, 60, False), (120, 40, 120, False),
@@ -58,7 +58,7 @@ def solve(A, k):
 def test_clusters_beyond_the_direct_path(n, m, k, direct):
     gap = 2.0 ** -44
     A, ref = clustered(n, m, gap, n + m)
-    w, Z, gave_up = solve(A, k)
+    w, Z, gave_up, _ = solve(A, k)
     assert gave_up != direct
     tol = n * 2.0 ** -52
     assert np.max(np.abs(w - ref[:k])) <= tol
@@ -66,3 +66,21 @@ def test_clusters_beyond_the_direct_path(n, m, k, direct):
     R = np.abs(A @ Z - Z * w)
     assert np.max(R[:, m:k]) <= tol
     assert np.max(R[:, :m]) <= tol + m * gap
+
+
+@pytest.mark.parametrize("n", [1704, 1705, 1814, 1815])
+def test_largest_rows_in_shared_memory(n):
+    """Up to 1814 rows (152 SMs) the reduction keeps its rows in shared memory, from 1705 on with
+    one vector less; beyond, the general path takes over."""
+    rng = np.random.default_rng(n)
+    X = rng.standard_normal((n, 40))
+    A = X @ X.T / n + np.diag(np.linspace(-1.0, 1.0, n))
+    A = 0.5 * (A + A.T)
+    w, Z, gave_up, direct = solve(A, 30)
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert direct == (n <= 1814) and not gave_up
+    ref = np.linalg.eigvalsh(A)
+    tol, norm = n * 2.0 ** -52, np.max(np.abs(ref))
+    assert np.max(np.abs(w - ref[:30])) <= tol * norm
+    assert np.max(np.abs(Z.T @ Z - np.eye(30))) <= tol
+    assert np.max(np.abs(A @ Z - Z * w)) <= tol * norm
