@@ -14,8 +14,8 @@
 //      and z outward from z_r = 1: z_i = -(e_i / q+_i) z_{i+1} and z_{i+1} = -(e_i / q-_{i+1}) z_i;
 //   3. reflectors in panels of 16: z -= V (T (V^T z));
 //   4. Z <- Z - (Z Z^T - 1) Z / 2, three times when the vectors need it.
-// Eigenvalues equal to rounding are told apart by the blocks into which T falls, and inside a
-// block by inverse iteration with projections.  What that cannot repair is left to inverse iteration
+// Eigenvalues equal to rounding are told apart by the blocks into which T falls, each with the
+// eigenvalue of its own block, and inside a block by inverse iteration with projections.  What that cannot repair is left to inverse iteration
 // and Gram-Schmidt over the whole matrix, or to implicit QL (eig.cu).
 // Device time at n = 900, k = 91 against 33-way bisection with a division a step, inverse iteration
 // from global memory, one reflector at a time and Gram-Schmidt with five grid barriers a vector:
@@ -313,18 +313,22 @@ size_t vectors_smem(int n) {
 }
 
 constexpr double kCluster = 0x1p-44;  // of ||T||: closer eigenvalues than that are one cluster
-constexpr double kSplit = 0x1p-46;    // of ||T||: inside a cluster a smaller subdiagonal entry separates blocks
+// Inside a cluster a subdiagonal entry up to 2^-52 sqrt(n) ||T|| separates blocks: twice what rounding
+// makes of a zero in the reduction, and what dropping it adds to a residual.  Where that leaves a block
+// with more members than inverse iteration has room for, entries up to 2^-46 ||T|| separate (a
+// projector of 900 rows: 117 ms by Gram-Schmidt over the grid, with residuals of 6e-14).
+__device__ __forceinline__ double split2_of(int n, int attempt) { return attempt ? 0x1p-92 : n * 0x1p-104; }
 
-// Counts of eigenvalues below x block by block of T (ends of blocks: subdiagonal <= kSplit):
+// Counts of eigenvalues below x block by block of T (ends of blocks: squared subdiagonal <= split2):
 // out[i] for the last row i of each block, -1 elsewhere.  One thread.
-__device__ void block_counts(const Row* __restrict__ T, int n, double x, int* __restrict__ out) {
+__device__ void block_counts(const Row* __restrict__ T, int n, double x, double split2, int* __restrict__ out) {
   double p0 = 1.0, p1 = 1.0, e2 = 0.0;
   int c = 0;
   for (int i = 0; i < n; ++i) {
     const double p = fma(T[i].d - x, p1, -(e2 * p0));
     c += (unsigned)(__double2hiint(p) ^ __double2hiint(p1)) >> 31;
     e2 = T[i].e2;
-    if (i == n - 1 || e2 <= kSplit * kSplit) {
+    if (i == n - 1 || e2 <= split2) {
       out[i] = c;
       c = 0;
       p0 = p1 = 1.0;
@@ -437,17 +441,39 @@ __device__ bool cluster_member(const Row* __restrict__ T, const double* __restri
   return true;
 }
 
-// CTA t: eigenvector t of T into row t of Y.  Eigenvalues closer than rounding come from different
-// blocks of a T that falls apart (equal eigenvalues of A make it do so): the members of such a
-// cluster are dealt out to the blocks that have an eigenvalue there, in order.
+// Integer with the order of the doubles (FP64 comparisons take 64 clocks a warp; no NaN, no -0 here).
+__device__ __forceinline__ long long sortable(double v) {
+  const long long b = __double_as_longlong(v);
+  return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+
+// Bisection of [lo, hi] for eigenvalue t by one thread.
+__device__ double bisect_thread(const Row* __restrict__ T, int n, int t, double lo, double hi) {
+  if (n == 1) return T[0].d;
+  for (int it = 0; it < 64; ++it) {
+    if (hi - lo <= fmax(2.0 * DBL_EPSILON * fmax(fabs(lo), fabs(hi)), 0x1p-58)) break;
+    const double x = 0.5 * (lo + hi);
+    if (count_below(T, n, x) > t) hi = x;
+    else lo = x;
+  }
+  return 0.5 * (lo + hi);
+}
+
+// CTA t: eigenvector t of T into row t of Y, and its eigenvalue into wv[t].  Eigenvalues closer than
+// rounding come from different blocks of a T that falls apart (equal eigenvalues of A make it do
+// so).  Every CTA of such a cluster forms the blocks' own eigenvalues there, the same bits in each,
+// and takes the one of its rank: 25 halvings a member, one thread each (10 us for blocks of one row),
+// or 3 rounds on the whole CTA for a few members of what may be large blocks.
 __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const double* __restrict__ d,
                                                          const double* __restrict__ e, const double* __restrict__ w,
-                                                         double* __restrict__ Y, EigControl* ctl) {
+                                                         double* __restrict__ Y, double* __restrict__ wv,
+                                                         EigControl* ctl) {
   extern __shared__ double smem_d[];
   __shared__ double sh[4];
   __shared__ unsigned shm[4];
   __shared__ unsigned long long best;
-  __shared__ int pick[5], leave;
+  __shared__ int pick[5], leave, found;
+  __shared__ double own;
   const int tid = threadIdx.x, t = (int)blockIdx.x;
   // Other CTAs of this grid may raise ctl->bad at any time: one thread reads it for all, or part of
   // the CTA would leave and the rest work on shared memory that was never written.
@@ -468,7 +494,7 @@ __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const dou
     if (tid == 0) ctl->bad = 1;
     return;
   }
-  const double scale = __hiloint2double((2045 - ex) << 20, 0);
+  const double scale = __hiloint2double((2045 - ex) << 20, 0), unscale = __hiloint2double((ex + 1) << 20, 0);
   for (int i = tid; i < n; i += NT) T[i] = scaled_row(d, e, n, i, scale);
   if (tid == 0) best = ~0ull;
   double l = w[t] * scale;
@@ -478,38 +504,78 @@ __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const dou
   while (tb + 1 < k && (w[tb + 1] - w[tb]) * scale <= kCluster) ++tb;
   __syncthreads();
   if (ta < tb) {
-    lo = w[ta] * scale - kCluster;
-    hi = w[tb] * scale + kCluster;
-    int *cl = (int*)fa, *ch = (int*)fb;
-    if (tid == 0) block_counts(T, n, lo, cl);
-    if (tid == 32) block_counts(T, n, hi, ch);
-    __syncthreads();
-    if (tid == 0) {
-      int left = t - ta, start = 0;
-      pick[3] = 0;
-      for (int i = 0; i < n; ++i)
-        if (cl[i] >= 0) {
-          const int m = ch[i] - cl[i];
-          if (left < m) {
-            pick[0] = start;
-            pick[1] = i + 1 - start;
-            pick[2] = cl[i];
-            pick[3] = m;
-            pick[4] = left;
-            break;
+    lo = w[ta] * scale - 0.5 * kCluster;
+    hi = w[tb] * scale + 0.5 * kCluster;
+    // the cluster's members in block order: last row of the block, number in it (arrays of n ints)
+    int *cl = (int*)fa, *ch = (int*)fb, *first = cl + n, *last = (int*)s, *number = last + n;
+    for (int attempt = 0; attempt < 2; ++attempt) {
+      if (tid == 0) block_counts(T, n, lo, split2_of(n, attempt), cl);
+      if (tid == 32) block_counts(T, n, hi, split2_of(n, attempt), ch);
+      __syncthreads();
+      if (tid == 0) {
+        int count = 0, start = 0;
+        bool large = false;
+        for (int i = 0; i < n; ++i)
+          if (cl[i] >= 0) {
+            const int m = ch[i] - cl[i];
+            large |= m > 1 && m * (i + 1 - start) > kMembers;
+            for (int q = cl[i]; q < ch[i] && count < n; ++q) {
+              last[count] = i;
+              number[count++] = q;
+            }
+            first[i] = start;
+            start = i + 1;
           }
-          left -= m;
-          start = i + 1;
-        }
+        found = large ? 0 : count;
+        pick[3] = 0;
+      }
+      __syncthreads();
+      if (found) break;
+    }
+    double* value = p;
+    const int members_in = found;
+    if (members_in > 8) {
+      for (int q = tid; q < members_in; q += NT) {
+        const int i = first[last[q]];
+        value[q] = bisect_thread(T + i, last[q] + 1 - i, number[q], lo, hi);
+      }
+    } else {
+      for (int q = 0; q < members_in; ++q) {
+        const int i = first[last[q]];
+        const double v = bisect(T + i, last[q] + 1 - i, number[q], lo, hi, shm);
+        if (tid == 0) value[q] = v;
+      }
+    }
+    __syncthreads();
+    for (int q = tid; q < members_in; q += NT) {
+      const double v = value[q];
+      const long long kv = sortable(v);
+      int rank = 0;
+      for (int r = 0; r < members_in; ++r) {
+        const long long kr = sortable(value[r]);
+        rank += kr < kv || (kr == kv && r < q);
+      }
+      if (rank == t - ta) {
+        const int i = last[q];
+        pick[0] = first[i];
+        pick[1] = i + 1 - first[i];
+        pick[2] = cl[i];
+        pick[3] = ch[i] - cl[i];
+        pick[4] = number[q] - cl[i];
+        own = v;
+      }
     }
     __syncthreads();
     const int m = pick[3];
-    if (m == 0 || (m > 1 && m * pick[1] > kMembers)) {
+    if (m == 0) {
       if (tid == 0) ctl->bad = 1;
       return;
     }
     i0 = pick[0];
     nb = pick[1];
+    l = own;
+    if (tid == 0) wv[t] = l * unscale;
+    __syncthreads();  // before the arrays that the values came from are used again
     if (m > 1) {
       const bool ok = cluster_member(T + i0, e + i0, scale, nb, pick[2], pick[4], lo, hi, p, n, members, sh, shm);
       if (!ok) {
@@ -520,8 +586,8 @@ __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const dou
       for (int i = tid; i < n; i += NT) Y[(size_t)t * n + i] = i >= i0 && i < i0 + nb ? z[i - i0] : 0.0;
       return;
     }
-    l = bisect(T + i0, nb, pick[2], lo, hi, shm);
-    __syncthreads();
+  } else if (tid == 0) {
+    wv[t] = w[t];
   }
   const Row* Tb = T + i0;
   if (tid < 32) minors(Tb, nb, l, 1, p, scp);
@@ -585,15 +651,18 @@ __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const dou
   for (int i = tid; i < n; i += NT) Y[(size_t)t * n + i] = i >= i0 && i < i0 + nb ? p[i - i0] * inv : 0.0;
 }
 
-// z <- H_0 .. H_{n-3} z for row blockIdx.x of Y, into Z.  Dynamic shared memory: z [n].
+// z <- H_0 .. H_{n-3} z for row blockIdx.x of Y, into Z; its eigenvalue from wv into w.  Dynamic shared
+// memory: z [n].
 __global__ void __launch_bounds__(NT) back_transform_kernel(const double* __restrict__ A, int n,
                                                             const double* __restrict__ Tf, const double* __restrict__ Y,
+                                                            const double* __restrict__ wv, double* __restrict__ w,
                                                             double* __restrict__ Z, const EigControl* ctl) {
   extern __shared__ double z[];
   __shared__ double red[NT / 32][kPanel], cs[kPanel];
   if (ctl->err | ctl->bad) return;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
   const size_t row = (size_t)blockIdx.x * n;
+  if (tid == 0) w[blockIdx.x] = wv[blockIdx.x];
   for (int i = tid; i < n; i += NT) z[i] = Y[row + i];
   __syncthreads();
   for (int b = (n - 2 + kPanel - 1) / kPanel - 1; b >= 0; --b) {
@@ -748,14 +817,15 @@ int trivec_launch(const double* A, int n, int k, const double* d, const double* 
   double* Y = Tf + (size_t)np * kPanel * kPanel;
   double* Q = Y + (size_t)n * k;
   double* E = Q + (size_t)n * k;
+  double* wv = E;  // eigenvalues on their way to w, before the Gram matrix
   DF_CUDA(cudaFuncSetAttribute(tri_values_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
   tri_values_kernel<<<k + np, NT, values_smem(n), s>>>(A, n, k, d, e, beta, w, Tf, ctl);
   DF_LAUNCHED("tri_values_kernel");
   DF_CUDA(cudaFuncSetAttribute(tri_vectors_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-  tri_vectors_kernel<<<k, NT, vectors_smem(n), s>>>(n, k, d, e, w, Y, ctl);
+  tri_vectors_kernel<<<k, NT, vectors_smem(n), s>>>(n, k, d, e, w, Y, wv, ctl);
   DF_LAUNCHED("tri_vectors_kernel");
   DF_CUDA(cudaFuncSetAttribute(back_transform_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-  back_transform_kernel<<<k, NT, sizeof(double) * (size_t)n, s>>>(A, n, Tf, Y, Q, ctl);
+  back_transform_kernel<<<k, NT, sizeof(double) * (size_t)n, s>>>(A, n, Tf, Y, wv, w, Q, ctl);
   DF_LAUNCHED("back_transform_kernel");
   const int kt = (k + GT - 1) / GT;
   const dim3 grid((n + NT - 1) / NT, kt);
