@@ -12,6 +12,7 @@
 //      in FP64 to the last bit; a bracket that FP64 does not confirm starts over in FP64;
 //   2. minors from both ends, pivots q+ and q-, the index r with the least |q+_r + q-_r - (d_r - l)|,
 //      and z outward from z_r = 1: z_i = -(e_i / q+_i) z_{i+1} and z_{i+1} = -(e_i / q-_{i+1}) z_i;
+//      then one correction of z: its residual in twice the precision, solved with the same factors;
 //   3. reflectors in panels of 16: z -= V (T (V^T z));
 //   4. Z <- Z - (Z Z^T - 1) Z / 2, three times when the vectors need it.
 // Eigenvalues equal to rounding are told apart by the blocks into which T falls, each with the
@@ -459,6 +460,39 @@ __device__ double bisect_thread(const Row* __restrict__ T, int n, int t, double 
   return 0.5 * (lo + hi);
 }
 
+// Row i of (T - l) z to about twice the working precision.
+__device__ __forceinline__ double residual_row(const Row* __restrict__ T, const double* __restrict__ e, double scale,
+                                               int n, double l, const double* __restrict__ z, int i) {
+  const double d = T[i].d, a = d - l, bb = a - d, al = (d - (a - bb)) + (-l - bb);  // a + al = d - l (Knuth)
+  const double zi = z[i], em = i > 0 ? e[i - 1] * scale : 0.0, zm = i > 0 ? z[i - 1] : 0.0;
+  const double ep = i + 1 < n ? e[i] * scale : 0.0, zp = i + 1 < n ? z[i + 1] : 0.0;
+  const double h1 = a * zi, h2 = em * zm, h3 = ep * zp;
+  const double l1 = fma(al, zi, fma(a, zi, -h1)), l2 = fma(em, zm, -h2), l3 = fma(ep, zp, -h3);
+  const double s1 = h1 + h2, t1 = s1 - h1, r1 = (h1 - (s1 - t1)) + (h2 - t1);
+  const double s2 = s1 + h3, t2 = s2 - s1, r2 = (s1 - (s2 - t2)) + (h3 - t2);
+  return s2 + (((l1 + l2) + (l3 + r1)) + r2);
+}
+
+// s[at] += f[at + df] s[at - dir] along `count` entries from `at`, the first as it is; one thread,
+// operands loaded eight ahead of the chain.
+__device__ __forceinline__ void chain(double* __restrict__ s, const double* __restrict__ f, int at, int count, int dir,
+                                      int df) {
+  if (count < 2) return;
+  double v = s[at];
+  for (int q = 1; q < count; q += 8) {
+    double c[8], x[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      const int i = at + dir * min(q + u, count - 1);
+      c[u] = f[i + df];
+      x[u] = s[i];
+    }
+#pragma unroll
+    for (int u = 0; u < 8; ++u)
+      if (q + u < count) s[at + dir * (q + u)] = v = fma(c[u], v, x[u]);
+  }
+}
+
 // CTA t: eigenvector t of T into row t of Y, and its eigenvalue into wv[t].  Eigenvalues closer than
 // rounding come from different blocks of a T that falls apart (equal eigenvalues of A make it do
 // so).  Every CTA of such a cluster forms the blocks' own eigenvalues there, the same bits in each,
@@ -590,6 +624,7 @@ __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const dou
     wv[t] = w[t];
   }
   const Row* Tb = T + i0;
+  double *qa = fb + n, *qz = members;  // pivots (n is below kMembers: vectors_smem)
   if (tid < 32) minors(Tb, nb, l, 1, p, scp);
   else if (tid < 64) minors(Tb, nb, l, -1, s, scs);
   __syncthreads();
@@ -601,6 +636,8 @@ __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const dou
     const int m = nb - 1 - i;  // position in the backward recurrence
     const double after = m > 0 ? (((m - 1) & 7) == 0 && m > 1 ? shifted(s[i + 1], scs[(m - 2) / 8]) : s[i + 1]) : 1.0;
     const double qf = p[i] / before, qb = s[i] / after;
+    qa[i] = qf;
+    qz[i] = qb;
     const double gamma = (qf + qb) - (Tb[i].d - l);
     const unsigned long long key = (unsigned long long)__double_as_longlong(fabs(gamma));
     if (key < mine) {
@@ -638,6 +675,8 @@ __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const dou
       for (int u = 0; u < 8; ++u)
         if (i + u < nb) p[i + u] = z *= f[u];
     }
+  } else if (tid >= 64) {
+    for (int i = tid - 64; i < nb; i += NT - 64) qa[i] = 1.0 / (i < r ? qa[i] : qz[i]);
   }
   __syncthreads();
   double n2 = 0.0;
@@ -648,7 +687,46 @@ __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const dou
     return;
   }
   const double inv = 1.0 / sqrt(n2);
-  for (int i = tid; i < n; i += NT) Y[(size_t)t * n + i] = i >= i0 && i < i0 + nb ? p[i - i0] * inv : 0.0;
+  for (int i = tid; i < nb; i += NT) p[i] *= inv;
+  __syncthreads();
+  // ---- correction: (T - l) y = (T - l) z - delta z without row r, y_r = 0, delta = z.(T - l) z ----------
+  // z's components along its neighbours, 1.4e-14 for the 90 lowest of 900 rows where inverse iteration
+  // left 4e-15, become negligible (the residual of a rounded z); 0.06 ms of 0.23 at 900 rows.
+  double c = 0.0;
+  for (int i = tid; i < nb; i += NT) {
+    const double b = residual_row(Tb, e + i0, scale, nb, l, p, i);
+    s[i] = b;
+    c = fma(p[i], b, c);
+  }
+  c = sum4(c, sh);
+  for (int i = tid; i < nb; i += NT) s[i] = i == r ? 0.0 : fma(-c, p[i], s[i]);
+  __syncthreads();
+  if (tid == 0) {
+    chain(s, fa, 0, r, 1, -1);
+  } else if (tid == 32) {
+    chain(s, fb, nb - 1, nb - 1 - r, -1, 1);
+  }
+  __syncthreads();
+  for (int i = tid; i < nb; i += NT) s[i] *= qa[i];  // s_r = 0
+  __syncthreads();
+  if (tid == 0) {
+    chain(s, fa, r, r + 1, -1, 0);
+  } else if (tid == 32) {
+    chain(s, fb, r, nb - r, 1, 0);
+  }
+  __syncthreads();
+  double y2 = 0.0, m2 = 0.0;
+  for (int i = tid; i < nb; i += NT) {
+    const double y = s[i], v = p[i] - y;
+    y2 = fma(y, y, y2);
+    m2 = fma(v, v, m2);
+  }
+  y2 = sum4(y2, sh);
+  m2 = sum4(m2, sh);
+  const bool take = y2 <= 1e-4;  // else the factors are too poor for it
+  const double norm = take ? 1.0 / sqrt(m2) : 1.0;
+  for (int i = tid; i < n; i += NT)
+    Y[(size_t)t * n + i] = i >= i0 && i < i0 + nb ? (take ? p[i - i0] - s[i - i0] : p[i - i0]) * norm : 0.0;
 }
 
 // z <- H_0 .. H_{n-3} z for row blockIdx.x of Y, into Z; its eigenvalue from wv into w.  Dynamic shared
