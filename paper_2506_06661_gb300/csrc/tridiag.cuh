@@ -22,7 +22,7 @@ constexpr int kPanel = 16;  // reflectors applied at once in the back-transforma
 struct TridiagPlan {
   int G = 0;  // CTAs (0: the size does not fit)
   int R = 0;  // rows per CTA
-  int vbs = 2;  // vectors of pending updates in shared memory
+  int vps = 2;  // vectors of pending updates in shared memory
   size_t smem = 0;
 };
 
