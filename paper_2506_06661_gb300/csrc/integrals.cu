@@ -15,11 +15,6 @@ __device__ __forceinline__ double norm_s(double a) {
   return sqrt(x * sqrt(x));
 }
 
-// Factors of an auxiliary function in one expression each, which rounds less often than norm_s(c) / c:
-// N_c / c = (2/pi)^(3/4) c^(-1/4), and that times (2 pi^{5/2})^(1/2) for the metric.
-__device__ __forceinline__ double aux_factor(double c) { return 0.71270547035499021 / sqrt(sqrt(c)); }
-__device__ __forceinline__ double metric_factor(double c) { return 4.2156294610216234 / sqrt(sqrt(c)); }
-
 __global__ void boys_kernel(const double* __restrict__ t, long n, double* __restrict__ out) {
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   if (i < n) out[i] = boys_f0(t[i]);
@@ -74,12 +69,12 @@ __global__ void int1e_kernel(const double* __restrict__ xyz, const double* __res
 // long-range operator erf(omega r)/r of the paper's LRDF split: the reduced exponent
 // rho = cd/(c+d) becomes rho f in the Boys argument and the prefactor gains sqrt(f),
 // f = omega^2 / (rho + omega^2).
-// One lane per column d and 16 rows c, whose factors are formed once per CTA.
+// One lane per column d and 16 rows c, whose factors N_c / c are formed once per CTA.
 constexpr int I2C_ROWS = 16;
 __global__ void __launch_bounds__(128) int2c_kernel(const double* __restrict__ xyz, const double* __restrict__ ex,
                                                     int naux, double omega, const double* __restrict__ table,
                                                     double* __restrict__ M) {
-  __shared__ double sc[I2C_ROWS][5];  // exponent, centre, N_c / c (2 pi^{5/2})^(1/2)
+  __shared__ double sc[I2C_ROWS][5];  // exponent, centre, N_c / c
   const int c0 = blockIdx.y * I2C_ROWS, nc = min(I2C_ROWS, naux - c0);
   if ((int)threadIdx.x < nc) {
     const int c = c0 + threadIdx.x;
@@ -88,18 +83,18 @@ __global__ void __launch_bounds__(128) int2c_kernel(const double* __restrict__ x
     sc[threadIdx.x][1] = xyz[3 * c];
     sc[threadIdx.x][2] = xyz[3 * c + 1];
     sc[threadIdx.x][3] = xyz[3 * c + 2];
-    sc[threadIdx.x][4] = metric_factor(e);
+    sc[threadIdx.x][4] = norm_s(e) / e;
   }
   __syncthreads();
   const int d = blockIdx.x * blockDim.x + threadIdx.x;
   if (d >= naux) return;
   const double ed = ex[d], x = xyz[3 * d], y = xyz[3 * d + 1], z = xyz[3 * d + 2];
-  const double nd = metric_factor(ed);
+  const double nd = norm_s(ed) / ed, k = 2.0 * kPi * kPi * sqrt(kPi);
   for (int i = 0; i < nc; ++i) {
     const double ec = sc[i][0], dx = sc[i][1] - x, dy = sc[i][2] - y, dz = sc[i][3] - z;
     const double r2 = dx * dx + dy * dy + dz * dz;
     const double q = rsqrt_fast(ec + ed);
-    double pre = (sc[i][4] * nd) * q, rho = ec * ed * (q * q);  // the same bits for (c, d) and (d, c)
+    double pre = (sc[i][4] * nd) * (k * q), rho = ec * ed * (q * q);  // the same bits for (c, d) and (d, c)
     if (omega > 0.0) {
       const double f = omega * omega / (rho + omega * omega);
       pre *= sqrt(f);
@@ -111,8 +106,7 @@ __global__ void __launch_bounds__(128) int2c_kernel(const double* __restrict__ x
 
 // Row k of the Boys table: (-1)^j F_j(t) / j!, j = 0..6, at t = k / 32.  Below t = 10, F_6 from its
 // series e^-t sum_i (2t)^i / (13 15 .. (13 + 2i)) (all terms positive) and downward recursion
-// F_{j-1} = (2t F_j + e^-t) / (2j - 1); above, upward from F_0.  F_0 itself, whose error is the
-// integral's, comes from erf from t = 2 on: the recursion's is 0.6 to 0.9 ulp there, erf's 0.4.
+// F_{j-1} = (2t F_j + e^-t) / (2j - 1); above, upward from F_0.
 __global__ void boys_table_kernel(double* __restrict__ table) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
   if (k >= BOYS_ROWS) return;
@@ -125,7 +119,6 @@ __global__ void boys_table_kernel(double* __restrict__ table) {
     F[6] = et * r * (1.0 / 13.0);
 #pragma unroll
     for (int j = 6; j >= 1; --j) F[j - 1] = fma(2.0 * t, F[j], et) * (1.0 / (2 * j - 1));
-    if (t >= 2.0) F[0] = boys_f0(t);
   } else {
     F[0] = boys_f0(t);
     const double h = 0.5 / t;
@@ -187,7 +180,7 @@ __global__ void __launch_bounds__(256) int3c_kernel(const double* __restrict__ p
     sq[threadIdx.x][1] = axyz[3 * q];
     sq[threadIdx.x][2] = axyz[3 * q + 1];
     sq[threadIdx.x][3] = axyz[3 * q + 2];
-    sq[threadIdx.x][4] = aux_factor(c);
+    sq[threadIdx.x][4] = norm_s(c) / c;
   }
   __syncthreads();
   const long ij = (long)blockIdx.x * blockDim.x + threadIdx.x;
