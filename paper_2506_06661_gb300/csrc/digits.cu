@@ -351,6 +351,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1) digit_gemm_kernel(const __gri
       if (p.mode == HALF_TRANSFORM && big) atomicMax(p.xkey + m, big);
     }
   }
+  __syncwarp();  // the one-lane roles above; TMEM is freed by a whole warp
   tc_fence_before();
   __syncthreads();
   if (abort_flag && warp == 0 && lane == 0) {

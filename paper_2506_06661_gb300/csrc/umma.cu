@@ -262,6 +262,7 @@ __global__ void __launch_bounds__(THREADS, 1) split_bf16_gemm_kernel(const __gri
       if (p.mode == HALF_TRANSFORM) atomicMax(p.xmax + grow % p.npad, __float_as_uint(lmax));
     }
   }
+  __syncwarp();  // the one-lane roles above; TMEM is freed by a whole warp
   tc_fence_before();
   __syncthreads();
   if (abort_flag && warp == 0 && lane == 0) {
@@ -363,6 +364,7 @@ __global__ void __launch_bounds__(THREADS, 1) syrk_pair_kernel(const __grid_cons
     tmem_alloc_pair(&tmem_base, ncols);
     tmem_relinquish_pair();
   }
+  __syncwarp();  // lane 0 initialised the barriers: the cluster barrier wants whole warps
   tc_fence_before();
   cluster_sync();  // both CTAs' barriers initialised and TMEM allocated before any remote use
   tc_fence_after();
@@ -454,6 +456,7 @@ __global__ void __launch_bounds__(THREADS, 1) syrk_pair_kernel(const __grid_cons
       }
     }
   }
+  __syncwarp();
   tc_fence_before();
   __syncthreads();
   if (abort_flag && warp == 0 && lane == 0) {
@@ -467,6 +470,7 @@ __global__ void __launch_bounds__(THREADS, 1) syrk_pair_kernel(const __grid_cons
           mbar_wait(&full_bar[s], (uint32_t)(last / p.stages) & 1u, nullptr);
       }
   }
+  __syncwarp();
   cluster_sync();  // no CTA leaves while its peer may still signal its barriers or read its TMEM
   if (warp == 1) {
     tc_fence_after();
