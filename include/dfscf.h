@@ -48,10 +48,20 @@ extern "C" {
 #define DF_ERR_NUMERIC 7     /* NaN/Inf detected in an SCF quantity                     */
 
 /* ---- precision modes -------------------------------------------------------------- */
-#define DF_FP64 0            /* every contraction to FP64 accuracy or better: the exchange
-                                contractions run on the tensor cores as exact sums of
-                                base-512 digit products in 64-bit integers, rounded to
-                                FP64 once (entry errors below 2^-51 sqrt(K_mm K_nn))     */
+#define DF_FP64 0            /* every contraction to FP64 accuracy in norm: those of the
+                                exchange, the whitening and the metric's Cholesky run on
+                                the tensor cores as sums of base-512 digit products in
+                                64-bit integers.  A row of an operand is held to 2^-62 of
+                                its largest element, so a sum of n products is off by at
+                                most 2^-60 sqrt(n) times its rows' largest elements, and
+                                by its rounding to FP64: X = B C once, K once per block of
+                                auxiliary rows and once per block added.  K's entries come
+                                out within (4 + blocks) 2^-53 sqrt(K_mm K_nn) unless the
+                                terms of X cancel (|C| far above 1 / ||S^1/2||).  Unlike
+                                an FP64 sum's, the error is not relative to the entry's
+                                own terms: an entry of K between functions far apart, 2^-9
+                                of the largest or less, is as exact in absolute terms, not
+                                in relative ones                                         */
 #define DF_MIXED 1           /* K contractions as split-BF16 GEMMs on tcgen05 tensor
                                 cores.  Every operand row (of B_P, of C^T, of X) is held
                                 as NP BF16 planes, NP = the knob "mixed_planes" (3, 4 or

@@ -38,7 +38,7 @@ constexpr int BOYS_ROWS = 40 * 32 + 1, BOYS_STRIDE = 8;
 constexpr size_t BOYS_TABLE = (size_t)BOYS_ROWS * BOYS_STRIDE;
 
 // 1 / sqrt(a) to about 1 ulp in 5 FP64 instructions: the hardware's 2^-20 estimate and one step of
-// third order (Householder): y (1 + e/2 + 3 e^2/8), e = 1 - a y^2.
+// third order (Householder): y (1 + e/2 + 3 e^2/8), e = 1 - a y^2 (tests/test_gpu_fp64_roots.py).
 __device__ __forceinline__ double rsqrt_fast(double a) {
   const unsigned h = (unsigned)__double2hiint(a);
   if (h - 0x00100000u >= 0x7fd00000u) return 1.0 / sqrt(a);  // not a positive normal number below 2^1023

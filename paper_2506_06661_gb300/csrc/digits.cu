@@ -43,7 +43,7 @@ struct Params {
   long ldc, sC;
   int lower, trans;     // lower tiles only; C stored transposed (C[col ldc + row])
   // half-transform
-  int nao, naux, p0;
+  int nao, p0;
   double* X;
   long ldx, xcol0;
   unsigned* xkey;
@@ -608,8 +608,7 @@ int slice_with_keys(const double* A, long lda, const DigitOperand& o, cudaStream
   return DF_OK;
 }
 
-int slice_packed(const double* B, long ldb, int nao, int naux, int p0, int np, const DigitOperand& o, cudaStream_t s) {
-  (void)naux;
+int slice_packed(const double* B, long ldb, int nao, int p0, int np, const DigitOperand& o, cudaStream_t s) {
   slice_packed_kernel<<<dim3((unsigned)((nao + PT - 1) / PT), (unsigned)np), 256, 0, s>>>(B, ldb, nao, p0, np,
                                                                                       plane_ld(nao), o.key, o.p);
   DF_LAUNCHED("slice_packed_kernel");
@@ -642,8 +641,8 @@ int digit_gemm(const DigitOperand& A, const DigitOperand& B, DigitSource A0, Dig
   return launch_any(A, B, p, std::max(1, splits), 0, s);
 }
 
-int digit_half_transform(const DigitOperand& A, const DigitOperand& Ct, const double* B, long ldb, int nao, int naux,
-                         int p0, const double* C, int nocc, double* X, long ldx, long xcol0, unsigned* xkey, int* err,
+int digit_half_transform(const DigitOperand& A, const DigitOperand& Ct, const double* B, long ldb, int nao, int p0,
+                         const double* C, int nocc, double* X, long ldx, long xcol0, unsigned* xkey, int* err,
                          cudaStream_t s) {
   DF_REQUIRE(A.rows < INT_MAX, DF_ERR_ARG, "half-transform: too many rows");
   Params p{};
@@ -653,7 +652,6 @@ int digit_half_transform(const DigitOperand& A, const DigitOperand& Ct, const do
   p.ka = A.key;
   p.kb = Ct.key;
   p.nao = nao;
-  p.naux = naux;
   p.p0 = p0;
   p.X = X;
   p.ldx = ldx;

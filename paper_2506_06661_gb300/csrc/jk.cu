@@ -513,8 +513,8 @@ int build_K_fp64(const double* B64, long ld, int nao, int naux, const double* C,
       for (int p0 = x0; p0 < x0 + nx; p0 += w.pb) {
         const int np = std::min(w.pb, x0 + nx - p0);
         const DigitOperand bp = digit_operand(w.Bp, (long)np * nao, nao);
-        DF_TRY(slice_packed(B64, ld, nao, naux, p0, np, bp, s));
-        DF_TRY(digit_half_transform(bp, ct, B64, ld, nao, naux, p0, C, nocc, w.X, kdim, (long)(p0 - x0) * nocc, xd.key,
+        DF_TRY(slice_packed(B64, ld, nao, p0, np, bp, s));
+        DF_TRY(digit_half_transform(bp, ct, B64, ld, nao, p0, C, nocc, w.X, kdim, (long)(p0 - x0) * nocc, xd.key,
                                     w.err, s));
       }
     }
