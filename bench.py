@@ -26,9 +26,9 @@ ROOT = os.path.dirname(os.path.abspath(__file__))
 sys.path.insert(0, ROOT)
 
 METRIC = "DF-JK builds/s + tensor-pipe %; SCF time-to-1e-6 Eh, mixed vs FP64"
-# FP64 ALU peak: 152 SMs x 2 FP64 FMA/clk/SM x 2 flop x 2.07 GHz (1.90 FMA/clk/SM measured)
-FP64_PEAK_TFLOPS = 152 * 2 * 2 * 2.07e9 / 1e12
-LAUNCHES_FP64 = 7   # kernels per FP64 build: Dw, J pass 1, J pass 2, J reduce, K half-transform, K SYRK, K mirror
+DIGIT_PRODUCTS = 28  # BF16 digit products of an FP64 product (7 digits, orders 0 to 6)
+FP64_PHASES = ("k_slice_b_fp64", "k_halftransform_fp64", "k_slice_x_fp64", "k_syrk_fp64")  # one launch a scope
+LAUNCHES_FP64 = 6   # kernels per FP64 build beside those: Dw, J pass 1, J pass 2, J reduce, digits of C, K mirror
 LAUNCHES_MIXED = 9  # Dw, J pass 1, J pass 2, J reduce, C^T planes, tcgen05 half-transform, X planes, tcgen05 SYRK,
 #                     K reduce
 
@@ -248,8 +248,6 @@ def time_builds(dfscf, torch, B, D, C, prec, steps, warmup, work, barrier):
         dfscf.jk(B, D, C, precision=prec, work=work, out_j=J, out_k=K)
     barrier()
     torch.cuda.synchronize()
-    dfscf.profile_reset()
-    dfscf.profile_enable(True)
     e0 = torch.cuda.Event(enable_timing=True)
     e1 = torch.cuda.Event(enable_timing=True)
     torch.cuda.nvtx.range_push(f"fock_{prec}")  # lets a profiler select the timed builds
@@ -259,10 +257,16 @@ def time_builds(dfscf, torch, B, D, C, prec, steps, warmup, work, barrier):
     e1.record(stream)
     torch.cuda.nvtx.range_pop()
     torch.cuda.synchronize()
-    dfscf.profile_enable(False)
-    prof = dfscf.profile_read()
     barrier()
-    return e0.elapsed_time(e1) / steps, prof
+    # the phases, from as many builds again up to three: their events stay out of the timed ones
+    again = min(steps, 3)
+    dfscf.profile_reset()
+    dfscf.profile_enable(True)
+    for _ in range(again):
+        dfscf.jk(B, D, C, precision=prec, work=work, out_j=J, out_k=K)
+    torch.cuda.synchronize()
+    dfscf.profile_enable(False)
+    return e0.elapsed_time(e1) / steps, {k: (ms / again, n / again) for k, (ms, n) in dfscf.profile_read().items()}
 
 
 def time_e2e(dfscf, torch, B, D, C, prec, steps, work):
@@ -296,17 +300,24 @@ def time_e2e(dfscf, torch, B, D, C, prec, steps, work):
     return ms, (hD.numel() + hC.numel()) * 8, (hJ.numel() + hK.numel()) * 8
 
 
-def roofline_of(prof, name, flops_per_launch=None, bytes_per_launch=None, peak=None, bound="alu", unit="TFLOP/s"):
+def roofline_of(prof, name, flops=None, nbytes=None, peak=None, bound="tensor", unit="TFLOP/s"):
+    """Rate of a phase: the operations or bytes of one build over the phase's time in one build, which
+    may be spread over several launches (prof: milliseconds and launches of a build)."""
     if name not in prof:
         return None
-    ms, calls = prof[name]
-    avg = ms / max(calls, 1)
-    if flops_per_launch is not None:
-        ach = flops_per_launch / (avg * 1e-3) / 1e12
-    else:
-        ach = bytes_per_launch / (avg * 1e-3) / 1e9
+    per_build, calls = prof[name]
+    ach = flops / (per_build * 1e-3) / 1e12 if flops is not None else nbytes / (per_build * 1e-3) / 1e9
     return {"kernel": name, "bound": bound, "achieved": ach, "peak": peak, "unit": unit, "frac": ach / peak,
-            "traffic": None, "avg_ms": avg, "launches": calls}
+            "traffic": None, "ms_per_build": per_build, "launches_per_build": calls}
+
+
+def digit_gemm_flops(m, n, k, lower=False):
+    """BF16 operations issued by the digit product of m x k and n x k: tiles of 128 x 64 (or one or two
+    groups of 16 columns up to 32), K in stages of 32."""
+    width = 64 if n > 32 else (32 if n > 16 else 16)
+    rows, cols = -(-m // 128), -(-n // width)
+    tiles = sum(min((min((r + 1) * 128, m) - 1) // width + 1, cols) for r in range(rows)) if lower else rows * cols
+    return DIGIT_PRODUCTS * 2.0 * tiles * 128 * width * (-(-k // 32) * 32)
 
 
 def scf_time_to_convergence(dfscf, torch, wl, oracle_energy=False, max_cycle=100):
@@ -394,26 +405,25 @@ def run_ours(args):
     syrk_flops = 1.0 * naux * nocc * nao * nao
     j_bytes = 8.0 * naux * dfscf.lib().df_B_ld(nao)
     rl = {}
-    for name, fl in (("k_halftransform_fp64", ht_flops), ("k_syrk_fp64", syrk_flops)):
-        r = roofline_of(prof64, name, flops_per_launch=fl, peak=FP64_PEAK_TFLOPS, bound="alu")
+    # the FP64 exchange runs as 28 BF16 digit products: those of the unpadded contraction against the
+    # tensor peak, what the padded tiles issue, and the FP64 rate they amount to
+    for name, fl, issued in (("k_halftransform_fp64", ht_flops, digit_gemm_flops(naux * nao, nocc, nao)),
+                             ("k_syrk_fp64", syrk_flops, digit_gemm_flops(nao, nao, naux * nocc, lower=True))):
+        r = roofline_of(prof64, name, flops=DIGIT_PRODUCTS * fl, peak=peaks["bf16_tflops_sustained"])
+        if r:
+            r["fp64_tflops"] = r["achieved"] / DIGIT_PRODUCTS
+            r["issued_tflops"] = issued / (r["ms_per_build"] * 1e-3) / 1e12
+            r["issued_frac"] = r["issued_tflops"] / peaks["bf16_tflops_sustained"]
+            rl[name] = r
+    # slicing: B's packed rows read (twice, the second time from L2) and 7 digit planes written
+    planes8 = 14.0 * (-(-nao // 8) * 8)
+    for name, nb in (("k_slice_b_fp64", j_bytes + naux * nao * planes8), ("k_slice_x_fp64", 22.0 * nao * naux * nocc),
+                     ("j_pass1", j_bytes), ("j_pass2", j_bytes)):
+        r = roofline_of(prof64, name, nbytes=nb, peak=peaks["hbm_gbs"], bound="hbm", unit="GB/s")
         if r:
             rl[name] = r
-    for name in ("j_pass1", "j_pass2"):
-        r = roofline_of(prof64, name, bytes_per_launch=j_bytes, peak=peaks["hbm_gbs"], bound="hbm", unit="GB/s")
-        if r:
-            rl[name] = r
-    dominant = max(rl.values(), key=lambda r: r["avg_ms"] * r["launches"]) if rl else None
-    # DRAM traffic of the FP64 half-transform: the ncu capture of the same kernel (32
-    # occupied columns per CTA, the variant this workload runs) on the 80-centre workload
-    # read 772.81 MB and wrote 144.74 MB against 926.0 MB of algorithmic bytes (B read once,
-    # X written once); traffic grows with those bytes, so one launch here moves that ratio
-    # times its own algorithmic bytes
-    if dominant and dominant["kernel"] == "k_halftransform_fp64":
-        ht_bytes = 8.0 * naux * dfscf.lib().df_B_ld(nao) + 8.0 * nao * naux * nocc
-        m80_bytes = 8.0 * 1200 * dfscf.lib().df_B_ld(400) + 8.0 * 400 * 1200 * 40
-        dominant["traffic"] = (772.808448e6 + 144.741120e6) / m80_bytes * ht_bytes
-        dominant["traffic_source"] = ("ncu dram__bytes_read.sum + dram__bytes_write.sum of the 80-centre capture, "
-                                      "scaled by the algorithmic bytes of this launch")
+    dominant = max(rl.values(), key=lambda r: r["ms_per_build"]) if rl else None
+    launches64 = round(args.steps * (LAUNCHES_FP64 + sum(prof64[p][1] for p in FP64_PHASES if p in prof64)))
 
     e2e_ms, h2d, d2h = time_e2e(dfscf, torch, B, D, C, "fp64", args.e2e_steps, work64)
 
@@ -448,20 +458,20 @@ def run_ours(args):
         rlm = {}
         for name, fl, alg in (("k_halftransform_tc", tc_ht, products * ht_flops),
                               ("k_syrk_tc", tc_syrk, products * syrk_flops)):
-            r = roofline_of(profm, name, flops_per_launch=alg, peak=peaks["bf16_tflops_sustained"], bound="tensor")
+            r = roofline_of(profm, name, flops=alg, peak=peaks["bf16_tflops_sustained"])
             if r:
-                r["issued_tflops"] = fl / (r["avg_ms"] * 1e-3) / 1e12
+                r["issued_tflops"] = fl / (r["ms_per_build"] * 1e-3) / 1e12
                 r["issued_frac"] = r["issued_tflops"] / peaks["bf16_tflops_sustained"]
                 rlm[name] = r
         for name in ("j_pass1", "j_pass2"):
-            r = roofline_of(profm, name, bytes_per_launch=j_bytes, peak=peaks["hbm_gbs"], bound="hbm", unit="GB/s")
+            r = roofline_of(profm, name, nbytes=j_bytes, peak=peaks["hbm_gbs"], bound="hbm", unit="GB/s")
             if r:
                 rlm[name] = r
         mixed = {"value": ws * 1000.0 / msm, "unit": "builds/s", "ms_per_step": msm, "steps": args.mixed_steps,
                  "dtype": f"bf16 planes x{planes}, {products} products, two fixed-point planes, exact fp32 sums of their products (K); f64 (J)",
                  "rel_err_vs_fp64": {"J": errj, "K": errk},
                  "kernels": rlm, "gpu_launches": LAUNCHES_MIXED * args.mixed_steps, "clocks": clkm.summary(),
-                 "phase_ms": {k: v[0] / max(v[1], 1) for k, v in profm.items()}}
+                 "phase_ms": {k: v[0] for k, v in profm.items()}}
 
     scf = None
     tune.reset()  # the SCF and batch blocks do not inherit this workload's launch knobs
@@ -516,14 +526,12 @@ def run_ours(args):
                        "knobs": knobs,
                        "l2": "inputs larger than L2 (B is %.1f GB)" % (8.0 * naux * npair / 1e9),
                        "parallelism": f"replicas x{ws}" if ws > 1 else "single GPU"},
-            "roofline": ({k: v for k, v in dominant.items() if k not in ("avg_ms", "launches")} | {"peak_source": (
-                "derived FP64 ALU peak: 152 SMs x 2 FMA/clk x 2 flop x 2.07 GHz" if dominant["bound"] == "alu"
-                else f"MEASURED_PEAKS.json ({peak_src})")}) if dominant else None,
+            "roofline": (dominant | {"peak_source": f"MEASURED_PEAKS.json ({peak_src})"}) if dominant else None,
             "kernels": rl,
-            "phase_ms": {k: v[0] / max(v[1], 1) for k, v in prof64.items()},
+            "phase_ms": {k: v[0] for k, v in prof64.items()},
             "e2e": {"value": ws * 1000.0 / e2e_ms, "unit": "builds/s", "h2d_bytes_per_step": h2d,
                     "d2h_bytes_per_step": d2h, "steps": args.e2e_steps},
-            "gpu_launches": LAUNCHES_FP64 * args.steps,
+            "gpu_launches": launches64,
             "clocks": clocks,
             "setup_s": t_setup,
             "mixed": mixed,

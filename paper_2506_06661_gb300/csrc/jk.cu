@@ -510,18 +510,24 @@ int build_K_fp64(const double* B64, long ld, int nao, int naux, const double* C,
     const long kdim = (long)nx * nocc;
     const DigitOperand xd = digit_operand(w.Xd, nao, kdim);
     DF_CUDA(cudaMemsetAsync(xd.key, 0, sizeof(unsigned) * (size_t)nao, s));
-    {
-      ProfScope ps("k_halftransform_fp64", s);
-      for (int p0 = x0; p0 < x0 + nx; p0 += w.pb) {
-        const int np = std::min(w.pb, x0 + nx - p0);
-        const DigitOperand bp = digit_operand(w.Bp, (long)np * nao, nao);
+    for (int p0 = x0; p0 < x0 + nx; p0 += w.pb) {
+      const int np = std::min(w.pb, x0 + nx - p0);
+      const DigitOperand bp = digit_operand(w.Bp, (long)np * nao, nao);
+      {
+        ProfScope ps("k_slice_b_fp64", s);
         DF_TRY(slice_packed(B64, ld, nao, p0, np, bp, s));
+      }
+      {
+        ProfScope ps("k_halftransform_fp64", s);
         DF_TRY(digit_half_transform(bp, ct, B64, ld, nao, p0, C, nocc, w.X, kdim, (long)(p0 - x0) * nocc, xd.key,
                                     w.err, s));
       }
     }
+    {
+      ProfScope ps("k_slice_x_fp64", s);
+      DF_TRY(slice_with_keys(w.X, kdim, xd, s));
+    }
     ProfScope ps("k_syrk_fp64", s);
-    DF_TRY(slice_with_keys(w.X, kdim, xd, s));
     const DigitSource src{w.X, kdim, 1};
     DF_TRY(digit_gemm(xd, xd, src, src, 1.0, x0 ? 1.0 : 0.0, w.Kpart, nao, (long)nao * nao, w.nsplit, DIGIT_LOWER, w.err,
                       s));
