@@ -153,10 +153,11 @@ __global__ void sum_partials_kernel(const float* __restrict__ part, int splits, 
   out[i] = s;
 }
 
-// G = 2 (out - Y) mask / (nvalid * 15); loss partial sums atomically into loss[0].
+// G = 2 (out - Y) mask / (nvalid * 15); the warps' parts of the loss into sum, in FP64: their order is
+// not fixed (in FP32 two runs of 4096 pairs differed by up to 2e-6).
 __global__ void mse_grad_kernel(const float* __restrict__ out, const float* __restrict__ Y,
                                 const float* __restrict__ mask, int n, float inv_count, float* __restrict__ G,
-                                float* __restrict__ loss) {
+                                double* __restrict__ sum) {
   long i = (long)blockIdx.x * blockDim.x + threadIdx.x;
   float l = 0.f;
   if (i < (long)n * NOUT) {
@@ -166,12 +167,14 @@ __global__ void mse_grad_kernel(const float* __restrict__ out, const float* __re
     l = d * d * inv_count;
   }
   l = warp_sumf(l);
-  if ((threadIdx.x & 31) == 0 && loss) atomicAdd(loss, l);
+  if ((threadIdx.x & 31) == 0) atomicAdd(sum, (double)l);
 }
 
-// db[c] = sum_r G[r][c]
-__global__ void column_sum_kernel(const float* __restrict__ G, int rows, int cols, float* __restrict__ db) {
+// db[c] = sum_r G[r][c]; with `sum`, also the finished loss.
+__global__ void column_sum_kernel(const float* __restrict__ G, int rows, int cols, float* __restrict__ db,
+                                  const double* __restrict__ sum, float* __restrict__ loss) {
   int c = blockIdx.x;
+  if (sum && c == 0 && threadIdx.x == 0) *loss = (float)*sum;
   float s = 0.f;
   for (int r = threadIdx.x; r < rows; r += blockDim.x) s += G[(size_t)r * cols + c];
   s = warp_sumf(s);
@@ -303,6 +306,7 @@ struct Work {
   float* dA;          // gradient w.r.t. the previous activation
   float* grad;        // parameter gradient (NPARAM)
   float* part;        // K ranges of a weight gradient
+  double* loss_sum;
   float* loss;
   __nv_bfloat16* Wp;  // BF16 weights of the tensor-core inference, zero-padded per layer
   int* err;           // bounded wait of the inference kernel gave up
@@ -324,6 +328,7 @@ static void layout(int n, Arena* a, Sizer* z, Work* w) {
       most = std::max(most, (size_t)grad_splits(layer_out(l), layer_in(l), n) * layer_out(l) * layer_in(l));
     TAKE(float, w->part, most);
   }
+  TAKE(double, w->loss_sum, 1);
   TAKE(float, w->loss, 1);
   TAKE(__nv_bfloat16, w->Wp, (size_t)(2 * NHID * NHID + 128 * NHID + 16 * NHID));
   TAKE(int, w->err, 1);
@@ -549,9 +554,9 @@ static int forward_bf16(const float* P, const float* X, int n, Work& w, cudaStre
 static int loss_grad(const float* P, const float* X, const float* Y, const float* mask, int n, float nvalid, Work& w,
                      cudaStream_t s) {
   DF_TRY(forward_fp32(P, X, n, w, s));
-  DF_CUDA(cudaMemsetAsync(w.loss, 0, sizeof(float), s));
+  DF_CUDA(cudaMemsetAsync(w.loss_sum, 0, sizeof(double), s));
   float inv = 1.f / (fmaxf(nvalid, 1.f) * NOUT);
-  mse_grad_kernel<<<nb((long)n * NOUT), 256, 0, s>>>(w.H[NLAYER - 1], Y, mask, n, inv, w.G, w.loss);
+  mse_grad_kernel<<<nb((long)n * NOUT), 256, 0, s>>>(w.H[NLAYER - 1], Y, mask, n, inv, w.G, w.loss_sum);
   DF_LAUNCHED("mse_grad_kernel");
   for (int l = NLAYER - 1; l >= 0; --l) {
     int fi = layer_in(l), fo = layer_out(l);
@@ -564,7 +569,8 @@ static int loss_grad(const float* P, const float* X, const float* Y, const float
       sum_partials_kernel<<<nb((long)fo * fi), 256, 0, s>>>(part, splits, fo * fi, w.grad + w_offset(l));
       DF_LAUNCHED("sum_partials_kernel");
     }
-    column_sum_kernel<<<fo, 256, 0, s>>>(w.G, n, fo, w.grad + b_offset(l));
+    column_sum_kernel<<<fo, 256, 0, s>>>(w.G, n, fo, w.grad + b_offset(l), l == NLAYER - 1 ? w.loss_sum : nullptr,
+                                         w.loss);
     DF_LAUNCHED("column_sum_kernel");
     if (l == 0) break;
     // dA = G W  [n][fi]; then G = dA * silu'(Z_{l-1})
