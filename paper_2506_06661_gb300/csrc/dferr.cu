@@ -203,6 +203,7 @@ extern "C" int df_fit_residual(const double* ao_xyz, const double* ao_exp, int n
   DF_REQUIRE(ld < (1L << 31), DF_ERR_ARG, "df_fit_residual: too many orbital pairs");
   // metric and its Cholesky factor (pivot check as in df_metric_chol)
   DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, w.L, pair_tab_boys(w.pair_tab, nao), s));
+  DF_TRY(reset_tc_errors((int*)w.subst, 1, TC_SETUP, s));
   DF_TRY(cholesky_inplace(w.L, naux, w.status, w.maxdiag, 1e-14, w.subst, s));
   int h_status = -1;
   DF_CUDA(cudaMemcpyAsync(&h_status, w.status, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -610,6 +610,7 @@ extern "C" int df_build_B(const double* ao_xyz, const double* ao_exp, int nao, c
   DF_REQUIRE(precision == DF_FP64 || naux <= 65535, DF_ERR_ARG, "df_build_B: naux > 65535 in mixed mode");
   work = aligned_work(work);
   char* subst = (char*)work + align_up(sizeof(double) * pair_tab_doubles(nao), 256);
+  DF_TRY(reset_tc_errors((int*)subst, 1, TC_SETUP, s));
   DF_TRY(build_B(ao_xyz, ao_exp, nao, aux_xyz, aux_exp, naux, L, precision, B, (double*)work, subst, s));
   return check_tc_errors((const int*)subst, 1, "df_build_B", s);
 }

@@ -41,7 +41,8 @@ int forward_substitution(double* R, long ld, long ncol, const double* L, int nau
 // Error words of the tensor-core kernels (digit products, split-BF16 GEMMs): a bounded wait that
 // gives up raises its word, and every later launch with that word skips its work.  reset before the
 // launches of a call; check reads them back (synchronising; not inside a stream capture) and
-// returns DF_ERR_TIMEOUT.  cholesky_inplace and forward_substitution keep theirs at the start of work.
+// returns DF_ERR_TIMEOUT.  cholesky_inplace and forward_substitution use the word at the start of
+// work, which their caller resets.
 enum TcUser { TC_SETUP = 1, TC_EXCHANGE = 2 };  // values of the test hook "tc_give_up"
 int reset_tc_errors(int* err, int n, TcUser user, cudaStream_t s);
 int check_tc_errors(const int* err, int n, const char* who, cudaStream_t s);

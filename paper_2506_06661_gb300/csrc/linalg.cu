@@ -97,9 +97,8 @@ __global__ void __launch_bounds__(256) dgemm_kernel(int M, int N, int K, double 
 // The same product in tiles of 16 x 8, one output per thread.  FP64 issues one warp instruction per
 // 64 clocks on each partition of an SM, so four warps fill it and a tile's time is its share of
 // the multiplications: 300^3 in 64 x 64 tiles put them on 25 of 152 SMs, 309 us; in 16 x 8 tiles
-// 722 CTAs spread over all of them (48 us are the FP64 units' own); in an SCF with 300 functions the
-// products took 309 and 236 us, now 24 and 24, with 100 functions 125, now 8.  The tiles of the
-// next 32 of K are on their way while this one's are multiplied.
+// 722 CTAs spread over all of them, 52 us (48 are the FP64 units' own); 100^3 125 us, now 11.  The
+// tiles of the next 32 of K are on their way while this one's are multiplied.
 constexpr int GS_M = 16, GS_N = 8, GS_K = 32;
 template <bool TA, bool TB>
 __global__ void __launch_bounds__(128) dgemm_small_kernel(int M, int N, int K, double alpha, const double* __restrict__ A,
@@ -301,7 +300,6 @@ size_t cholesky_bytes(int n) { return 256 + (n > CH_NB ? digit_operand_bytes(n, 
 
 int cholesky_inplace(double* A, int n, int* d_status, double* d_maxdiag, double tol, void* work, cudaStream_t s) {
   int* err = (int*)work;
-  DF_TRY(reset_tc_errors(err, 1, TC_SETUP, s));
   chol_init_kernel<<<1, 1024, 0, s>>>(A, n, d_maxdiag, d_status);
   DF_LAUNCHED("chol_init_kernel");
   for (int k0 = 0; k0 < n; k0 += CH_NB) {
@@ -404,7 +402,6 @@ int forward_substitution(double* R, long ld, long ncol, const double* L, int nau
   char* xmem = (char*)work + 256;
   char* lmem = xmem + digit_operand_bytes(cmax, FS_NBO);
   int* err = (int*)work;
-  DF_TRY(reset_tc_errors(err, 1, TC_SETUP, s));
   // R[r0.., :] -= L[r0.., k0..k0+b) R[k0..k0+b, :] over nr rows and the columns of chunk c0 (digits
   // of R's rows k0.. in x)
   auto update = [&](int r0, int nr, int k0, int b, long c0, const DigitOperand& x, const DigitOperand& l) -> int {
@@ -471,6 +468,7 @@ extern "C" int df_metric_chol(const double* aux_xyz, const double* aux_exp, int 
   DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, L, (double*)((char*)work + 512), s));
   if (M_out) DF_CUDA(cudaMemcpyAsync(M_out, L, sizeof(double) * naux * naux, cudaMemcpyDeviceToDevice, s));
   void* chol = (char*)work + 512 + sizeof(double) * align_up(boys_table_doubles(), 32);
+  DF_TRY(reset_tc_errors((int*)chol, 1, TC_SETUP, s));
   DF_TRY(cholesky_inplace(L, naux, d_status, d_maxdiag, 1e-14, chol, s));
   int h_status = -1;
   DF_CUDA(cudaMemcpyAsync(&h_status, d_status, sizeof(int), cudaMemcpyDeviceToHost, s));

@@ -196,6 +196,7 @@ extern "C" int df_lrdf_build(const double* ao_xyz, const double* ao_exp, int nao
   double* pair_tab = a.take<double>(pair_tab_doubles(nao));
   void* subst = a.take<char>(forward_substitution_bytes(B_ld(nao), naux));
   DF_TRY(launch_int2c(aux_xyz, aux_exp, naux, L, pair_tab_boys(pair_tab, nao), s, omega));
+  DF_TRY(reset_tc_errors((int*)subst, 1, TC_SETUP, s));
   DF_TRY(cholesky_inplace(L, naux, status, maxdiag, 1e-14, subst, s));
   int h = -1;
   DF_CUDA(cudaMemcpyAsync(&h, status, sizeof(int), cudaMemcpyDeviceToHost, s));

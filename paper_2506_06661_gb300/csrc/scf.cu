@@ -809,7 +809,7 @@ struct ScfMol {
   bool outputs_done = false;  // outputs already written for the current solution
   double* h_eps = nullptr;  // pinned: eigenvalues of S, then E_nuc (nao + 1 doubles); then of dm0
   int* h_ints = nullptr;    // pinned: [0] eigensolver status, [1] Cholesky status, [2, 3] error words of the
-                            // tensor-core kernels (metric and B; then the stability analysis)
+                            // tensor-core kernels ([2] of the metric and B; then both of the stability analysis)
   double* h_dav = nullptr;  // pinned: read-backs of the stability analysis
   DavState dav;
   std::vector<int> dm0_ids; // eigenvalue indices of the dm0 split (source of an async copy)
@@ -835,14 +835,16 @@ static int setup_launch(ScfMol& M) {
   DF_LAUNCHED("axpy_kernel");
   DF_TRY(launch_enuc(mol->xyz, mol->charges, mol->natm, W.enuc, s));
   DF_TRY(launch_int2c(mol->aux_xyz, mol->aux_exp, naux, W.L, pair_tab_boys(W.pair_tab, nao), s));
+  DF_TRY(reset_tc_errors((int*)W.subst, 1, TC_SETUP, s));
   DF_TRY(cholesky_inplace(W.L, naux, W.chol_status, W.maxdiag, 1e-14, W.subst, s));
-  DF_CUDA(cudaMemcpyAsync(M.h_ints + 2, W.subst, sizeof(int), cudaMemcpyDeviceToHost, s));  // its error word
   DF_TRY(build_B(mol->ao_xyz, mol->ao_exp, nao, mol->aux_xyz, mol->aux_exp, naux, W.L, M.opt.precision, W.B,
                  W.pair_tab, W.subst, s));
-  DF_CUDA(cudaMemcpyAsync(M.h_ints + 3, W.subst, sizeof(int), cudaMemcpyDeviceToHost, s));
   DF_CUDA(cudaMemcpyAsync(W.T1, W.S, sizeof(double) * nn, cudaMemcpyDeviceToDevice, s));
   DF_TRY(eig_rows(W.T1, nao, W.eps, W.ZT, W, s));
+  // all read-backs at the end: a copy between the kernels holds up the other molecules' queues behind
+  // it (one after the metric and one after B: 256 molecules 12.4 -> 16.6 s)
   DF_CUDA(cudaMemcpyAsync(M.h_eps, W.eps, sizeof(double) * nao, cudaMemcpyDeviceToHost, s));
+  DF_CUDA(cudaMemcpyAsync(M.h_ints + 2, W.subst, sizeof(int), cudaMemcpyDeviceToHost, s));
   DF_CUDA(cudaMemcpyAsync(M.h_ints, W.eig_status, sizeof(int), cudaMemcpyDeviceToHost, s));
   DF_CUDA(cudaMemcpyAsync(M.h_ints + 1, W.chol_status, sizeof(int), cudaMemcpyDeviceToHost, s));
   DF_CUDA(cudaMemcpyAsync(M.h_eps + nao, W.enuc, sizeof(double), cudaMemcpyDeviceToHost, s));
@@ -924,8 +926,7 @@ static int setup_orthogonalize(ScfMol& M) {
   const int nao = M.nao, nocc = M.nocc;
   const long nn = (long)nao * nao;
   M.res.e_nuc = M.h_eps[nao];
-  DF_REQUIRE(!(M.h_ints[2] | M.h_ints[3]), DF_ERR_TIMEOUT,
-             "scf: a bounded wait of the tensor-core kernels gave up in the metric or in B");
+  DF_REQUIRE(!M.h_ints[2], DF_ERR_TIMEOUT, "scf: a bounded wait of the tensor-core kernels gave up in the metric or in B");
   DF_REQUIRE(M.h_ints[1] < 0, DF_ERR_NOT_SPD, "scf: auxiliary metric not positive definite at pivot %d", M.h_ints[1]);
   DF_REQUIRE(M.h_ints[0] != 3, DF_ERR_TIMEOUT, "scf: a grid barrier of the eigensolver timed out on S");
   DF_REQUIRE(M.h_ints[0] == 0, DF_ERR_NOCONV, "scf: eigensolver failed on S");
