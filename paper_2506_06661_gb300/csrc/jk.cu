@@ -365,8 +365,8 @@ __global__ void ksum_mirror_kernel(const double* __restrict__ Kpart, int nsplit,
 // Block sizes of the FP64 exchange.  Each half-transform launch should fill the GPU for whole waves
 // of 128-row tiles (pb), and each SYRK launch should have a long K (px), within 1 GB of X and its
 // digits and within 64 splits of 4096 stages.  The digits of a wave's rows of B take more than B itself
-// in small molecules, and every molecule of a batch holds them: four waves where they fit in half of
-// B and 512 MB, two where they fit in 5/4 of it, else one.  Four waves, two, one (MB of workspace,
+// in small molecules, and every molecule of a batch holds them: four or three waves where they fit in
+// half of B and 540 MB, two where they fit in 5/4 of it, else one.  Four waves, two, one (MB of workspace,
 // ms): 20 centres 52, 52, 37 MB, 0.18, 0.18, 0.19 ms; 40 centres 280, 170, 116 MB, 0.61, 0.63, 0.67
 // ms; 63 centres 566, 389, 302 MB, 1.64, 1.70, 1.85 ms; 100 centres 1399, 1134, 997 MB, 7.9, 8.1, 8.0
 // ms; 200 centres (100 columns: half the rows a wave) 1605, 1381 MB, 69.4, 72.7 ms.
@@ -375,10 +375,9 @@ static void fp64_k_blocks(int nao, int naux, int nocc, Fp64KWork* w) {
   const size_t bytes_b = digits::plane_bytes(nao, nao), bytes_x = (size_t)nao * nocc * (2 * digits::NS + 8);
   const size_t bytes_B = sizeof(double) * (size_t)B_ld(nao) * naux;
   auto waves = [&](long n) { return std::max(1L, std::min(n * 152 * digits::BM / coltiles / nao, (long)naux)); };
-  auto fits = [&](long pb, size_t most) { return (size_t)pb * bytes_b <= std::min(most, (size_t)512 << 20); };
-  long pb = waves(4);
-  if (!fits(pb, bytes_B / 2)) pb = waves(2);
-  if (!fits(pb, bytes_B / 4 * 5)) pb = waves(1);
+  auto fits = [&](long n, size_t most) { return (size_t)waves(n) * bytes_b <= std::min(most, (size_t)540000000); };
+  const long n = fits(4, bytes_B / 2) ? 4 : fits(3, bytes_B / 2) ? 3 : fits(2, bytes_B / 4 * 5) ? 2 : 1;
+  long pb = waves(n);
   if (knob("fp64_k_pb") > 0) pb = std::min(knob("fp64_k_pb"), naux);
   long px = std::max(pb, (long)((1ul << 30) / bytes_x) / pb * pb);
   px = std::min(px, std::max(1L, 64L * 4096 * digits::BK / nocc));
