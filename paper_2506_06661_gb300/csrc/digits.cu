@@ -9,7 +9,8 @@
 // on the other: the groups run 64-term chunks staggered by one 32-term stage, so each stage is
 // used by both groups back to back and two 84 KB stages suffice.
 // FP64 exchange at nao 1000, naux 3000, nocc 100: 914 ms with FP64 FMAs (0.99 TFLOP/s, 0.8 of the
-// FP64 peak), 65 ms here: slicing 27 ms, the two contractions 38 ms.
+// FP64 peak), 70 ms here: slicing 28 ms, the two contractions 42 ms.  At nao 1500, naux 4500, nocc
+// 150 the half-transform issues 0.51 and the SYRK 0.53 of the sustained BF16 rate.
 #include <algorithm>
 #include <climits>
 #include <type_traits>

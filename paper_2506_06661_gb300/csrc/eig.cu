@@ -11,8 +11,8 @@
 // All of these are textbook algorithms (Householder 1958; QL with implicit shifts as
 // in Bowdler, Martin, Reinsch and Wilkinson 1968) written here for a thread block.
 //
-// eigh_lowest, start to end: n = 100, k = 11 3.1 ms on one CTA -> 0.57; 300, 31 6.1 -> 1.9;
-// 900, 91 23.4 -> 8.6.  Full spectra: n = 30 2.4 ms (QL) -> 0.26; 100 22.5 -> 0.6; 300 21 -> 2.5.
+// eigh_lowest, start to end: n = 100, k = 11 3.1 ms on one CTA -> 0.59; 300, 31 6.1 -> 2.1;
+// 900, 91 23.4 -> 10.0.  Full spectra: n = 30 2.4 ms (QL) -> 0.26; 100 22.5 -> 0.63; 300 21 -> 2.6.
 #include <algorithm>
 #include <cfloat>
 

@@ -17,9 +17,10 @@
 // CTA leaves when it has no row left to publish, before it reads.  Waits are bounded.
 //
 // Device time against two block reductions, square root and division on every warp and a grid
-// barrier per step: n = 100 1.66 (one CTA) -> 0.31 ms, n = 300 2.29 -> 1.31 ms, n = 900 9.47 -> 6.9 ms.
-// A step takes about 3 us at n = 100, of which 1.2 are chains of FP64 additions across lanes; at
-// n = 900 7.7 us, half of them the packets' way through L2 (152 CTAs read 900 each).
+// barrier per step: n = 100 1.66 (one CTA) -> 0.34 ms, n = 300 2.29 -> 1.54 ms, n = 900 9.47 -> 8.25 ms
+// (6.9 with the update rounded twice, see rank2).  A step takes about 3 us at n = 100, of which 1.2
+// are chains of FP64 additions across lanes; at n = 900 9.2 us, 4 of them the packets' way through
+// L2 (152 CTAs read 900 each), the rest the FP64 pass over the rows.
 #include <algorithm>
 
 #include "fp64.cuh"
@@ -193,8 +194,8 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
   const int nrows = (n - 1 - cta) / G + 1, last_row = (nrows - 1) * G + cta;
   bool lost = false;
   unsigned it = 0;
-  // A wait ends after `limit` polls, or two seconds: a poll takes a microsecond, and several when
-  // every CTA of a full grid polls.
+  // A wait ends after `limit` polls, or two seconds and 0.1 ms a row after the kernel's start: a poll
+  // takes a microsecond, and several when every CTA of a full grid polls.
   const unsigned long long t0 = global_ns();
   auto tired = [&]() {
     const bool look = (++it & 255u) == 0u;
@@ -406,8 +407,9 @@ TridiagPlan tridiag_plan(int n, int forced) {
   if (cudaGetDevice(&dev) != cudaSuccess) return P;
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // More CTAs shorten the pass over the rows and lengthen the exchange.  All of eigh_lowest, us:
-  // n = 100: 8 CTAs 634, 16 582, 25 567, 50 627; 200: 16 1311, 32 1141, 50 1121, 100 1191;
-  // 300: 25 2183, 50 1905, 100 1955, 152 2128; 450: 50 3374, 100 3029, 152 3207; 900: 152 8642.
+  // n = 100: 8 CTAs 651, 16 592, 25 588, 50 596; 200: 16 1424, 32 1237, 50 1235, 100 1315;
+  // 300: 25 2442, 50 2161, 100 2112, 152 2296; 450: 50 3879, 100 3535, 152 3440; 900: 100 10973,
+  // 152 10051.
   int G = forced > 1 ? forced : std::min(sms, std::max(16, n / 5));
   G = std::min(G, n);
   const int R = (n + G - 1) / G;

@@ -16,13 +16,14 @@
 //   3. reflectors in panels of 16: z -= V (T (V^T z));
 //   4. Z <- Z - (Z Z^T - 1) Z / 2, three times when the vectors need it.
 // Eigenvalues equal to rounding are told apart by the blocks into which T falls, each with the
-// eigenvalue of its own block, and inside a block by inverse iteration with projections.  What that cannot repair is left to inverse iteration
-// and Gram-Schmidt over the whole matrix, or to implicit QL (eig.cu).
+// eigenvalue of its own block, and inside a block by inverse iteration with projections.  What that
+// cannot repair is left to inverse iteration and Gram-Schmidt over the whole matrix, or to implicit
+// QL (eig.cu).
 // Device time at n = 900, k = 91 against 33-way bisection with a division a step, inverse iteration
 // from global memory, one reflector at a time and Gram-Schmidt with five grid barriers a vector:
-// eigenvalues 5.2 -> 0.57 ms, eigenvectors 3.1 -> 0.23, back-transformation 2.5 -> 0.71,
-// orthonormalisation 3.0 -> 0.08; at n = 100, k = 11 (one CTA before) 936 -> 85 us, 213 -> 35,
-// 112 -> 32, 100 -> 25.
+// eigenvalues 5.2 -> 0.57 ms, eigenvectors 3.1 -> 0.36 (0.23 without the correction),
+// back-transformation 2.5 -> 0.71, orthonormalisation 3.0 -> 0.07; at n = 100, k = 11 (one CTA before)
+// 936 -> 72 us, 213 -> 52, 112 -> 32, 100 -> 22.
 #include <algorithm>
 #include <cfloat>
 
@@ -691,7 +692,7 @@ __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const dou
   __syncthreads();
   // ---- correction: (T - l) y = (T - l) z - delta z without row r, y_r = 0, delta = z.(T - l) z ----------
   // z's components along its neighbours, 1.4e-14 for the 90 lowest of 900 rows where inverse iteration
-  // left 4e-15, become negligible (the residual of a rounded z); 0.06 ms of 0.23 at 900 rows.
+  // left 4e-15, become negligible (the residual of a rounded z).
   double c = 0.0;
   for (int i = tid; i < nb; i += NT) {
     const double b = residual_row(Tb, e + i0, scale, nb, l, p, i);
