@@ -1004,9 +1004,10 @@ constexpr int kMultiSm = 8;
 constexpr int kQlMax = 160;
 
 // k lowest eigenpairs (full: k = n, the whole spectrum asked for).  aux: eigh_coop_aux_bytes(n)
-// of scratch for the multi-SM path; *done is false when only the one-CTA kernels apply.
+// of scratch for the multi-SM path; exact: see tridiag.cu; *done is false when only the one-CTA kernels
+// apply.
 int eigh_multi_sm(double* A, int n, int k, bool full, double* w, double* ZT, double* scratch, int* status,
-                  cudaStream_t s, void* aux, bool* done) {
+                  cudaStream_t s, void* aux, bool exact, bool* done) {
   *done = false;
   const int forced = knob("eig_ctas");
   if (!aux || forced == 1 || (forced == 0 && n < kMultiSm) || n < 3) return DF_OK;
@@ -1018,7 +1019,7 @@ int eigh_multi_sm(double* A, int n, int k, bool full, double* w, double* ZT, dou
   double* part = (double*)p;
   p += align_up(sizeof(double) * kCoopMaxCtas, 256);
   EigControl* ctl = (EigControl*)p;
-  const TridiagPlan T = tridiag_plan(n, forced);
+  const TridiagPlan T = tridiag_plan(n, forced, exact);
   const CoopPlan F = coop_plan((const void*)eigh_fallback_coop_kernel, n, k, 0);
   const bool fast = T.G > 0 && F.G > 0 && trivec_fits(n);
   CoopPlan C;
@@ -1035,7 +1036,8 @@ int eigh_multi_sm(double* A, int n, int k, bool full, double* w, double* ZT, dou
                        status));
   } else {
     DF_TRY(tridiag_launch(A, n, scratch, scratch + n, scratch + 2 * (size_t)n, T, exchange, ctl, s));
-    DF_TRY(trivec_launch(A, n, k, scratch, scratch + n, scratch + 2 * (size_t)n, w, ZT, scratch + 4 * (size_t)n, ctl, s));
+    DF_TRY(trivec_launch(A, n, k, scratch, scratch + n, scratch + 2 * (size_t)n, w, ZT, scratch + 4 * (size_t)n, exact,
+                         ctl, s));
     if (full && n < kQlMax) {
       eigh_fallback_ql_kernel<<<1, 1024, 0, s>>>(A, n, w, ZT, scratch, ctl, status);
       DF_LAUNCHED("eigh_fallback_ql_kernel");
@@ -1050,9 +1052,9 @@ int eigh_multi_sm(double* A, int n, int k, bool full, double* w, double* ZT, dou
 }  // namespace
 
 int eigh_lowest_rows(double* A, int n, int k, double* w, double* ZT, double* scratch, int* status, cudaStream_t s,
-                     void* aux) {
+                     void* aux, bool exact) {
   bool done = false;
-  DF_TRY(eigh_multi_sm(A, n, k, false, w, ZT, scratch, status, s, aux, &done));
+  DF_TRY(eigh_multi_sm(A, n, k, false, w, ZT, scratch, status, s, aux, exact, &done));
   if (done) return DF_OK;
   eigh_lowest_kernel<<<1, 1024, 0, s>>>(A, n, k, w, ZT, scratch, status);
   DF_LAUNCHED("eigh_lowest_kernel");
@@ -1066,9 +1068,9 @@ size_t eigh_full_scratch_doubles(int n) {
 // Full spectrum: the multi-SM solver with k = n where it applies (aux given, n large enough),
 // else one CTA with implicit QL.  scratch: eigh_full_scratch_doubles(n).
 int eigh_full_rows(double* A, int n, double* w, double* ZT, double* scratch, int* status, cudaStream_t s,
-                   void* aux) {
+                   void* aux, bool exact) {
   bool done = false;
-  DF_TRY(eigh_multi_sm(A, n, n, true, w, ZT, scratch, status, s, aux, &done));
+  DF_TRY(eigh_multi_sm(A, n, n, true, w, ZT, scratch, status, s, aux, exact, &done));
   if (done) return DF_OK;
   return eigh_rows(A, n, w, ZT, scratch, status, s);
 }
@@ -1102,7 +1104,7 @@ extern "C" int df_eigh(double* A, int n, double* w, double* Z, void* work, size_
   double* ZT = a.take<double>((size_t)n * n);
   int* status = a.take<int>(1);
   void* aux = a.take<char>(eigh_coop_aux_bytes(n));
-  DF_TRY(eigh_full_rows(A, n, w, ZT, scratch, status, s, aux));
+  DF_TRY(eigh_full_rows(A, n, w, ZT, scratch, status, s, aux, true));
   DF_TRY(transpose(ZT, n, n, Z, s));
   int h = 0;
   DF_CUDA(cudaMemcpyAsync(&h, status, sizeof(int), cudaMemcpyDeviceToHost, s));
@@ -1132,7 +1134,7 @@ extern "C" int df_eigh_lowest(double* A, int n, int k, double* w, double* Z, voi
   double* ZT = a.take<double>((size_t)n * k);
   int* status = a.take<int>(1);
   void* aux = a.take<char>(eigh_coop_aux_bytes(n));
-  DF_TRY(eigh_lowest_rows(A, n, k, w, ZT, scratch, status, s, aux));
+  DF_TRY(eigh_lowest_rows(A, n, k, w, ZT, scratch, status, s, aux, true));
   DF_TRY(transpose(ZT, k, n, Z, s));
   int h = 0;
   DF_CUDA(cudaMemcpyAsync(&h, status, sizeof(int), cudaMemcpyDeviceToHost, s));

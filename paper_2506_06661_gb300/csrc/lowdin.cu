@@ -63,7 +63,7 @@ extern "C" int df_lowdin_factors(const double* ao_xyz, const double* ao_exp, int
   void* aux = a.take<char>(eigh_coop_aux_bytes(nao));
   const long nn = (long)nao * nao;
   DF_TRY(launch_int1e(ao_xyz, ao_exp, nao, nullptr, nullptr, 0, S, nullptr, nullptr, s));
-  DF_TRY(eigh_full_rows(S, nao, w, ZT, scr, status, s, aux));
+  DF_TRY(eigh_full_rows(S, nao, w, ZT, scr, status, s, aux, true));
   // S^p = sum_k u_k s_k^p u_k^T = ZT^T diag(s^p) ZT
   if (Shalf) {
     scaled_rows_kernel<<<nblk(nn), 256, 0, s>>>(ZT, w, nao, lindep, 0.5, W);

@@ -608,6 +608,7 @@ struct ScfWork {
   size_t guess_bytes;
   char* subst;    // digits of the whitening
   void* eig_aux;  // p vector and grid barrier of the multi-SM eigensolver
+  bool eig_exact = false;  // its rounding: df_core_guess sets it, the iterations need no more than the faster one
   ScfStatus* st;
   DiisState* diis;
   void* B;
@@ -713,7 +714,7 @@ static void scf_layout(int nao, int naux, int nocc, int precision, Arena* a, Siz
 }
 
 static int eig_rows(double* A, int n, double* w, double* ZT, ScfWork& W, cudaStream_t s) {
-  return eigh_full_rows(A, n, w, ZT, W.eig_scratch, W.eig_status, s, W.eig_aux);
+  return eigh_full_rows(A, n, w, ZT, W.eig_scratch, W.eig_status, s, W.eig_aux, W.eig_exact);
 }
 
 // Occupied orbitals of the orthogonal-basis Fock matrix W.Fp [nmo][nmo] (destroyed):
@@ -724,7 +725,7 @@ static int diagonalize_orth(int nao, int nmo, int nocc, ScfWork& W, cudaStream_t
   {
     ProfScope ps("scf_eigensolver", s);
     if (nmo >= 16 && 2 * k <= nmo)
-      DF_TRY(eigh_lowest_rows(W.Fp, nmo, k, W.eps, W.ZT, W.eig_scratch, W.eig_status, s, W.eig_aux));
+      DF_TRY(eigh_lowest_rows(W.Fp, nmo, k, W.eps, W.ZT, W.eig_scratch, W.eig_status, s, W.eig_aux, W.eig_exact));
     else
       DF_TRY(eig_rows(W.Fp, nmo, W.eps, W.ZT, W, s));
   }
@@ -1052,7 +1053,7 @@ static int incremental_prep(ScfMol& M) {
   ProfScope ps_inc("scf_incremental_prep", s);
   DF_TRY(dgemm(true, false, nocc, nocc, nmo, 1.0, W.Cbase, nocc, 0, W.Cp, nocc, 0, 0.0, W.Minc, nocc, 0, 1, s, 0, 0));
   DF_TRY(dgemm(true, false, nocc, nocc, nocc, 1.0, W.Minc, nocc, 0, W.Minc, nocc, 0, 0.0, W.Tinc, nocc, 0, 1, s, 0, 0));
-  DF_TRY(eigh_full_rows(W.Tinc, nocc, W.cinc, W.Winc, W.eig_scratch, W.inc_status, s, W.eig_aux));
+  DF_TRY(eigh_full_rows(W.Tinc, nocc, W.cinc, W.Winc, W.eig_scratch, W.inc_status, s, W.eig_aux, W.eig_exact));
   inc_status_kernel<<<1, 256, 0, s>>>(W.cinc, nocc, W.inc_status, W.st);
   DF_LAUNCHED("inc_status_kernel");
   return DF_OK;
@@ -1079,7 +1080,7 @@ static int soscf_init(ScfMol& M) {
   const int nmo = M.nmo;
   const long ne = (long)nmo * nmo;
   DF_CUDA(cudaMemcpyAsync(W.Fp, W.Fbar, sizeof(double) * ne, cudaMemcpyDeviceToDevice, s));
-  DF_TRY(eigh_full_rows(W.Fp, nmo, W.eps, W.ZT, W.eig_scratch, W.eig_status, s, W.eig_aux));
+  DF_TRY(eigh_full_rows(W.Fp, nmo, W.eps, W.ZT, W.eig_scratch, W.eig_status, s, W.eig_aux, W.eig_exact));
   DF_TRY(transpose(W.ZT, nmo, nmo, W.Call, s));
   DF_TRY(occupied_from_all(M));
   if (M.inc) DF_TRY(incremental_prep(M));
@@ -1177,7 +1178,7 @@ static int rotate_orbitals(ScfMol& M) {
   const int nmo = M.nmo, nocc = M.nocc, nvir = nmo - nocc;
   const long ne = (long)nmo * nmo;
   DF_TRY(dgemm(true, false, nocc, nocc, nvir, 1.0, W.cg_x, nocc, 0, W.cg_x, nocc, 0, 0.0, W.kk, nocc, 0, 1, s, 0, 0));
-  DF_TRY(eigh_full_rows(W.kk, nocc, W.ksig, W.kVrow, W.eig_scratch, W.k_status, s, W.eig_aux));
+  DF_TRY(eigh_full_rows(W.kk, nocc, W.ksig, W.kVrow, W.eig_scratch, W.k_status, s, W.eig_aux, W.eig_exact));
   rotation_mats_kernel<<<blocks_for((long)nocc * nocc), 256, 0, s>>>(W.kVrow, W.ksig, nocc, W.Pc, W.Ps, W.Pd);
   DF_LAUNCHED("rotation_mats_kernel");
   // occupied: C'_o Pc + C'_v (k Ps)
@@ -1451,7 +1452,7 @@ static int dav_begin(ScfMol& M, double mode_scale) {
   if (nvo <= 0) return DF_OK;  // stage stays OFF: nothing to analyse
   // canonical orbitals of the last Fock matrix F' (W.Fo)
   DF_CUDA(cudaMemcpyAsync(W.Fp, W.Fo, sizeof(double) * ne, cudaMemcpyDeviceToDevice, s));
-  DF_TRY(eigh_full_rows(W.Fp, nmo, W.eps, W.ZT, W.eig_scratch, W.eig_status, s, W.eig_aux));
+  DF_TRY(eigh_full_rows(W.Fp, nmo, W.eps, W.ZT, W.eig_scratch, W.eig_status, s, W.eig_aux, W.eig_exact));
   DF_TRY(transpose(W.ZT, nmo, nmo, W.Call, s));
   DF_TRY(occupied_from_all(M));
   DF_TRY(dgemm(false, false, nmo, nmo, nmo, 1.0, W.Fo, nmo, 0, W.Call, nmo, 0, 0.0, W.T1, nmo, 0, 1, s, 0, 0));
@@ -2451,6 +2452,7 @@ extern "C" int df_core_guess(const df_molecule* mol, double lindep, double* S_ou
   Arena a(work, work_bytes);
   ScfWork W;
   guess_layout(nao, nocc, &a, nullptr, &W);
+  W.eig_exact = true;
   const long nn = (long)nao * nao;
   DF_TRY(launch_int1e(mol->ao_xyz, mol->ao_exp, nao, mol->xyz, mol->charges, mol->natm, W.S, W.h, W.V, s));
   axpy_kernel<<<blocks_for(nn), 256, 0, s>>>(W.h, W.V, nn, 1.0);

@@ -18,7 +18,7 @@
 //
 // Device time against two block reductions, square root and division on every warp and a grid
 // barrier per step: n = 100 1.66 (one CTA) -> 0.34 ms, n = 300 2.29 -> 1.54 ms, n = 900 9.47 -> 8.25 ms
-// (6.9 with the update rounded twice, see rank2).  A step takes about 3 us at n = 100, of which 1.2
+// (6.9 without EXACT).  A step takes about 3 us at n = 100, of which 1.2
 // are chains of FP64 additions across lanes; at n = 900 9.2 us, 4 of them the packets' way through
 // L2 (152 CTAs read 900 each), the rest the FP64 pass over the rows.
 #include <algorithm>
@@ -71,17 +71,21 @@ __device__ __forceinline__ void bar(int id, int threads) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
 }
 
-// v_i w_j + w_i v_j.  Rounded before it is subtracted: two FMAs into the element, one instruction
-// less, round it twice at its own size: the 90 lowest vectors of 900 rows span a space 1.7e-14 off
-// instead of 1.2e-14 (20 random matrices; one thread block and inverse iteration: 1.3e-14), and
-// eigh_lowest takes 9.3 ms instead of 10.0.
+// Two roundings of the same reduction.  EXACT (the eigensolver's own entry points): the update
+// v_i w_j + w_i v_j is rounded before it is subtracted, w carries the factor b, and the reflector's
+// norm and b are good to half an ulp.  Otherwise (the iterations of an SCF): the update is two FMAs into
+// the element, which round it twice at its own size, v carries b, and norm and b are good to one or
+// two ulps.  Space of the 90 lowest of 900 rows, with the vectors of trivec.cu, geometric mean over 20
+// random matrices: 1.2e-14 off and 10.0 ms against 2.3e-14 and 9.0 (inverse iteration on one thread
+// block: 1.3e-14).  An SCF's density is determined to 1e-10 by its thresholds, and it is 2 to 6%
+// faster with the second.
 __device__ __forceinline__ double rank2(double vi, double wj, double wi, double vj) { return fma(vi, wj, wi * vj); }
 
 // One pass over S owned rows (slots s0 .. s0 + S - 1, global rows from r0 in steps of G): the
 // pending update, y = row . x, and the entry of column kk + 1.  The S sums are
 // reduced together: P - 1 + log2(32 / P) additions (P = S rounded up to a power of two) instead
 // of 5 S.
-template <int S>
+template <int S, bool EXACT>
 __device__ __forceinline__ void rows_pass(double* __restrict__ rows, int n, int s0, int r0, int G, int kk,
                                           const double* __restrict__ x, const double* __restrict__ vp,
                                           const double* __restrict__ wt, double* red, int R, double* cnew) {
@@ -112,9 +116,13 @@ __device__ __forceinline__ void rows_pass(double* __restrict__ rows, int n, int 
     const int next = col + HALF;
     double xn = 0.0, vn = 0.0, wn = 0.0, an[S];
     if (next < n) fetch(next, xn, vn, wn, an);
+    if (!EXACT) {
+#pragma unroll
+      for (int s = 0; s < S; ++s) a[s] = fma(-vr[s], wc, a[s]);
+    }
 #pragma unroll
     for (int s = 0; s < S; ++s) {
-      a[s] -= rank2(vr[s], wc, wr[s], vc);
+      a[s] = EXACT ? a[s] - rank2(vr[s], wc, wr[s], vc) : fma(-wr[s], vc, a[s]);
       row[(size_t)s * n + col] = a[s];
     }
 #pragma unroll
@@ -147,11 +155,12 @@ __device__ __forceinline__ void rows_pass(double* __restrict__ rows, int n, int 
   if (lane % W == 0 && lane / W < S) red[wid * R + s0 + lane / W] = acc[0];
 }
 
+template <bool EXACT>
 __device__ __forceinline__ void all_rows(double* rows, int n, int s0, int s1, int cta, int G, int kk, const double* x,
                                          const double* vp, const double* wt, double* red, int R, double* cnew) {
 #define DF_PASS(S)                                                                          \
   case S:                                                                                   \
-    rows_pass<S>(rows, n, s0, s0 * G + cta, G, kk, x, vp, wt, red, R, cnew);                \
+    rows_pass<S, EXACT>(rows, n, s0, s0 * G + cta, G, kk, x, vp, wt, red, R, cnew);         \
     break
   for (; s0 < s1; s0 += 8) switch (min(s1 - s0, 8)) {
       DF_PASS(1);
@@ -170,12 +179,12 @@ __device__ __forceinline__ void all_rows(double* rows, int n, int s0, int s1, in
 // there is one vp and red and cnew lie in cn: the reflector half then waits for the pass over the
 // rows before it writes vp, and the row half for itself before it writes cn.  NC: columns per thread
 // whose packets are in flight together.
-template <int NC>
+template <int NC, bool EXACT>
 __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict__ A, int n, double* __restrict__ d,
                                                              double* __restrict__ e, double* __restrict__ beta, int R,
                                                              int vps, Packet* ex, EigControl* ctl) {
   extern __shared__ double smem_d[];
-  __shared__ double sh_sigma[4], sh_pv[4], sh_ref[4];
+  __shared__ double sh_sigma[4], sh_pv[4], sh_ref[5];
   __shared__ int give_up;
   __shared__ unsigned sh_top;
   if (NC < 8) vps = 2;  // the plan takes one vp for large n only
@@ -183,7 +192,7 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
   const int t = tid & (HALF - 1), lane = tid & 31, wid = t >> 5;
   const bool reflector_half = tid >= HALF;
   double* x = smem_d;         // current column, rows kk + 1 ..
-  double* v2 = smem_d + n;    // the pending update is A -= v wt^T + wt v^T, wt = b (A v - kap v); by parity
+  double* v2 = smem_d + n;    // the pending update is A -= v2 wt^T + wt v2^T; by parity
   double* wt = v2 + vps * (size_t)n;
   double* cn = wt + n;  // the next column before this step's update
   double* rows = cn + n;
@@ -273,19 +282,19 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
         if (__double_as_longlong(sigma) != 0) {
           const double n2 = fma(x0, x0, sigma);
           const bool fast = ordinary(n2);
-          // both rounded to half an ulp: what they miss, the reflector is short of orthogonal
           const double rs = fast ? rsqrt_ordinary(n2) : 0.0, nr = n2 * rs;
-          const double nrm = fast ? fma(fma(-nr, nr, n2), 0.5 * rs, nr) : sqrt(n2);
+          const double nrm = !fast ? sqrt(n2) : EXACT ? fma(fma(-nr, nr, n2), 0.5 * rs, nr) : nr;
           alpha = __double2hiint(x0) >= 0 ? -nrm : nrm;
           v0 = x0 - alpha;
           const double vv = fma(v0, v0, sigma), rc = fast ? rcp_ordinary(vv) : 0.0;
-          b = fast ? 2.0 * fma(fma(-vv, rc, 1.0), rc, rc) : 2.0 / vv;
+          b = !fast ? 2.0 / vv : EXACT ? 2.0 * fma(fma(-vv, rc, 1.0), rc, rc) : 2.0 * rc;
         }
         if (lane == 0) {
           sh_ref[0] = alpha;
           sh_ref[1] = b;
           sh_ref[2] = v0;
           sh_ref[3] = 0.5 * b;
+          sh_ref[4] = EXACT ? v0 : b * v0;
           if (writer) {
             A[(size_t)kk * n + kk + 1] = v0;
             e[kk] = alpha * up;
@@ -298,7 +307,7 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
       for (int col = base + t; col < n; col += HALF)
         if (col >= c1) {
           const double v = x[col];
-          vn[col] = v;
+          vn[col] = EXACT ? v : sh_ref[1] * v;
           if (writer) A[(size_t)kk * n + col] = v;
         }
       bar(3, 2 * HALF);
@@ -311,7 +320,7 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
     const unsigned tag = (unsigned)(kk + 1), want = tag + off_tag;
     Packet* buf = ex + (size_t)(kk & 1) * n;
     if (s0 * G + cta <= kk) ++s0;
-    all_rows(rows, n, s0, nrows, cta, G, kk, x, vp, wt, red, R, cnew);
+    all_rows<EXACT>(rows, n, s0, nrows, cta, G, kk, x, vp, wt, red, R, cnew);
     bar(1, HALF);
     for (int s = s0 + t; s < nrows; s += HALF) {
       const double y = (red[s] + red[R + s]) + (red[2 * R + s] + red[3 * R + s]);
@@ -361,17 +370,17 @@ __global__ void __launch_bounds__(2 * HALF, 1) tridiag_kernel(double* __restrict
     if (lane == 0) sh_pv[wid] = pv;
     bar(1, HALF);
     pv = (sh_pv[0] + sh_pv[1]) + (sh_pv[2] + sh_pv[3]);
-    // ---- 3. w = b (A v - (b/2)(v.Av) v) and the next column -------------------------------------------
-    const double b = sh_ref[1], v0 = sh_ref[2];
+    // ---- 3. w = A v - (b/2)(v.Av) v and the next column -------------------------------------------
+    const double b = sh_ref[1], v0 = sh_ref[2], u0 = sh_ref[4];
     const double av0 = fma(-alpha, d0, y0), kap = sh_ref[3] * fma(av0, v0, pv);
-    const double w0 = b * fma(-kap, v0, av0);
+    const double w0 = EXACT ? b * fma(-kap, v0, av0) : fma(-kap, v0, av0);
     for (int col = base + t; col < n; col += HALF)
       if (col >= c1) {
-        const double v = x[col], w = b * fma(-kap, v, wt[col]);
+        const double v = x[col], w1 = fma(-kap, v, wt[col]), w = EXACT ? b * w1 : w1;
         wt[col] = w;
-        x[col] = cn[col] - rank2(v, w0, w, v0);
+        x[col] = EXACT ? cn[col] - rank2(v, w0, w, v0) : fma(-u0, w, fma(-vn[col], w0, cn[col]));
       }
-    if (writer && tid == 0) d[kk + 1] = up * fma(-2.0 * v0, w0, d0);
+    if (writer && tid == 0) d[kk + 1] = up * fma(-2.0 * u0, w0, d0);
     if (lost) give_up = 1;
     bar(3, 2 * HALF);
     if (give_up) return;
@@ -394,14 +403,17 @@ size_t smem_of(int n, int R, int vps) {
 
 namespace {
 using Kernel = void (*)(double*, int, double*, double*, double*, int, int, Packet*, EigControl*);
-Kernel kernel_of(int n) {
-  return n <= HALF ? tridiag_kernel<1> : n <= 2 * HALF ? tridiag_kernel<2> : n <= 4 * HALF ? tridiag_kernel<4> : tridiag_kernel<8>;
+template <bool EXACT>
+Kernel kernel_for(int n) {
+  return n <= HALF ? tridiag_kernel<1, EXACT>
+                   : n <= 2 * HALF ? tridiag_kernel<2, EXACT> : n <= 4 * HALF ? tridiag_kernel<4, EXACT> : tridiag_kernel<8, EXACT>;
 }
+Kernel kernel_of(int n, bool exact) { return exact ? kernel_for<true>(n) : kernel_for<false>(n); }
 }  // namespace
 
 size_t tridiag_exchange_bytes(int n) { return 2 * sizeof(Packet) * (size_t)n; }
 
-TridiagPlan tridiag_plan(int n, int forced) {
+TridiagPlan tridiag_plan(int n, int forced, bool exact) {
   TridiagPlan P;
   int dev = 0, sms = 0, per_sm = 0;
   if (cudaGetDevice(&dev) != cudaSuccess) return P;
@@ -418,13 +430,14 @@ TridiagPlan tridiag_plan(int n, int forced) {
   const int vps = n <= 4 * HALF || smem_of(n, R, 2) <= kSmemLimit ? 2 : 1;
   const size_t smem = smem_of(n, R, vps);
   if (smem > kSmemLimit) return P;
-  if (cudaFuncSetAttribute(kernel_of(n), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel_of(n), 2 * HALF, smem) != cudaSuccess)
+  if (cudaFuncSetAttribute(kernel_of(n, exact), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmemLimit) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel_of(n, exact), 2 * HALF, smem) != cudaSuccess)
     return P;
   if (G > sms * per_sm) return P;
   P.G = G;
   P.R = R;
   P.vps = vps;
+  P.exact = exact;
   P.smem = smem;
   return P;
 }
@@ -441,7 +454,7 @@ int tridiag_launch(double* A, int n, double* d, double* e, double* beta, const T
   attr[0].val.cooperative = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  DF_CUDA(cudaLaunchKernelEx(&cfg, kernel_of(n), A, n, d, e, beta, P.R, P.vps, (Packet*)exchange, ctl));
+  DF_CUDA(cudaLaunchKernelEx(&cfg, kernel_of(n, P.exact), A, n, d, e, beta, P.R, P.vps, (Packet*)exchange, ctl));
   return DF_OK;
 }
 

@@ -23,22 +23,23 @@ struct TridiagPlan {
   int G = 0;  // CTAs (0: the size does not fit)
   int R = 0;  // rows per CTA
   int vps = 2;  // vectors of pending updates in shared memory
+  bool exact = true;
   size_t smem = 0;
 };
 
-// forced: CTA count asked for by the caller (0: choose).
-TridiagPlan tridiag_plan(int n, int forced);
+// forced: CTA count asked for by the caller (0: choose).  exact: which rounding (tridiag.cu).
+TridiagPlan tridiag_plan(int n, int forced, bool exact);
 size_t tridiag_exchange_bytes(int n);  // zeroed by the caller before each launch
 // A [n][n] symmetric -> d, e, beta; reflector r in row r of A, columns r + 1 .. n - 1.
 int tridiag_launch(double* A, int n, double* d, double* e, double* beta, const TridiagPlan& P, void* exchange,
                    EigControl* ctl, cudaStream_t s);
 
 // The k lowest eigenpairs from the output of tridiag_launch: w [k], ZT [k][n].  Scratch:
-// trivec_scratch_doubles(n, k).  Leaves ctl->bad or ctl->emax for eig_needs_fallback.
+// trivec_scratch_doubles(n, k).  exact: the vectors are corrected once.  Leaves ctl->bad or ctl->emax for eig_needs_fallback.
 size_t trivec_scratch_doubles(int n, int k);
 bool trivec_fits(int n);
 int trivec_launch(const double* A, int n, int k, const double* d, const double* e, const double* beta, double* w,
-                  double* ZT, double* scratch, EigControl* ctl, cudaStream_t s);
+                  double* ZT, double* scratch, bool exact, EigControl* ctl, cudaStream_t s);
 
 // Re-orthonormalisation Z <- Z - (Z Z^T - 1) Z / 2 leaves 3/4 ||Z Z^T - 1||^2.
 constexpr double kOrthoDone = 1e-8;

@@ -12,7 +12,8 @@
 //      in FP64 to the last bit; a bracket that FP64 does not confirm starts over in FP64;
 //   2. minors from both ends, pivots q+ and q-, the index r with the least |q+_r + q-_r - (d_r - l)|,
 //      and z outward from z_r = 1: z_i = -(e_i / q+_i) z_{i+1} and z_{i+1} = -(e_i / q-_{i+1}) z_i;
-//      then one correction of z: its residual in twice the precision, solved with the same factors;
+//      then, where the caller wants exact vectors, one correction of z: its residual in twice the
+//      precision, solved with the same factors;
 //   3. reflectors in panels of 16: z -= V (T (V^T z));
 //   4. Z <- Z - (Z Z^T - 1) Z / 2, three times when the vectors need it.
 // Eigenvalues equal to rounding are told apart by the blocks into which T falls, each with the
@@ -502,7 +503,7 @@ __device__ __forceinline__ void chain(double* __restrict__ s, const double* __re
 __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const double* __restrict__ d,
                                                          const double* __restrict__ e, const double* __restrict__ w,
                                                          double* __restrict__ Y, double* __restrict__ wv,
-                                                         EigControl* ctl) {
+                                                         bool exact, EigControl* ctl) {
   extern __shared__ double smem_d[];
   __shared__ double sh[4];
   __shared__ unsigned shm[4];
@@ -690,6 +691,10 @@ __global__ void __launch_bounds__(NT) tri_vectors_kernel(int n, int k, const dou
   const double inv = 1.0 / sqrt(n2);
   for (int i = tid; i < nb; i += NT) p[i] *= inv;
   __syncthreads();
+  if (!exact) {
+    for (int i = tid; i < n; i += NT) Y[(size_t)t * n + i] = i >= i0 && i < i0 + nb ? p[i - i0] : 0.0;
+    return;
+  }
   // ---- correction: (T - l) y = (T - l) z - delta z without row r, y_r = 0, delta = z.(T - l) z ----------
   // z's components along its neighbours, 1.4e-14 for the 90 lowest of 900 rows where inverse iteration
   // left 4e-15, become negligible (the residual of a rounded z).
@@ -890,7 +895,7 @@ size_t trivec_scratch_doubles(int n, int k) {
 bool trivec_fits(int n) { return vectors_smem(n) <= 220 * 1024 && values_smem(n) <= 220 * 1024; }
 
 int trivec_launch(const double* A, int n, int k, const double* d, const double* e, const double* beta, double* w,
-                  double* ZT, double* scratch, EigControl* ctl, cudaStream_t s) {
+                  double* ZT, double* scratch, bool exact, EigControl* ctl, cudaStream_t s) {
   const int np = (int)panels_of(n);
   double* Tf = scratch;
   double* Y = Tf + (size_t)np * kPanel * kPanel;
@@ -901,7 +906,7 @@ int trivec_launch(const double* A, int n, int k, const double* d, const double* 
   tri_values_kernel<<<k + np, NT, values_smem(n), s>>>(A, n, k, d, e, beta, w, Tf, ctl);
   DF_LAUNCHED("tri_values_kernel");
   DF_CUDA(cudaFuncSetAttribute(tri_vectors_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
-  tri_vectors_kernel<<<k, NT, vectors_smem(n), s>>>(n, k, d, e, w, Y, wv, ctl);
+  tri_vectors_kernel<<<k, NT, vectors_smem(n), s>>>(n, k, d, e, w, Y, wv, exact, ctl);
   DF_LAUNCHED("tri_vectors_kernel");
   DF_CUDA(cudaFuncSetAttribute(back_transform_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 220 * 1024));
   back_transform_kernel<<<k, NT, sizeof(double) * (size_t)n, s>>>(A, n, Tf, Y, wv, w, Q, ctl);
