@@ -638,10 +638,12 @@ extern "C" int df_jk(const void* B, int nao, int naux, int precision, const doub
   DF_REQUIRE(!J || D, DF_ERR_ARG, "df_jk: J requested without D");
   DF_REQUIRE(!K || (C && nocc > 0), DF_ERR_ARG, "df_jk: K requested without C / nocc");
   DF_REQUIRE(naux <= 65535, DF_ERR_ARG, "df_jk: naux > 65535");
-  size_t need = df_jk_work_bytes(nao, naux, nocc, precision);
-  DF_REQUIRE(work && work_bytes >= need, DF_ERR_NOMEM, "df_jk: workspace of %zu bytes < %zu", work_bytes, need);
+  const int cols = layout_columns(nocc, nocc && precision == DF_FP64 ? nao : nocc, work_bytes,
+                                  [&](int n) { return df_jk_work_bytes(nao, naux, n, precision); });
+  DF_REQUIRE(work && cols >= 0, DF_ERR_NOMEM, "df_jk: workspace of %zu bytes < %zu", work_bytes,
+             df_jk_work_bytes(nao, naux, nocc, precision));
   Arena a(work, work_bytes);
-  JKWork w = jk_work_layout(nao, naux, nocc, precision, &a, nullptr, false);
+  JKWork w = jk_work_layout(nao, naux, cols, precision, &a, nullptr, false);
   DF_REQUIRE(!a.overflow, DF_ERR_NOMEM, "df_jk: workspace overflow");
   if (K) DF_TRY(reset_tc_errors(w.err, 2, TC_EXCHANGE, s));
   DF_TRY(run_jk(B, nao, naux, precision, D, C, nocc, J, K, w, s));

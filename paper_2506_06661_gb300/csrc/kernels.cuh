@@ -4,6 +4,8 @@
 #include <vector>
 #include <algorithm>
 
+#include <algorithm>
+
 #include "common.cuh"
 
 namespace dfscf {
@@ -129,6 +131,15 @@ int build_K_mixed(const void* B, const BLayout& L, int nao, int naux, const doub
                   const MixedKWork& w, cudaStream_t s);
 int build_J(const void* Bbuf, const BLayout& L, int nao, int naux, int precision, const double* D, double* J,
             const JKWork& w, cudaStream_t s);
+// A workspace sized for more occupied columns serves fewer, though the size of the FP64 exchange's blocks
+// does not grow with every column: the number of columns from nocc on whose layout fits in
+// work_bytes (at most `most`), -1 if there is none.  bytes(n): the size for n columns.
+template <typename Bytes>
+int layout_columns(int nocc, int most, size_t work_bytes, Bytes bytes) {
+  for (int n = nocc; n <= std::max(nocc, most); ++n)
+    if (work_bytes >= bytes(n)) return n;
+  return -1;
+}
 int run_jk(const void* B, int nao, int naux, int precision, const double* D, const double* C, int nocc, double* J,
            double* K, const JKWork& w, cudaStream_t s);
 int build_B(const double* ao_xyz, const double* ao_exp, int nao, const double* aux_xyz, const double* aux_exp,

@@ -225,8 +225,9 @@ extern "C" int df_lrdf_jk(const void* B_lr, const double* ao_xyz, const double* 
   DF_REQUIRE(omega > 0.0 && std::isfinite(omega), DF_ERR_ARG, "df_lrdf_jk: omega must be positive and finite");
   DF_REQUIRE(!J || D, DF_ERR_ARG, "df_lrdf_jk: J requested without D");
   DF_REQUIRE(!K || (C && nocc > 0), DF_ERR_ARG, "df_lrdf_jk: K requested without C / nocc");
-  DF_REQUIRE(work && work_bytes >= df_lrdf_jk_work_bytes(nao, naux, nocc), DF_ERR_NOMEM,
-             "df_lrdf_jk: workspace too small");
+  DF_REQUIRE(work && layout_columns(nocc, nocc ? nao : 0, work_bytes, [&](int n) {
+               return df_lrdf_jk_work_bytes(nao, naux, n);
+             }) >= 0, DF_ERR_NOMEM, "df_lrdf_jk: workspace too small");
   Arena a(work, work_bytes);
   LrWork w{};
   lr_layout(nao, &a, nullptr, &w);

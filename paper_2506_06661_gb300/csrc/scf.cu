@@ -2021,6 +2021,12 @@ static int check_molecule(const df_molecule* mol, const scf_opts& o) {
 int scf_run_on(const df_molecule* mol, const scf_opts& o, const double* dm0, double* D_out, double* C_out,
                double* mo_energy, scf_result* res, void* work, size_t work_bytes, cudaStream_t s);
 
+// Occupied columns that a molecule's workspace is laid out for.
+static int scf_layout_columns(const df_molecule& mol, int precision, size_t work_bytes) {
+  return layout_columns(mol.nelec / 2, precision == DF_MIXED ? std::min(mol.nao, 256) : mol.nao, work_bytes,
+                        [&](int n) { return scf_work_bytes(mol.nao, mol.naux, n, precision); });
+}
+
 static int init_mol(ScfMol& M, const df_molecule* mol, const scf_opts& o, void* work, size_t work_bytes,
                     cudaStream_t s) {
   M.mol = *mol;
@@ -2032,7 +2038,9 @@ static int init_mol(ScfMol& M, const df_molecule* mol, const scf_opts& o, void* 
   M.nocc = mol->nelec / 2;
   M.s = s;
   Arena a(work, work_bytes);
-  scf_layout(M.nao, M.naux, M.nocc, o.precision, &a, nullptr, &M.W);
+  const int cols = scf_layout_columns(*mol, o.precision, work_bytes);
+  DF_REQUIRE(cols >= 0, DF_ERR_NOMEM, "scf: workspace overflow");
+  scf_layout(M.nao, M.naux, cols, o.precision, &a, nullptr, &M.W);
   DF_REQUIRE(!a.overflow, DF_ERR_NOMEM, "scf: workspace overflow");
   return DF_OK;
 }
@@ -2072,7 +2080,8 @@ extern "C" int scf_run(const df_molecule* mol, const scf_opts* opt, const double
   if (opt) o = *opt; else scf_default_opts(&o);
   DF_TRY(check_molecule(mol, o));
   size_t need = scf_work_bytes(mol->nao, mol->naux, mol->nelec / 2, o.precision);
-  DF_REQUIRE(work && work_bytes >= need, DF_ERR_NOMEM, "scf_run: workspace of %zu bytes < %zu", work_bytes, need);
+  DF_REQUIRE(work && scf_layout_columns(*mol, o.precision, work_bytes) >= 0, DF_ERR_NOMEM,
+             "scf_run: workspace of %zu bytes < %zu", work_bytes, need);
   // The iterations are captured into CUDA graphs, which the legacy default stream does
   // not allow; run on a private stream ordered after the caller's and join back at the end.
   cudaStream_t ps = nullptr;
