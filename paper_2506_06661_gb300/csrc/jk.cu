@@ -365,18 +365,20 @@ __global__ void ksum_mirror_kernel(const double* __restrict__ Kpart, int nsplit,
 // Block sizes of the FP64 exchange.  Each half-transform launch should fill the GPU for whole waves
 // of 128-row tiles (pb), and each SYRK launch should have a long K (px), within 1 GB of X and its
 // digits and within 64 splits of 4096 stages.  The digits of a wave's rows of B take more than B itself
-// in small molecules, and every molecule of a batch holds them: four or three waves where they fit in
-// half of B and 540 MB, two where they fit in 5/4 of it, else one.  Four waves, two, one (MB of workspace,
-// ms): 20 centres 52, 52, 37 MB, 0.18, 0.18, 0.19 ms; 40 centres 280, 170, 116 MB, 0.61, 0.63, 0.67
-// ms; 63 centres 566, 389, 302 MB, 1.64, 1.70, 1.85 ms; 100 centres 1399, 1134, 997 MB, 7.9, 8.1, 8.0
-// ms; 200 centres (100 columns: half the rows a wave) 1605, 1381 MB, 69.4, 72.7 ms.
+// in small molecules, and every molecule of a batch holds them: two waves where they fit in 5/4 of B,
+// else one.  With n tiles of columns a wave has an n-th of the rows: four waves or three then, where
+// they fit in half of B and 540 MB.  Four waves, two, one (MB of workspace, ms): 20 centres 52, 52, 37
+// MB, 0.18, 0.18, 0.19 ms; 40 centres 280, 170, 116 MB, 0.61, 0.63, 0.67 ms; 63 centres 564, 389, 302
+// MB, 1.59, 1.70, 1.85 ms; 77 centres 812, 599, 491 MB, 3.46, 3.68, 4.07 ms; 100 centres 1410, 1134,
+// 997 MB, 7.8, 8.0, 7.9 ms; 150 centres (75 columns, two tiles) 1531, 1304, 1219 MB, 28.4, 30.7, 34.7 ms.
 static void fp64_k_blocks(int nao, int naux, int nocc, Fp64KWork* w) {
   const long coltiles = (nocc + 63) / 64;
   const size_t bytes_b = digits::plane_bytes(nao, nao), bytes_x = (size_t)nao * nocc * (2 * digits::NS + 8);
   const size_t bytes_B = sizeof(double) * (size_t)B_ld(nao) * naux;
   auto waves = [&](long n) { return std::max(1L, std::min(n * 152 * digits::BM / coltiles / nao, (long)naux)); };
   auto fits = [&](long n, size_t most) { return (size_t)waves(n) * bytes_b <= std::min(most, (size_t)540000000); };
-  const long n = fits(4, bytes_B / 2) ? 4 : fits(3, bytes_B / 2) ? 3 : fits(2, bytes_B / 4 * 5) ? 2 : 1;
+  const size_t half = coltiles > 1 ? bytes_B / 2 : 0;
+  const long n = fits(4, half) ? 4 : fits(3, half) ? 3 : fits(2, bytes_B / 4 * 5) ? 2 : 1;
   long pb = waves(n);
   if (knob("fp64_k_pb") > 0) pb = std::min(knob("fp64_k_pb"), naux);
   long px = std::max(pb, (long)((1ul << 30) / bytes_x) / pb * pb);
