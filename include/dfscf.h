@@ -158,7 +158,8 @@ int df_B_get_packed(const void* B, int nao, int naux, int P, double* row, cudaSt
  * up, K is filled with NaN and, unless the stream is being captured into a graph, df_jk
  * (which then synchronises the stream once to read the flag) returns DF_ERR_TIMEOUT.  A
  * df_jk with K outside a capture therefore returns with the stream drained.
- * work: df_jk_work_bytes(nao, naux, nocc, precision) bytes.                           */
+ * work: df_jk_work_bytes(nao, naux, nocc, precision) bytes, or the size for more columns (which
+ * may be the smaller one); the same holds for df_lrdf_jk and scf_run.                     */
 size_t df_jk_work_bytes(int nao, int naux, int nocc, int precision);
 int df_jk(const void* B, int nao, int naux, int precision, const double* D, const double* C,
           int nocc, double* J, double* K, void* work, size_t work_bytes, cudaStream_t s);
@@ -396,8 +397,8 @@ int df_fit_residual(const double* ao_xyz, const double* ao_exp, int nao, const d
  *     (mn|kl) ~ (mn|kl)^SR + sum_P T_{P,mn} T_{P,kl}.
  * df_lrdf_build writes T (omega > 0) into B in the DF_FP64 layout of df_build_B
  * (df_B_bytes(nao, naux, DF_FP64) bytes), synchronising for the metric's pivot check
- * (DF_ERR_NOT_SPD) and at the end (DF_ERR_TIMEOUT as in df_build_B).  df_lrdf_jk returns J[D] and K[C C^T] (either may be NULL) as the
- * long-range DF part (df_jk on T) plus the short-range four-centre part, summed directly over
+ * (DF_ERR_NOT_SPD) and at the end (DF_ERR_TIMEOUT as in df_build_B).  df_lrdf_jk
+ * returns J[D] and K[C C^T] (either may be NULL) as the long-range DF part (df_jk on T) plus the short-range four-centre part, summed directly over
  * orbital pairs (quartets whose pair factors multiply to less than 1e-16 of the largest are
  * skipped).  The short-range sums cost O(npair^2) for J and O(nao^4) for K: meant for
  * molecules of up to a few hundred basis functions.  Both synchronise the stream.
